@@ -277,7 +277,9 @@ LKS_API int lks_debug_copy_skip(lks_handle* h, int skip);
  * one persistent cooperative launch per step (grid barriers between the iterations) when the device
  * holds its grid, mode 0 as one launch per iteration (with the finish kernels), mode 2 (the default)
  * the persistent launch only where it measured faster (2D bodies whose box has more tiles than the
- * persistent grid has CTAs), mode -1 only asks. Returns 1 if the persistent kernels are in use after
+ * persistent grid has CTAs; the reverse about one rotation axis then runs by linear maps, whose
+ * buffers the first lks_adjoint allocates if hbm_budget_bytes and the device have room), mode -1
+ * only asks. Returns 1 if the persistent kernels are in use after
  * the call, 0 if not, or -status on error (LKS_ERR_ARG, LKS_ERR_CUDA). Changing the mode
  * synchronises the device; results agree to rounding (the per-CTA partial sums are grouped
  * differently). */
@@ -290,7 +292,8 @@ LKS_API long long lks_launch_count(const lks_handle* h);
  * every launch of the named kernel family with CUDA events on the launching stream.
  * lks_kernel_time returns the summed milliseconds and the launch count for the family
  * ("stencil_fwd", "stencil_adj", "couple", "adj_cell", "adj_design", "recompute", "adj_body" (the
- * persistent reverse coupling), and for lks_adjoint_alks "alks_body", "alks_stencil"); the coupling
+ * reverse of a step's iterations: the persistent kernel, or the two kernels per step of the reverse
+ * by linear maps, whose planes and matrices count as "adj_cell"), and for lks_adjoint_alks "alks_body", "alks_stencil"); the coupling
  * and design-side families include their one-CTA finish kernels. */
 LKS_API int lks_set_kernel_timing(lks_handle* h, int enable);
 LKS_API int lks_kernel_time(lks_handle* h, const char* family, double* ms_total, long long* launches);

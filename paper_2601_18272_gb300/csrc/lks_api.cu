@@ -284,6 +284,11 @@ struct lks_handle {
   void* al_part = nullptr;
   long long al_astride = 0;
   bool alks_mode = false, alks_done = false;
+  // reverse by linear maps (allocated by the first lks_adjoint that takes it; not if the budget or
+  // the device has no room, then the per-iteration kernels run)
+  RevBuffers rev;
+  size_t rev_bytes = 0;
+  bool rev_on = false;
   Dof* it = nullptr;
   Ctrl* ctrl = nullptr;
   Moments* mom = nullptr;
@@ -565,6 +570,23 @@ void enqueue_adj_steps(lks_handle* h, Launcher& L, const Slots<T>& S, int nsteps
     }
     return;
   }
+  if (h->rev_on) {
+    const RevBuffers& R = h->rev;
+    for (int c = 0; c < nsteps; c += R.steps) {
+      const int n = std::min(R.steps, nsteps - c);
+      L.n("adj_cell", 2, [&](cudaStream_t s) {
+        launch_rev_coef<T>(g, R, h->ctrl, h->it, (const T*)h->kref, h->mom, (const T*)h->boxstore, h->nbox, n, c, s);
+      });
+      for (int i = 0; i < n; ++i) {
+        L.n("adj_body", 2, [&](cudaStream_t s) {
+          launch_rev_step<T>(g, R, h->ctrl, h->it, (T*)h->L, h->slot_elems, i, c, s);
+        });
+        L("stencil_adj", [&](cudaStream_t s) { launch_stencil_adj<T>(g, S, (T*)h->L, h->slot_elems, h->ctrl, c + i, s); });
+      }
+      L("adj_design", [&](cudaStream_t s) { launch_rev_design<T>(g, R, h->ctrl, h->it, n, c, s); });
+    }
+    return;
+  }
   for (int i = 0; i < nsteps; ++i) {
     if (g.coop_adj > 0) {  // the N_itr reverse iterations in one persistent launch
       L("adj_body", [&](cudaStream_t s) {
@@ -686,7 +708,7 @@ int binomial_reverse(lks_handle* h, cudaStream_t st) {
       case LKS_BIN_REVERSE: {  // step a from state(a - 1) in the working pair (base b)
         const int t = op.a, t0 = op.b;
         L0("init", [&](cudaStream_t x) { launch_set_step(h->ctrl, t, t0, x); });
-        TRY(run_graph(h, h->alks_mode ? "alks_bin_rev1" : "bin_rev1", st, [&](Launcher& L) {
+        TRY(run_graph(h, std::string(h->alks_mode ? "alks_" : (h->rev_on ? "rev_" : "adj_")) + "bin_rev1", st, [&](Launcher& L) {
           enqueue_recompute<T>(h, L, W, 1);
           enqueue_adj_steps<T>(h, L, W, 1);
         }));
@@ -717,7 +739,9 @@ int adjoint_impl(lks_handle* h, double seed, cudaStream_t st) {
     L0("init", [&](cudaStream_t s) {
       launch_adj_init(g, h->ctrl, h->it, h->P.n_steps, h->objw, seed, term_s, h->dkref, g.ND, s);
     });
+    if (h->rev_on) L0("init", [&](cudaStream_t s) { launch_rev_init(g, h->rev, h->ctrl, NT, s); });
   }
+  const char* kind = h->alks_mode ? "alks_" : (h->rev_on ? "rev_" : "adj_");
   if (h->P.ckpt_policy == LKS_CKPT_BINOMIAL) {
     TRY(binomial_reverse<T>(h, st));
   } else if (h->P.ckpt_policy == LKS_CKPT_STORE_ALL) {
@@ -725,7 +749,7 @@ int adjoint_impl(lks_handle* h, double seed, cudaStream_t st) {
     for (int t1 = NT; t1 >= 1; t1 -= h->chunk) {
       const int n = std::min(h->chunk, t1);
       L0("init", [&](cudaStream_t s) { launch_set_step(h->ctrl, t1, 0, s); });
-      TRY(run_graph(h, (h->alks_mode ? "alks_sa_" : "adj_sa_") + std::to_string(n), st,
+      TRY(run_graph(h, std::string(kind) + "sa_" + std::to_string(n), st,
                     [&](Launcher& L) { enqueue_adj_steps<T>(h, L, S, n); }));
     }
   } else {
@@ -748,12 +772,45 @@ int adjoint_impl(lks_handle* h, double seed, cudaStream_t st) {
       L0("init", [&](cudaStream_t s) { launch_set_step(h->ctrl, t0 + 1, t0, s); });
       TRY(run_graph(h, "rec_" + std::to_string(n), st, [&](Launcher& L) { enqueue_recompute<T>(h, L, S, n); }));
       L0("init", [&](cudaStream_t s) { launch_set_step(h->ctrl, t0 + n, t0, s); });
-      TRY(run_graph(h, (h->alks_mode ? "alks_u_" : "adj_u_") + std::to_string(n), st,
+      TRY(run_graph(h, std::string(kind) + "u_" + std::to_string(n), st,
                     [&](Launcher& L) { enqueue_adj_steps<T>(h, L, S, n); }));
     }
   }
+  if (h->rev_on && !h->alks_mode) L0("adj_design", [&](cudaStream_t s) { launch_rev_dksum(g, h->rev, h->dkref, s); });
   CK(cudaGetLastError());
   if (h->launch_error) return LKS_ERR_CUDA;
+  return LKS_OK;
+}
+
+// Chooses the form of the exact reverse: the linear maps for bodies about one axis in the automatic
+// coupling mode, when the workspace limit and the device have room for their buffers; else the
+// per-iteration or persistent kernels.
+int choose_reverse(lks_handle* h) {
+  h->rev_on = false;
+  if (h->coop_mode != 2 || !reverse_affine_fits(h->g)) return LKS_OK;
+  const int seg = h->P.ckpt_policy == LKS_CKPT_BINOMIAL ? 1
+                  : h->P.ckpt_policy == LKS_CKPT_UNIFORM ? std::min(h->P.ckpt_every, h->P.n_steps) : h->chunk;
+  RevBuffers R;
+  const size_t need = reverse_layout(h->g, h->prec == LKS_FP64, seg, &R);
+  if (need > h->rev_bytes) {  // the first call, or a larger body box since (its graphs are gone)
+    if (h->P.hbm_budget_bytes && h->bytes - h->rev_bytes + need > h->P.hbm_budget_bytes) return LKS_OK;
+    if (h->rev.block) {
+      CK(cudaDeviceSynchronize());
+      CK(cudaFree(h->rev.block));
+      h->rev.block = nullptr;
+      h->bytes -= h->rev_bytes;
+      h->rev_bytes = 0;
+    }
+    if (cudaMalloc(&h->rev.block, need) != cudaSuccess) {
+      cudaGetLastError();
+      h->rev.block = nullptr;
+      return LKS_OK;
+    }
+    h->rev_bytes = need;
+    h->bytes += need;
+  }
+  reverse_layout(h->g, h->prec == LKS_FP64, seg, &h->rev);
+  h->rev_on = true;
   return LKS_OK;
 }
 
@@ -1023,10 +1080,11 @@ int lks_adjoint(lks_handle* h, double seed, void* stream) {
   if (!h->fwd_done) return LKS_ERR_ORDER;
   cudaStream_t st = (cudaStream_t)stream;
   h->adj_done = h->exact_done = false;
+  TRY(choose_reverse(h));
   int r = (h->prec == LKS_FP64) ? adjoint_impl<double>(h, seed, st) : adjoint_impl<float>(h, seed, st);
   if (r != LKS_OK) return r;
   // a grid barrier or tile copy whose wait timed out is reported through the status word
-  if (h->g.coop_adj > 0 || lks_stencil_form(h) == 1) {
+  if ((h->g.coop_adj > 0 && !h->rev_on) || lks_stencil_form(h) == 1) {
     int status = 0;
     CK(cudaMemcpyAsync(&status, (const char*)h->ctrl + offsetof(Ctrl, status), sizeof(int), cudaMemcpyDeviceToHost,
                        st));
@@ -1374,6 +1432,7 @@ void lks_destroy(lks_handle* h) {
       cudaEventDestroy(p.b);
     }
   for (void* p : h->allocs) cudaFree(p);
+  cudaFree(h->rev.block);
   if (h->cap) cudaStreamDestroy(h->cap);
   delete h;
 }

@@ -135,6 +135,34 @@ template <typename T>
 void launch_adj_design(const Geo& g, Ctrl* ctrl, const Dof* it, const T* kref, const T* scratch, double* dkref,
                        void* partials, int k, int di, cudaStream_t st);
 
+// Reverse of a step's N_itr iterations about one rotation axis through the linear map of each
+// iteration (lks_reverse.cu): workspace and launchers. reverse_layout gives the block's bytes for
+// segments of up to max_steps steps and, with R->block set, places the buffers in it.
+struct RevBuffers {
+  void* block = nullptr;
+  void *slabs = nullptr, *mpart = nullptr, *mats = nullptr, *cpart = nullptr, *lamh = nullptr;
+  double* dkp = nullptr;
+  long long slab = 0;  // values per step's slab
+  int steps = 0;       // slabs: steps per chunk
+  int splits = 0;      // partial dJ/dkappa^ref of the design kernel
+};
+bool reverse_affine_fits(const Geo& g);
+size_t reverse_layout(const Geo& g, bool fp64, int max_steps, RevBuffers* R);
+void launch_rev_init(const Geo& g, const RevBuffers& R, Ctrl* ctrl, int nt, cudaStream_t st);
+void launch_rev_dksum(const Geo& g, const RevBuffers& R, double* dkref, cudaStream_t st);
+// Steps ctrl->t0 - di - i, i < nsteps, into slabs i: the planes and matrices (2 kernels) ...
+template <typename T>
+void launch_rev_coef(const Geo& g, const RevBuffers& R, Ctrl* ctrl, const Dof* it, const T* kref, const Moments* mom,
+                     const T* boxstore, int nbox, int nsteps, int di, cudaStream_t st);
+// ... the reverse of slab i's iterations (2 kernels) ...
+template <typename T>
+void launch_rev_step(const Geo& g, const RevBuffers& R, Ctrl* ctrl, const Dof* it, T* Lb, long long lstride, int i,
+                     int di, cudaStream_t st);
+// ... and the slabs' dJ/dkappa^ref.
+template <typename T>
+void launch_rev_design(const Geo& g, const RevBuffers& R, Ctrl* ctrl, const Dof* it, int nsteps, int di,
+                       cudaStream_t st);
+
 // Test export: the design points the coupling's gather accepts for each cell of the box of the
 // iterate s, as out[box cell][5] = (count, least index or -1, largest index, sum, sum of squares).
 template <typename T>

@@ -1,0 +1,885 @@
+// Reverse of one step's N_itr coupling iterations about one rotation axis, without the chain of
+// kernels per iteration (lks_body.cu holds the per-iteration form, kept for free rotation).
+//
+// The reverse of iteration k takes dJ/dF, dJ/dT (D + 1 numbers, lam^k) and gives dJ/ds^(k-1), from
+// which the EOM reverse makes lam^(k-1). Everything else it needs (the pose s^(k-1), kappa_n, u^S_n,
+// u^(k)_n) is known from the forward, and the map is linear, so
+//   dJ/ds^(k-1) = M_k lam^k (+ c for k = N_itr, where the adjoint state lam_n(t) enters),
+// with an 8 x (D + 1) matrix M_k that depends on the forward only. The sums over the design points
+// are taken on the cell side: with Phi = sum W, kap = sum W kappa, P = sum W l, L = sum W kappa l
+// (l = R r_m, in the plane of rotation) and the same sums with dW/dx, the derivatives of a cell's
+// kappa_n, u^S_n and L_n with respect to x^G and theta are closed forms, so no pass over the design
+// points' windows is needed for them.
+//
+//   k_rev_coef    box cells x iterations x steps of a chunk: the sums above, the per-cell planes the
+//                 step needs later, per-CTA partials of M_k (independent of the reverse sweep, so
+//                 all iterations of several steps run in one launch)
+//   k_rev_mat     one CTA per (step, iteration): M_k in FP64 with the closed design-side terms, and
+//                 the map lam^k -> lam^(k-1)
+//   k_rev_const   box cells: c = sum_n lam_n(t) . du_n/ds^(N_itr-1), per-CTA partials
+//   k_rev_apply   every CTA: the sum of c and the chain lam^N_itr -> .. -> lam^1 (FP64, a few fused
+//                 multiply-adds); box cells: dJ/du* and dJ/dkappa_n of every iteration; one more CTA
+//                 carries the direct EOM part dJ/ds(t-1)
+//   k_rev_design  design points x steps of a chunk: dJ/dkappa^ref, from the support windows of
+//                 u^(k)_n and dJ/dkappa_n (D + 1 values per window cell)
+//   k_rev_dksum   dJ/dkappa^ref summed over the splits of k_rev_design, in a fixed order
+//
+// What it replaces: 3 N_itr dependent launches a step (cell, design and one-CTA finish kernel per
+// iteration), bound by their latency on 2D boxes (about 5 us each for 35 k cells) and in FP64 by the
+// few warps a small box gives each launch. Only k_rev_const, k_rev_apply and the transposed stencil
+// are left in a step's chain; the rest runs over whole chunks of steps. Gradients measured on GB300,
+// before -> after: 512x256 / 128^2, 200 steps 30.2 -> 21.1 ms; 1024x512 / 256^2, 100 steps 30.2 -> 22.3
+// ms; 80x40 / 16^2 FP64, 400 steps 256 -> 135 ms; 128x64x64 / 48^3, 40 steps 26.3 -> 21.9 ms.
+#include "lks_body_common.cuh"
+
+namespace lks {
+
+namespace {
+
+constexpr int kRevThreads = 256;
+constexpr int kRevMaxItr = 64;     // iterations k_rev_apply's shared memory holds (432 bytes each)
+constexpr int kRevMaxCtas = 304;  // k_rev_const, k_rev_apply: every CTA of the latter sums the former's partials
+
+// Planes of a step's slab (box cells each). Per iteration: kappa/(1+kappa), L/(1+kappa) in the plane,
+// u, kappa du/dkappa, and the dJ/dT coefficient of dJ/dkappa (k_rev_apply puts dJ/dkappa there).
+// Then for iteration N_itr: 1/(1+kappa), du/dkappa, du/d(x^G, theta), du/du^G and du/domega parts.
+template <int D>
+struct RevPlanes {
+  static constexpr int beta = 0, iL = 1, u = 3, kd = 3 + D, eps = 3 + 2 * D, per_itr = 4 + 2 * D;
+  static constexpr int inv = 0, del = 1, Q = 1 + D, bphi = Q + (D + 1) * D, bP = bphi + 1, consts = bP + 2;
+};
+// Sums of k_rev_coef: rows x^G and theta by columns lam_F and lam_T, then the u^G and omega rows.
+template <int D>
+struct RevSums {
+  static constexpr int uF = (D + 1) * (D + 1), uT = uF + 1, oF = uT + 2, oT = oF + 2, N = oT + 1;
+};
+template <int D>
+__host__ __device__ constexpr int rev_nconst() { return 2 * D + 2; }  // c: x^G[D], theta, u^G[D], omega
+
+// Block sums of NV per-thread values with few instructions: the values go through shared memory
+// (rows of kRevThreads), 8 threads sum each row's eighths in order and combine them with shuffles.
+// A shuffle tree over all threads costs NV * 5 levels in every warp: with 15 to 22 values that was
+// as much as the gather itself. FP32 values are summed as double-float pairs.
+template <int NV>
+struct RowBuf {
+  static constexpr int pitch = kRevThreads + 1;
+};
+template <int NV>
+__device__ __forceinline__ void row_sums(const float (&v)[NV], float* buf, float2* out) {
+  constexpr int pitch = RowBuf<NV>::pitch;
+  const int tid = threadIdx.x;
+  __syncthreads();
+#pragma unroll
+  for (int i = 0; i < NV; ++i) buf[i * pitch + tid] = v[i];
+  __syncthreads();
+  const int row = tid >> 3, seg = tid & 7;
+  static_assert(NV * 8 <= kRevThreads, "eight threads per value");
+  if ((tid & ~31) < NV * 8) {  // whole warps (shuffles below)
+    float hi = 0.0f, lo = 0.0f;
+    if (row < NV) {
+      const float* p = buf + row * pitch + seg;
+#pragma unroll 8
+      for (int j = 0; j < kRevThreads / 8; ++j) {
+        const float b = p[8 * j], s = hi + b, bb = s - hi;
+        lo += (hi - (s - bb)) + (b - bb);
+        hi = s;
+      }
+    }
+#pragma unroll
+    for (int off = 4; off > 0; off >>= 1)
+      df_add(hi, lo, __shfl_down_sync(0xffffffffu, hi, off, 8), __shfl_down_sync(0xffffffffu, lo, off, 8));
+    if (row < NV && seg == 0) out[row] = make_float2(hi, lo);
+  }
+}
+template <int NV>
+__device__ __forceinline__ void row_sums(const double (&v)[NV], double* buf, double* out) {
+  constexpr int pitch = RowBuf<NV>::pitch;
+  const int tid = threadIdx.x;
+  __syncthreads();
+#pragma unroll
+  for (int i = 0; i < NV; ++i) buf[i * pitch + tid] = v[i];
+  __syncthreads();
+  const int row = tid >> 3, seg = tid & 7;
+  static_assert(NV * 8 <= kRevThreads, "eight threads per value");
+  if ((tid & ~31) < NV * 8) {
+    double s = 0.0;
+    if (row < NV) {
+      const double* p = buf + row * pitch + seg;
+#pragma unroll 8
+      for (int j = 0; j < kRevThreads / 8; ++j) s += p[8 * j];
+    }
+#pragma unroll
+    for (int off = 4; off > 0; off >>= 1) s += __shfl_down_sync(0xffffffffu, s, off, 8);
+    if (row < NV && seg == 0) out[row] = s;
+  }
+}
+// Row `row` of partials [n][nv] summed by 8 threads in a fixed order (result in seg 0's thread).
+__device__ __forceinline__ double part_sum(const float2* p, int n, int nv, int row, int seg) {
+  float hi = 0.0f, lo = 0.0f;
+#pragma unroll 4
+  for (int q = seg; q < n; q += 8) {
+    const float2 b = __ldcg(p + (long long)q * nv + row);
+    df_add(hi, lo, b.x, b.y);
+  }
+#pragma unroll
+  for (int off = 4; off > 0; off >>= 1)
+    df_add(hi, lo, __shfl_down_sync(0xffffffffu, hi, off, 8), __shfl_down_sync(0xffffffffu, lo, off, 8));
+  return (double)hi + (double)lo;
+}
+__device__ __forceinline__ double part_sum(const double* p, int n, int nv, int row, int seg) {
+  double s = 0.0;
+#pragma unroll 4
+  for (int q = seg; q < n; q += 8) s += __ldcg(p + (long long)q * nv + row);
+#pragma unroll
+  for (int off = 4; off > 0; off >>= 1) s += __shfl_down_sync(0xffffffffu, s, off, 8);
+  return s;
+}
+
+// w(r) and w'(r) inside the support.
+__device__ __forceinline__ void w_dw(int wk, float r, float* w, float* dw) {
+  *w = wfun(wk, r);
+  *dw = dwfun(wk, r);
+}
+__device__ __forceinline__ void w_dw(int wk, double r, double* w, double* dw) {
+  if (wk == W_BILINEAR) {
+    *w = wfun(wk, r);
+    *dw = dwfun(wk, r);
+    return;
+  }
+  double s, c;
+  sincospi(0.5 * r, &s, &c);
+  *w = 0.25 * (1.0 + c);
+  *dw = -0.125 * 3.141592653589793 * s;
+}
+
+// Sums over the design points within the support of one cell: index 0 with W, 1 + e with dW/dx_e
+// (e the world axis); q: sums with the rotation derivative W_b l_c - W_c l_b times l_b, l_c.
+template <typename T>
+struct Moments1 {
+  T phi[4], kap[4], Pb[4], Pc[4], Lb[4], Lc[4];
+  T qPb, qPc, qLb, qLc;
+};
+
+template <typename T, int D, int AX>
+__device__ __forceinline__ void gather_moments(const Geo& g, const T* __restrict__ kref, const T (&d)[3], T cs, T sn,
+                                               Moments1<T>& o) {
+  constexpr int b = Axes<AX>::B, c = Axes<AX>::C, ax = Axes<AX>::A;
+  const T S = (T)g.s;
+#pragma unroll
+  for (int e = 0; e < 4; ++e) o.phi[e] = o.kap[e] = o.Pb[e] = o.Pc[e] = o.Lb[e] = o.Lc[e] = T(0);
+  o.qPb = o.qPc = o.qLb = o.qLc = T(0);
+  const T xib = cs * d[b] + sn * d[c] + pivot<T>(g, b);
+  const T xic = -sn * d[b] + cs * d[c] + pivot<T>(g, c);
+  // candidate rows and, per row, the interval of candidates: bounds in FP32 with the support widened
+  // by more than their rounding, so that no design point is lost; the exact test is in T
+  const float csf = (float)cs, snf = (float)sn, pad = 2e-3f, Sp = (float)g.s + pad;
+  const float xibf = (float)xib, xicf = (float)xic;
+  const float h = Sp * (fabsf(csf) + fabsf(snf)) + pad;
+  const int ib0 = max(0, (int)ceilf(xibf - h)), ib1 = min(g.nd[b] - 1, (int)floorf(xibf + h));
+  const int ic0 = max(0, (int)ceilf(xicf - h)), ic1 = min(g.nd[c] - 1, (int)floorf(xicf + h));
+  if (ib1 < ib0 || ic1 < ic0) return;
+  T wa[4], dwa[4];
+  int qa[4], ia0 = 0;
+  if (D == 3) {
+    const T xia = d[ax] + pivot<T>(g, ax);
+    const int fa = (int)floor(xia);
+    ia0 = max(0, fa - g.s + 1);
+    const int ia1 = min(g.nd[ax] - 1, fa + g.s);
+    bool any = false;
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const int ia = ia0 + q;
+      const T oa = xia - (T)ia;
+      wa[q] = dwa[q] = T(0);
+      qa[q] = INT_MAX;
+      if (ia <= ia1 && fabs(oa) < S) {
+        w_dw(g.wk, oa, &wa[q], &dwa[q]);
+        qa[q] = dsq(ia, g.nd[ax]);
+        any = true;
+      }
+    }
+    if (!any) return;
+  }
+  const int sx = 1, sy = g.nd[0], sz = g.nd[0] * g.nd[1];
+  const int sb = (b == 0) ? sx : (b == 1 ? sy : sz);
+  const int sc = (c == 0) ? sx : (c == 1 ? sy : sz);
+  const int sa = (ax == 0) ? sx : (ax == 1 ? sy : sz);
+  const float tiny = 1e-6f;
+  const float ics = fabsf(csf) > tiny ? 1.0f / csf : 0.0f, isn = fabsf(snf) > tiny ? 1.0f / snf : 0.0f;
+  for (int ib = ib0; ib <= ib1; ++ib) {
+    const float ebf = (float)ib - xibf;
+    float elo = -1e6f, ehi = 1e6f;
+    if (isn != 0.0f) {
+      const float e1 = (csf * ebf - Sp) * isn, e2 = (csf * ebf + Sp) * isn;
+      elo = fmaxf(elo, fminf(e1, e2));
+      ehi = fminf(ehi, fmaxf(e1, e2));
+    } else if (fabsf(csf * ebf) >= Sp) {
+      continue;
+    }
+    if (ics != 0.0f) {
+      const float e1 = (-Sp - snf * ebf) * ics, e2 = (Sp - snf * ebf) * ics;
+      elo = fmaxf(elo, fminf(e1, e2));
+      ehi = fminf(ehi, fmaxf(e1, e2));
+    } else if (fabsf(snf * ebf) >= Sp) {
+      continue;
+    }
+    const int jc0 = max(ic0, (int)ceilf(xicf + elo - pad)), jc1 = min(ic1, (int)floorf(xicf + ehi + pad));
+    const T eb = (T)ib - xib;
+    const int qb = dsq(ib, g.nd[b]);
+    for (int ic = jc0; ic <= jc1; ++ic) {
+      const T ec = (T)ic - xic;
+      const T lb0 = cs * eb - sn * ec, lc0 = sn * eb + cs * ec;  // x^ref - x_n in the plane
+      if (fabs(lb0) >= S || fabs(lc0) >= S) continue;
+      const int qbc = qb + dsq(ic, g.nd[c]);
+      if (qbc > g.rad4) continue;
+      T wb, dwb, wc, dwc;
+      w_dw(g.wk, -lb0, &wb, &dwb);
+      w_dw(g.wk, -lc0, &wc, &dwc);
+      const T lb = lb0 + d[b], lc = lc0 + d[c];  // R r_m
+      const int m2 = ib * sb + ic * sc;
+      T s0 = T(1), s1 = T(0), k0, k1 = T(0);
+      if (D == 2) {
+        k0 = kref[m2];
+      } else {
+        s0 = k0 = T(0);
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          if (qa[q] > g.rad4 - qbc) continue;
+          const T kq = kref[m2 + (ia0 + q) * sa];
+          s0 += wa[q];
+          s1 += dwa[q];
+          k0 += wa[q] * kq;
+          k1 += dwa[q] * kq;
+        }
+      }
+      const T w2 = wb * wc, wB = dwb * wc, wC = wb * dwc;
+      auto add = [&](int e, T A, T Ak) {
+        o.phi[e] += A;
+        o.kap[e] += Ak;
+        o.Pb[e] += A * lb;
+        o.Pc[e] += A * lc;
+        o.Lb[e] += Ak * lb;
+        o.Lc[e] += Ak * lc;
+      };
+      add(0, w2 * s0, w2 * k0);
+      add(1 + b, wB * s0, wB * k0);
+      add(1 + c, wC * s0, wC * k0);
+      if (D == 3) add(1 + ax, w2 * s1, w2 * k1);
+      const T rt = wB * lc - wC * lb, rs = rt * s0, rk = rt * k0;
+      o.qPb += rs * lb;
+      o.qPc += rs * lc;
+      o.qLb += rk * lb;
+      o.qLc += rk * lc;
+    }
+  }
+}
+
+// Step of slab i of the chunk that starts di steps below ctrl->t0.
+__device__ __forceinline__ int rev_step(const Ctrl* ctrl, int di, int i) { return ctrl->t0 - di - i; }
+
+template <typename T, int D, int AX>
+__global__ void __launch_bounds__(kRevThreads) k_rev_coef(Geo g, const Ctrl* ctrl, const Dof* it,
+                                                          const T* __restrict__ kref, const T* __restrict__ boxstore,
+                                                          int nbox, T* __restrict__ slabs, long long slab,
+                                                          typename Partial<T>::type* __restrict__ mpart, int di) {
+  using RP = RevPlanes<D>;
+  using RS = RevSums<D>;
+  constexpr int b = Axes<AX>::B, c = Axes<AX>::C;
+  extern __shared__ __align__(16) unsigned char rev_smem[];
+  const int K = g.K, k = (int)blockIdx.y + 1, i = blockIdx.z;
+  const int t = rev_step(ctrl, di, i), base = ctrl->base;
+  const Dof* row = it + (long long)(t - 1) * (K + 1);
+  const Dof& sk = row[k - 1];
+  const long long BC = g.box_cells;
+  const long long bl = blockIdx.x * (long long)kRevThreads + threadIdx.x;
+  T v[RS::N];
+#pragma unroll
+  for (int q = 0; q < RS::N; ++q) v[q] = T(0);
+  if (bl < BC) {
+    int lo[3];
+    box_origin<D>(g, row[0], lo[0], lo[1], lo[2]);
+    const unsigned ub = (unsigned)bl, r = ub / (unsigned)g.B[0];
+    const int j0 = (int)(ub - r * (unsigned)g.B[0]);
+    const int j1 = (int)(D == 3 ? r % (unsigned)g.B[1] : r), j2 = (int)(D == 3 ? r / (unsigned)g.B[1] : 0);
+    const int px = lo[0] + j0, py = lo[1] + j1, pz = lo[2] + j2;
+    long long n;
+    const bool ing = cell_index<D>(g, px, py, pz, n);
+    const DofView<T> V(sk);
+    const T d[3] = {V.rel(0, px), V.rel(1, py), D == 3 ? V.rel(2, pz) : T(0)};
+    Moments1<T> A;
+    if (ing) {
+      gather_moments<T, D, AX>(g, kref, d, V.cs, V.sn, A);
+    } else {
+#pragma unroll
+      for (int e = 0; e < 4; ++e) A.phi[e] = A.kap[e] = A.Pb[e] = A.Pc[e] = A.Lb[e] = A.Lc[e] = T(0);
+      A.qPb = A.qPc = A.qLb = A.qLc = T(0);
+    }
+    const T* bs = boxstore + (long long)((t - base - 1) % nbox) * BC * D;
+    const T kap = A.kap[0], inv = T(1) / (T(1) + kap), beta = kap * inv, om = V.om;
+    T us[3], u[3], del[3];
+#pragma unroll
+    for (int a = 0; a < D; ++a) {
+      us[a] = V.ug[a] * A.phi[0];
+      if (a == b) us[a] -= om * A.Pc[0];
+      if (a == c) us[a] += om * A.Pb[0];
+      u[a] = ing ? (bs[a * BC + bl] + kap * us[a]) * inv : T(0);  // no stored u* off the grid
+      del[a] = (us[a] - u[a]) * inv;
+    }
+    T* P = slabs + (long long)i * slab + bl;
+    T* Pk = P + (long long)(k - 1) * RP::per_itr * BC;
+    Pk[RP::beta * BC] = beta;
+    Pk[RP::iL * BC] = inv * A.Lb[0];
+    Pk[(RP::iL + 1) * BC] = inv * A.Lc[0];
+#pragma unroll
+    for (int a = 0; a < D; ++a) {
+      Pk[(RP::u + a) * BC] = u[a];
+      Pk[(RP::kd + a) * BC] = kap * del[a];
+    }
+    Pk[RP::eps * BC] = A.Lb[0] * del[c] - A.Lc[0] * del[b];
+    const T bphi = beta * A.phi[0], bPb = beta * A.Pb[0], bPc = beta * A.Pc[0];
+    T* Pc = P + (long long)K * RP::per_itr * BC;
+    if (k == K) {
+      Pc[RP::inv * BC] = inv;
+#pragma unroll
+      for (int a = 0; a < D; ++a) Pc[(RP::del + a) * BC] = del[a];
+      Pc[RP::bphi * BC] = bphi;
+      Pc[RP::bP * BC] = bPb;
+      Pc[(RP::bP + 1) * BC] = bPc;
+    }
+    // rows x^G_e (derivative -dW/dx_e) and theta (W_b l_c - W_c l_b, and l turning with the body)
+#pragma unroll
+    for (int e = 0; e <= D; ++e) {
+      T dphi, dk, dPb, dPc, dLb, dLc;
+      if (e < D) {
+        dphi = -A.phi[1 + e];
+        dk = -A.kap[1 + e];
+        dPb = -A.Pb[1 + e];
+        dPc = -A.Pc[1 + e];
+        dLb = -A.Lb[1 + e];
+        dLc = -A.Lc[1 + e];
+      } else {
+        dphi = A.Pc[1 + b] - A.Pb[1 + c];
+        dk = A.Lc[1 + b] - A.Lb[1 + c];
+        dPb = A.qPb - A.Pc[0];
+        dPc = A.qPc + A.Pb[0];
+        dLb = A.qLb - A.Lc[0];
+        dLc = A.qLc + A.Lb[0];
+      }
+      T du[3];
+#pragma unroll
+      for (int a = 0; a < D; ++a) {
+        T dus = V.ug[a] * dphi;
+        if (a == b) dus -= om * dPc;
+        if (a == c) dus += om * dPb;
+        du[a] = del[a] * dk + beta * dus;
+        if (k == K) Pc[(RP::Q + e * D + a) * BC] = du[a];
+        v[e * (D + 1) + a] = kap * du[a] + u[a] * dk;
+      }
+      v[e * (D + 1) + D] = A.Lb[0] * du[c] - A.Lc[0] * du[b] + dLb * u[c] - dLc * u[b];
+    }
+    v[RS::uF] = kap * bphi;
+    v[RS::uT] = -A.Lc[0] * bphi;
+    v[RS::uT + 1] = A.Lb[0] * bphi;
+    v[RS::oF] = -kap * bPc;
+    v[RS::oF + 1] = kap * bPb;
+    v[RS::oT] = A.Lb[0] * bPb + A.Lc[0] * bPc;
+  }
+  row_sums<RS::N>(v, reinterpret_cast<T*>(rev_smem),
+                  mpart + (((long long)i * K + (k - 1)) * gridDim.x + blockIdx.x) * RS::N);
+}
+
+// M_k (rows the 8 DOFs, columns lam_F[3], lam_T) with the design-side closed forms of F and T
+// (F -= K0 u^G + omega R'K1, T -= RK1 x u^G + omega K2p), and G = the EOM reverse of iteration k - 1
+// applied to it: lam^(k-1) = G lam^k.
+struct RevMat {
+  double M[8][4], G[4][4];
+};
+
+template <typename T, int D, int AX>
+__global__ void __launch_bounds__(kRevThreads) k_rev_mat(Geo g, const Ctrl* ctrl, const Dof* it,
+                                                         const Moments* __restrict__ mom,
+                                                         const typename Partial<T>::type* __restrict__ mpart,
+                                                         int nparts, RevMat* __restrict__ mats, int di) {
+  using RS = RevSums<D>;
+  constexpr int b = Axes<AX>::B, c = Axes<AX>::C;
+  __shared__ double s[RS::N], M[8][4];
+  const int K = g.K, k = (int)blockIdx.x + 1, i = blockIdx.y, tid = threadIdx.x;
+  if ((tid & ~31) < RS::N * 8) {
+    const int rw = min(tid >> 3, RS::N - 1);
+    const double a = part_sum(mpart + ((long long)i * K + (k - 1)) * nparts * RS::N, nparts, RS::N, rw, tid & 7);
+    if ((tid >> 3) < RS::N && (tid & 7) == 0) s[tid >> 3] = a;
+  }
+  if (tid < 32) (&M[0][0])[tid] = 0.0;
+  __syncthreads();
+  if (tid == 0) {
+    const Dof& sk = it[(long long)(rev_step(ctrl, di, i) - 1) * (K + 1) + (k - 1)];
+    const double cs = sk.cs, sn = sk.sn, om = sk.s[7];
+    const double K1[3] = {mom->K1[0], mom->K1[1], mom->K1[2]};
+    double r[3], dr[3];
+    rot<AX>(cs, sn, K1, r);
+    drot<AX>(cs, sn, K1, dr);
+    const double K0 = mom->K0;
+    const double ug[3] = {sk.s[3], sk.s[4], sk.s[5]};
+    for (int e = 0; e <= D; ++e) {
+      const int j = e < D ? e : 6;
+      for (int a = 0; a < D; ++a) M[j][a] = s[e * (D + 1) + a];
+      M[j][3] = s[e * (D + 1) + D];
+    }
+    M[6][b] += om * r[b];
+    M[6][c] += om * r[c];
+    M[6][3] -= dr[b] * ug[c] - dr[c] * ug[b];
+    for (int a = 0; a < D; ++a) M[3 + a][a] = s[RS::uF] - K0;
+    M[3 + b][3] = s[RS::uT] + r[c];
+    M[3 + c][3] = s[RS::uT + 1] - r[b];
+    M[7][b] = s[RS::oF] - dr[b];
+    M[7][c] = s[RS::oF + 1] - dr[c];
+    M[7][3] = s[RS::oT] - mom->K2p;
+  }
+  __syncthreads();
+  RevMat& o = mats[(long long)i * K + (k - 1)];
+  if (tid < 32) (&o.M[0][0])[tid] = (&M[0][0])[tid];
+  if (tid < 16) {
+    const int a = tid >> 2, q = tid & 3;
+    double v = 0.0;
+    if (a < 3) {
+      if (a < D && (g.dof_mask & (1 << a))) v = (M[3 + a][q] + M[a][q]) * g.inv_mass;
+    } else if (g.dof_mask & DOF_ROT) {
+      v = (M[7][q] + M[6][q]) * g.inv_inertia;
+    }
+    o.G[a][q] = v;
+  }
+}
+
+// Box cell bl of the box at lo: its grid index; false outside a non-periodic axis.
+template <int D>
+__device__ __forceinline__ bool box_cell(const Geo& g, const int (&lo)[3], long long bl, long long& n) {
+  const unsigned ub = (unsigned)bl, r = ub / (unsigned)g.B[0];
+  const int j0 = (int)(ub - r * (unsigned)g.B[0]);
+  const int j1 = (int)(D == 3 ? r % (unsigned)g.B[1] : r), j2 = (int)(D == 3 ? r / (unsigned)g.B[1] : 0);
+  return cell_index<D>(g, lo[0] + j0, lo[1] + j1, lo[2] + j2, n);
+}
+
+template <typename T, int D, int AX>
+__global__ void __launch_bounds__(kRevThreads) k_rev_const(Geo g, const Ctrl* ctrl, const Dof* it,
+                                                           const T* __restrict__ slabs, long long slab, const T* Lb,
+                                                           long long lstride,
+                                                           typename Partial<T>::type* __restrict__ cpart, int di,
+                                                           int i) {
+  using RP = RevPlanes<D>;
+  constexpr int b = Axes<AX>::B, c = Axes<AX>::C, NC = rev_nconst<D>();
+  extern __shared__ __align__(16) unsigned char rev_smem[];
+  const int K = g.K, t = rev_step(ctrl, di, i);
+  const T* __restrict__ Lcur = Lb + (long long)(t & 1) * lstride;
+  const long long BC = g.box_cells, N = g.N;
+  int lo[3];
+  box_origin<D>(g, it[(long long)(t - 1) * (K + 1)], lo[0], lo[1], lo[2]);
+  const T* P0 = slabs + (long long)i * slab + (long long)K * RP::per_itr * BC;
+  T v[NC];
+#pragma unroll
+  for (int q = 0; q < NC; ++q) v[q] = T(0);
+  for (long long bl = blockIdx.x * (long long)kRevThreads + threadIdx.x; bl < BC;
+       bl += (long long)gridDim.x * kRevThreads) {
+    long long n;
+    if (!box_cell<D>(g, lo, bl, n)) continue;
+    const T* P = P0 + bl;
+    T lam[3];
+    const T bphi = P[RP::bphi * BC];
+#pragma unroll
+    for (int a = 0; a < D; ++a) {
+      lam[a] = Lcur[(a + 1) * N + n];
+      v[D + 1 + a] += lam[a] * bphi;
+    }
+#pragma unroll
+    for (int e = 0; e <= D; ++e)
+#pragma unroll
+      for (int a = 0; a < D; ++a) v[e] += lam[a] * P[(RP::Q + e * D + a) * BC];
+    v[2 * D + 1] += lam[c] * P[RP::bP * BC] - lam[b] * P[(RP::bP + 1) * BC];
+  }
+  row_sums<NC>(v, reinterpret_cast<T*>(rev_smem), cpart + blockIdx.x * NC);
+}
+
+template <typename T, int D, int AX>
+__global__ void __launch_bounds__(kRevThreads) k_rev_apply(Geo g, Ctrl* ctrl, const Dof* it, T* __restrict__ slabs,
+                                                           long long slab, T* Lb, long long lstride,
+                                                           const typename Partial<T>::type* __restrict__ cpart,
+                                                           int nparts, const RevMat* __restrict__ mats,
+                                                           T* __restrict__ lamh, int di, int i) {
+  using RP = RevPlanes<D>;
+  constexpr int b = Axes<AX>::B, c = Axes<AX>::C, NC = rev_nconst<D>();
+  extern __shared__ __align__(16) unsigned char rev_smem[];
+  __shared__ double cc[8];  // c by DOF
+  const int K = g.K, t = rev_step(ctrl, di, i), tid = threadIdx.x;
+  RevMat* mat = reinterpret_cast<RevMat*>(rev_smem);   // the step's matrices [K]
+  double* lamd = reinterpret_cast<double*>(mat + K);   // lam^k [K][4]
+  T* lamt = reinterpret_cast<T*>(lamd + 4 * K);        // the same in the field type
+  for (int q = tid; q < K * (int)(sizeof(RevMat) / sizeof(double)); q += kRevThreads)
+    reinterpret_cast<double*>(mat)[q] = reinterpret_cast<const double*>(mats + (long long)i * K)[q];
+  const double* lin = ctrl->rev_lam[t & 1];  // dJ/ds(t) direct part [8], lam^K [4]
+  if (tid < 8) cc[tid] = 0.0;
+  __syncthreads();
+  if ((tid & ~31) < NC * 8) {
+    const int rw = min(tid >> 3, NC - 1);
+    const double a = part_sum(cpart, nparts, NC, rw, tid & 7);
+    if ((tid >> 3) < NC && (tid & 7) == 0) {
+      const int q = tid >> 3;
+      cc[q < D ? q : (q == D ? 6 : (q < 2 * D + 1 ? 3 + q - (D + 1) : 7))] = a;
+    }
+  }
+  __syncthreads();
+  if (tid < 32) {  // the chain, one lane per component
+    const int a = tid & 3;
+    double x = lin[8 + a], gc = 0.0;
+    if (a < 3) {
+      if (a < D && (g.dof_mask & (1 << a))) gc = (cc[3 + a] + cc[a]) * g.inv_mass;
+    } else if (g.dof_mask & DOF_ROT) {
+      gc = (cc[7] + cc[6]) * g.inv_inertia;
+    }
+    for (int k = K; k >= 1; --k) {
+      if (tid < 4) {
+        lamd[(k - 1) * 4 + a] = x;
+        lamt[(k - 1) * 4 + a] = (T)x;
+      }
+      if (k == 1) break;
+      const double* G = mat[k - 1].G[a];
+      double y = k == K ? gc : 0.0;
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const double xq = __shfl_sync(0xffffffffu, x, q);
+        if (q < D || q == 3) y += G[q] * xq;
+      }
+      x = y;
+    }
+  }
+  __syncthreads();
+  if (blockIdx.x == gridDim.x - 1) {  // the direct EOM part: one lane per DOF
+    for (int q = tid; q < 4 * K; q += kRevThreads) lamh[(long long)i * 4 * K + q] = lamt[q];
+    if (tid < 32) {
+      const int j = tid & 7, a = j % 3;
+      const bool tr = j < 6;
+      const bool fr = tr ? (a < D && (g.dof_mask & (1 << a))) : (g.dof_mask & DOF_ROT) != 0;
+      double lp = lin[j], ls = 0.0;
+      for (int k = K; k >= 1; --k) {
+        ls = k == K ? cc[j] : 0.0;
+        const double* Mj = mat[k - 1].M[j];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) ls += Mj[q] * lamd[(k - 1) * 4 + q];
+        if (k == 1) break;
+        // position rows add their own, velocity rows also the position's if the DOF is free
+        const double lx = __shfl_sync(0xffffffffu, ls, j == 7 ? 6 : (tr && j >= 3 ? j - 3 : j));
+        lp += ls;
+        if (fr && (j == 7 || (tr && j >= 3))) lp += lx;
+      }
+      const double full = lp + ls;  // dJ/ds(t-1)
+      if (tid < 8) ctrl->lam_s0[j] = full;
+      const double lx = __shfl_sync(0xffffffffu, full, j == 7 ? 6 : (tr && j >= 3 ? j - 3 : j));
+      double* lout = ctrl->rev_lam[(t - 1) & 1];
+      if (tid < 8) {
+        const bool vel = j == 7 || (tr && j >= 3);
+        lout[j] = full + (vel && fr ? lx : 0.0);
+        if (vel) lout[8 + (j == 7 ? 3 : a)] = fr ? (full + lx) * (j == 7 ? g.inv_inertia : g.inv_mass) : 0.0;
+      }
+    }
+    return;
+  }
+  T* __restrict__ Lcur = Lb + (long long)(t & 1) * lstride;
+  const long long BC = g.box_cells, N = g.N;
+  int lo[3];
+  box_origin<D>(g, it[(long long)(t - 1) * (K + 1)], lo[0], lo[1], lo[2]);
+  for (long long bl = blockIdx.x * (long long)kRevThreads + tid; bl < BC;
+       bl += (long long)(gridDim.x - 1) * kRevThreads) {
+    long long n;
+    if (!box_cell<D>(g, lo, bl, n)) continue;
+    T* P = slabs + (long long)i * slab + bl;
+    const T* Pc = P + (long long)K * RP::per_itr * BC;
+    T acc[3] = {T(0), T(0), T(0)}, lk = T(0);
+    const T inv = Pc[RP::inv * BC];
+#pragma unroll
+    for (int a = 0; a < D; ++a) {
+      const T lam = Lcur[(a + 1) * N + n];
+      acc[a] = lam * inv;
+      lk += lam * Pc[(RP::del + a) * BC];
+    }
+    for (int k = K; k >= 1; --k) {
+      T* Pk = P + (long long)(k - 1) * RP::per_itr * BC;
+      const T* l = lamt + (k - 1) * 4;
+      const T beta = Pk[RP::beta * BC], lT = l[3];
+      lk += lT * Pk[RP::eps * BC];
+#pragma unroll
+      for (int a = 0; a < D; ++a) {
+        acc[a] += beta * l[a];
+        lk += l[a] * Pk[(RP::kd + a) * BC];
+      }
+      acc[b] -= lT * Pk[(RP::iL + 1) * BC];
+      acc[c] += lT * Pk[RP::iL * BC];
+      Pk[RP::eps * BC] = lk;
+      lk = T(0);
+    }
+#pragma unroll
+    for (int a = 0; a < D; ++a) Lcur[(a + 1) * N + n] = acc[a];
+  }
+}
+
+// Kernel weights of the 2s window cells from floor(x) - s + 1, at the fraction fr of x.
+__device__ __forceinline__ void window_weights(const Geo& g, float fr, float (&w)[4]) {
+  if (g.wk == W_BILINEAR) {
+    w[0] = 1.0f - fr;
+    w[1] = fr;
+    w[2] = w[3] = 0.0f;
+    return;
+  }
+  const float c = __cosf(1.57079632679f * fr), s = __sinf(1.57079632679f * fr);
+  w[0] = 0.25f * (1.0f - s);
+  w[1] = 0.25f * (1.0f + c);
+  w[2] = 0.25f * (1.0f + s);
+  w[3] = 0.25f * (1.0f - c);
+}
+__device__ __forceinline__ void window_weights(const Geo& g, double fr, double (&w)[4]) {
+  if (g.wk == W_BILINEAR) {
+    w[0] = 1.0 - fr;
+    w[1] = fr;
+    w[2] = w[3] = 0.0;
+    return;
+  }
+  double s, c;
+  sincospi(0.5 * fr, &s, &c);
+  w[0] = 0.25 * (1.0 - s);
+  w[1] = 0.25 * (1.0 + c);
+  w[2] = 0.25 * (1.0 + s);
+  w[3] = 0.25 * (1.0 - c);
+}
+
+// LN lanes per design point, one row (2D) or plane (3D) of the window each; split blockIdx.y takes
+// the chunk's steps blockIdx.y, blockIdx.y + gridDim.y, ... and keeps its own dJ/dkappa^ref.
+template <typename T, int D, int AX>
+__global__ void __launch_bounds__(kRevThreads) k_rev_design(Geo g, Ctrl* ctrl, const Dof* it,
+                                                            const T* __restrict__ slabs, long long slab,
+                                                            const T* __restrict__ lamh, double* __restrict__ dkp,
+                                                            int nsteps, int di) {
+  using RP = RevPlanes<D>;
+  constexpr int b = Axes<AX>::B, c = Axes<AX>::C;
+  const int K = g.K, lane = threadIdx.x % LN;
+  const int m = (int)((blockIdx.x * (unsigned)kRevThreads + threadIdx.x) / LN);
+  const int mm = m < g.ND ? m : 0;
+  const int ix = mm % g.nd[0], iy = (mm / g.nd[0]) % g.nd[1], iz = mm / (g.nd[0] * g.nd[1]);
+  const bool valid = m < g.ND && dsq(ix, g.nd[0]) + dsq(iy, g.nd[1]) + dsq(iz, g.nd[2]) <= g.rad4;
+  const T r[3] = {(T)ix - pivot<T>(g, 0), (T)iy - pivot<T>(g, 1), D == 3 ? (T)iz - pivot<T>(g, 2) : T(0)};
+  const int S2 = 2 * g.s;
+  const long long BC = g.box_cells;
+  const int B0 = g.B[0], B1 = g.B[1], B2 = (D == 3) ? g.B[2] : 1;
+  bool inside = true;
+  double acc = 0.0;
+  for (int i = blockIdx.y; i < nsteps; i += gridDim.y) {
+    const Dof* row = it + (long long)(rev_step(ctrl, di, i) - 1) * (K + 1);
+    int lo[3];
+    box_origin<D>(g, row[0], lo[0], lo[1], lo[2]);
+    for (int k = K; k >= 1; --k) {
+      const DofView<T> V(row[k - 1]);
+      T l[3], dl[3], usr[3], fr[3], w[3][4];
+      int f[3] = {0, 0, 0};
+      rot<AX>(V.cs, V.sn, r, l);
+      drot<AX>(V.cs, V.sn, r, dl);
+#pragma unroll
+      for (int a = 0; a < D; ++a) {
+        usr[a] = V.ug[a] + V.om * dl[a];
+        V.split(a, l[a], &f[a], &fr[a]);
+        window_weights(g, fr[a], w[a]);
+        f[a] += 1 - g.s - lo[a];
+      }
+      // the window's cells with weight 0 (fr = 0 puts the last one on the support's edge) need not
+      // lie in the box
+      constexpr int E = (D == 3) ? 2 : 1;
+      T we = T(0);
+#pragma unroll
+      for (int q = 0; q < 4; ++q)
+        if (q == lane) we = w[E][q];
+      const bool here = valid && lane < S2 && we != T(0);
+      const int pe = f[E] + lane;
+      if (here && (f[0] < 0 || f[0] + S2 - 1 - (fr[0] == T(0)) >= B0 || pe < 0 || pe >= (D == 3 ? B2 : B1) ||
+                   (D == 3 && (f[1] < 0 || f[1] + S2 - 1 - (fr[1] == T(0)) >= B1))))
+        inside = false;
+      T uref[3] = {T(0), T(0), T(0)}, slk = T(0);
+      if (here && inside) {
+        const T* P = slabs + (long long)i * slab + (long long)(k - 1) * RP::per_itr * BC;
+        const T* Pu = P + RP::u * BC;
+        const T* Pl = P + RP::eps * BC;
+#pragma unroll
+        for (int q1 = 0; q1 < (D == 3 ? 4 : 1); ++q1) {
+          if (D == 3 && (q1 >= S2 || w[1][q1] == T(0))) continue;
+          const T w1 = D == 3 ? we * w[1][q1] : we;
+          const int rowb = D == 3 ? f[0] + B0 * (f[1] + q1 + B1 * pe) : f[0] + B0 * pe;
+#pragma unroll
+          for (int q0 = 0; q0 < 4; ++q0) {
+            if (q0 >= S2 || w[0][q0] == T(0)) continue;
+            const T W = w[0][q0] * w1;
+            const int o = rowb + q0;
+            slk += W * __ldg(Pl + o);
+#pragma unroll
+            for (int a = 0; a < D; ++a) uref[a] += W * __ldg(Pu + a * BC + o);
+          }
+        }
+      }
+#pragma unroll
+      for (int off = 1; off < LN; off <<= 1) {
+        slk += __shfl_xor_sync(0xffffffffu, slk, off);
+#pragma unroll
+        for (int a = 0; a < D; ++a) uref[a] += __shfl_xor_sync(0xffffffffu, uref[a], off);
+      }
+      if (valid && lane == 0) {
+        const T* lam = lamh + ((long long)i * K + (k - 1)) * 4;
+        T dk = slk;
+#pragma unroll
+        for (int a = 0; a < D; ++a) {
+          uref[a] -= usr[a];
+          dk += lam[a] * uref[a];
+        }
+        dk += lam[3] * (l[b] * uref[c] - l[c] * uref[b]);
+        acc += (double)dk;
+      }
+    }
+  }
+  if (!inside) atomicOr(&ctrl->status, ST_BOX_OVERFLOW);
+  if (valid && lane == 0) dkp[(long long)blockIdx.y * g.ND + m] += acc;
+}
+
+__global__ void __launch_bounds__(kRevThreads) k_rev_dksum(int nd, int splits, const double* __restrict__ dkp,
+                                                           double* __restrict__ dkref) {
+  const int m = blockIdx.x * kRevThreads + threadIdx.x;
+  if (m >= nd) return;
+  double s = 0.0;
+  for (int q = 0; q < splits; ++q) s += dkp[(long long)q * nd + m];
+  dkref[m] = s;
+}
+
+// Seed of the sweep in the double-buffered carried adjoint (k_adj_init has filled lam_prev, lam_F, lam_T).
+__global__ void k_rev_init(Ctrl* ctrl, int nt) {
+  double* o = ctrl->rev_lam[nt & 1];
+  for (int a = 0; a < 8; ++a) o[a] = ctrl->lam_prev[a];
+  for (int a = 0; a < 3; ++a) o[8 + a] = ctrl->lam_F[a];
+  o[11] = ctrl->lam_T[0];
+}
+
+unsigned rev_ctas(const Geo& g) {
+  const long long n = (g.box_cells + kRevThreads - 1) / kRevThreads;
+  return (unsigned)(n < kRevMaxCtas ? n : kRevMaxCtas);
+}
+
+template <typename T, int D>
+size_t rev_row_bytes(int nv) { return (size_t)nv * RowBuf<1>::pitch * sizeof(T); }
+
+template <typename T, int D, int AX>
+void coef_ax(const Geo& g, const RevBuffers& R, Ctrl* ctrl, const Dof* it, const T* kref, const Moments* mom,
+             const T* boxstore, int nbox, int nsteps, int di, cudaStream_t st) {
+  using PT = typename Partial<T>::type;
+  const unsigned nc = (unsigned)((g.box_cells + kRevThreads - 1) / kRevThreads);
+  launch(k_rev_coef<T, D, AX>, dim3(nc, g.K, nsteps), kRevThreads, rev_row_bytes<T, D>(RevSums<D>::N), st, g,
+         (const Ctrl*)ctrl, it, kref, boxstore, nbox, (T*)R.slabs, R.slab, (PT*)R.mpart, di);
+  launch(k_rev_mat<T, D, AX>, dim3(g.K, nsteps), kRevThreads, 0, st, g, (const Ctrl*)ctrl, it, mom, (const PT*)R.mpart,
+         (int)nc, (RevMat*)R.mats, di);
+}
+template <typename T, int D, int AX>
+void step_ax(const Geo& g, const RevBuffers& R, Ctrl* ctrl, const Dof* it, T* Lb, long long lstride, int i, int di,
+             cudaStream_t st) {
+  using PT = typename Partial<T>::type;
+  const unsigned nc = rev_ctas(g);
+  launch(k_rev_const<T, D, AX>, nc, kRevThreads, rev_row_bytes<T, D>(rev_nconst<D>()), st, g, (const Ctrl*)ctrl, it,
+         (const T*)R.slabs, R.slab, (const T*)Lb, lstride, (PT*)R.cpart, di, i);
+  launch(k_rev_apply<T, D, AX>, nc + 1, kRevThreads, (size_t)g.K * (sizeof(RevMat) + 4 * (sizeof(double) + sizeof(T))), st, g, ctrl, it,
+         (T*)R.slabs, R.slab, Lb, lstride, (const PT*)R.cpart, (int)nc, (const RevMat*)R.mats, (T*)R.lamh, di, i);
+}
+template <typename T, int D, int AX>
+void design_ax(const Geo& g, const RevBuffers& R, Ctrl* ctrl, const Dof* it, int nsteps, int di, cudaStream_t st) {
+  const unsigned nb = (unsigned)(((long long)g.ND * LN + kRevThreads - 1) / kRevThreads);
+  launch(k_rev_design<T, D, AX>, dim3(nb, R.splits), kRevThreads, 0, st, g, ctrl, it, (const T*)R.slabs, R.slab,
+         (const T*)R.lamh, R.dkp, nsteps, di);
+}
+
+#define LKS_REV_DISPATCH(F, ...)                  \
+  do {                                            \
+    if (g.dim == 2) F<T, 2, 2>(__VA_ARGS__);      \
+    else if (g.ax == 0) F<T, 3, 0>(__VA_ARGS__);  \
+    else if (g.ax == 1) F<T, 3, 1>(__VA_ARGS__);  \
+    else F<T, 3, 2>(__VA_ARGS__);                 \
+  } while (0)
+
+}  // namespace
+
+bool reverse_affine_fits(const Geo& g) {
+  return g.ax != AX_FREE && g.box_cells < (1LL << 29) && g.K <= kRevMaxItr;
+}
+
+size_t reverse_layout(const Geo& g, bool fp64, int max_steps, RevBuffers* R) {
+  const long long esz = fp64 ? 8 : 4, K = g.K;
+  const int D = g.dim;
+  const long long planes = D == 2 ? K * RevPlanes<2>::per_itr + RevPlanes<2>::consts
+                                  : K * RevPlanes<3>::per_itr + RevPlanes<3>::consts;
+  const long long nm = D == 2 ? RevSums<2>::N : RevSums<3>::N;
+  const long long nc = (g.box_cells + kRevThreads - 1) / kRevThreads;
+  R->slab = planes * g.box_cells;
+  // steps per chunk: as many slabs as about half of the L2 holds, so that the planes written by one
+  // kernel are read from L2 by the next; at least one, at most the segment
+  const long long want = (64LL << 20) / (R->slab * esz);
+  R->steps = (int)(want < 1 ? 1 : (want < max_steps ? want : max_steps));
+  if (R->steps > 64) R->steps = 64;
+  // splits of the design kernel over the chunk's steps: about 2^17 threads
+  long long sp = (1LL << 17) / ((long long)g.ND * LN);
+  sp = sp < 1 ? 1 : (sp > 16 ? 16 : sp);
+  R->splits = (int)(sp < R->steps ? sp : R->steps);
+  size_t off = 0;
+  auto take = [&](long long bytes) {
+    const size_t at = off;
+    off += (size_t)((bytes + 255) & ~255LL);
+    return at;
+  };
+  const size_t slabs = take(R->steps * R->slab * esz);
+  const size_t mpart = take(R->steps * K * nc * nm * 8);
+  const size_t mats = take(R->steps * K * (long long)sizeof(RevMat));
+  const size_t cpart = take((long long)kRevMaxCtas * 8 * 8);
+  const size_t lamh = take(R->steps * K * 4 * esz);
+  const size_t dkp = take((long long)R->splits * g.ND * 8);
+  if (R->block) {
+    char* p = (char*)R->block;
+    R->slabs = p + slabs;
+    R->mpart = p + mpart;
+    R->mats = p + mats;
+    R->cpart = p + cpart;
+    R->lamh = p + lamh;
+    R->dkp = (double*)(p + dkp);
+  }
+  return off;
+}
+
+void launch_rev_init(const Geo& g, const RevBuffers& R, Ctrl* ctrl, int nt, cudaStream_t st) {
+  cudaMemsetAsync(R.dkp, 0, sizeof(double) * (size_t)R.splits * g.ND, st);
+  launch(k_rev_init, 1, 1, 0, st, ctrl, nt);
+}
+void launch_rev_dksum(const Geo& g, const RevBuffers& R, double* dkref, cudaStream_t st) {
+  launch(k_rev_dksum, (g.ND + kRevThreads - 1) / kRevThreads, kRevThreads, 0, st, g.ND, R.splits,
+         (const double*)R.dkp, dkref);
+}
+
+template <typename T>
+void launch_rev_coef(const Geo& g, const RevBuffers& R, Ctrl* ctrl, const Dof* it, const T* kref, const Moments* mom,
+                     const T* boxstore, int nbox, int nsteps, int di, cudaStream_t st) {
+  LKS_REV_DISPATCH(coef_ax, g, R, ctrl, it, kref, mom, boxstore, nbox, nsteps, di, st);
+}
+template <typename T>
+void launch_rev_step(const Geo& g, const RevBuffers& R, Ctrl* ctrl, const Dof* it, T* Lb, long long lstride, int i,
+                     int di, cudaStream_t st) {
+  LKS_REV_DISPATCH(step_ax, g, R, ctrl, it, Lb, lstride, i, di, st);
+}
+template <typename T>
+void launch_rev_design(const Geo& g, const RevBuffers& R, Ctrl* ctrl, const Dof* it, int nsteps, int di,
+                       cudaStream_t st) {
+  LKS_REV_DISPATCH(design_ax, g, R, ctrl, it, nsteps, di, st);
+}
+
+#define LKS_REV_INST(T)                                                                                             \
+  template void launch_rev_coef<T>(const Geo&, const RevBuffers&, Ctrl*, const Dof*, const T*, const Moments*,      \
+                                   const T*, int, int, int, cudaStream_t);                                          \
+  template void launch_rev_step<T>(const Geo&, const RevBuffers&, Ctrl*, const Dof*, T*, long long, int, int,       \
+                                   cudaStream_t);                                                                   \
+  template void launch_rev_design<T>(const Geo&, const RevBuffers&, Ctrl*, const Dof*, int, int, cudaStream_t);
+LKS_REV_INST(float)
+LKS_REV_INST(double)
+
+}  // namespace lks
