@@ -60,8 +60,8 @@ typedef enum lks_status {
   LKS_ERR_ORDER = 7,        /* adjoint or sensitivity requested before a forward / adjoint */
   LKS_ERR_CUDA = 8,         /* a CUDA runtime call failed */
   LKS_ERR_UNSUPPORTED = 9,  /* valid but not supported by the library (e.g. grid/tile shape) */
-  LKS_ERR_TIMEOUT = 10      /* a bounded wait on the device (a grid barrier of the persistent coupling
-                             * kernels, or a tile copy of the row-streamed 3D stencils) waited longer
+  LKS_ERR_TIMEOUT = 10      /* a bounded wait on the device (a grid barrier or a flagged word of the
+                             * coupling kernels, or a tile copy of the row-streamed 3D stencils) waited longer
                              * than one second; the kernels returned early and the results of the call
                              * are void */
 } lks_status;
@@ -259,8 +259,8 @@ LKS_API int lks_get_initial_adjoint(lks_handle* h, double* lam_p_host, double* l
 LKS_API int lks_support_sets(lks_handle* h, const double* s_host, int* box_host, long long* stats_host,
                              size_t capacity);
 
-/* Test hook of the bounded grid barriers: skip != 0 makes the first CTA of every persistent coupling
- * kernel skip its barrier arrivals, so the other CTAs' waits run out (after one second) and the
+/* Test hook of the bounded waits of the coupling kernels: skip != 0 makes the first CTA of every
+ * persistent coupling kernel skip its barrier arrivals (its published words in 2D's default form), so the other CTAs' waits run out (after one second) and the
  * forward or adjoint returns LKS_ERR_TIMEOUT; skip = 0 restores normal operation. Synchronises the
  * device. Errors: LKS_ERR_ARG, LKS_ERR_CUDA. */
 LKS_API int lks_debug_sync_skip(lks_handle* h, int skip);
@@ -276,13 +276,17 @@ LKS_API int lks_debug_copy_skip(lks_handle* h, int skip);
 /* How the handle runs each step's N_itr coupling iterations (Sec. 3.1) and their reverse: mode 1 as
  * one persistent cooperative launch per step (grid barriers between the iterations) when the device
  * holds its grid, mode 0 as one launch per iteration (with the finish kernels), mode 2 (the default)
- * the persistent launch only where it measured faster (2D bodies whose box has more tiles than the
- * persistent grid has CTAs; the reverse about one rotation axis then runs by linear maps, whose
- * buffers the first lks_adjoint allocates if hbm_budget_bytes and the device have room), mode -1
- * only asks. Returns 1 if the persistent kernels are in use after
- * the call, 0 if not, or -status on error (LKS_ERR_ARG, LKS_ERR_CUDA). Changing the mode
- * synchronises the device; results agree to rounding (the per-CTA partial sums are grouped
- * differently). */
+ * by the problem: in 2D the forward runs as one cooperative launch per step whose CTAs exchange their
+ * sums through flagged words (bounded waits of one second, LKS_ERR_TIMEOUT), in 3D as one launch per
+ * iteration; the reverse about one rotation axis runs by linear maps of the iterations (no waits),
+ * with free rotation as one launch per iteration. The words and the maps' buffers are allocated by the
+ * first lks_forward and lks_adjoint if hbm_budget_bytes and the device have room; without it 2D bodies
+ * whose box has more tiles than the persistent grid has CTAs take the persistent launch and the others
+ * one launch per iteration. Mode -1 only asks. Returns 1 if the grid-barrier kernels are chosen (in
+ * mode 2: the body is 2D and its box has more tiles than their grid has CTAs, so that a CTA of the
+ * persistent launch works on several tiles), 0 if not, or -status on error (LKS_ERR_ARG,
+ * LKS_ERR_CUDA). Changing the mode synchronises the device; results agree to rounding (the per-CTA
+ * partial sums are grouped differently). */
 LKS_API int lks_persistent_coupling(lks_handle* h, int mode);
 
 /* Number of kernels this handle has launched (graph nodes counted per replay). */

@@ -292,6 +292,8 @@ struct lks_handle {
   Dof* it = nullptr;
   Ctrl* ctrl = nullptr;
   Moments* mom = nullptr;
+  void* words = nullptr;  // 2D: the coupling sums' flagged words (allocated by the first lks_forward)
+  bool no_words = false;  // the budget or the device had no room for them: the other forms run
   double* partials = nullptr;
   long long pstride = 0;  // elements per half of the double-buffered coupling partials
   double* init_p = nullptr;
@@ -529,6 +531,12 @@ void enqueue_fwd_steps(lks_handle* h, Launcher& L, const Slots<T>& S, int nsteps
   T* bs = store_box ? (T*)h->boxstore : nullptr;
   for (int i = 0; i < nsteps; ++i) {
     L("stencil_fwd", [&](cudaStream_t s) { launch_stencil_fwd<T>(g, S, h->ctrl, i, s); });
+    if (g.flag_ctas > 0) {  // 2D: all N_itr iterations and the last EOM, sums exchanged through flagged words
+      L("couple", [&](cudaStream_t s) {
+        launch_couple_flag<T>(g, S, h->ctrl, h->it, (const T*)h->kref, h->mom, h->words, bs, h->nbox, i, s);
+      });
+      continue;
+    }
     if (g.coop_fwd > 0) {  // all N_itr iterations and the last EOM in one persistent launch
       L("couple", [&](cudaStream_t s) {
         launch_couple_coop<T>(g, S, h->ctrl, h->it, (const T*)h->kref, h->mom, h->partials, h->pstride, bs, h->nbox,
@@ -615,6 +623,7 @@ int forward_impl(lks_handle* h, cudaStream_t st) {
   const Geo& g = h->g;
   const int NT = h->P.n_steps;
   Launcher L0{h, st, false};
+  if (g.flag_ctas > 0) CK(cudaMemsetAsync(h->words, 0, couple_flag_bytes(g.flag_ctas), st));
   CK(cudaMemsetAsync(&h->ctrl->sync_bar, 0, sizeof(unsigned), st));  // a barrier that timed out leaves it set
   if (h->P.ckpt_policy == LKS_CKPT_BINOMIAL) {
     // march in pieces between the snapshot steps of the first descent, snapshotting each
@@ -668,7 +677,7 @@ int forward_impl(lks_handle* h, cudaStream_t st) {
       }));
     }
   }
-  if (g.coop_fwd == 0)  // the persistent kernel runs the last EOM itself
+  if (g.coop_fwd == 0 && g.flag_ctas == 0)  // the persistent kernels run the last EOM themselves
     L0("couple", [&](cudaStream_t s) { launch_couple_last<T>(g, h->ctrl, h->it, h->mom, h->partials, h->pstride, NT, s); });
   CK(cudaGetLastError());
   if (h->launch_error) return LKS_ERR_CUDA;
@@ -780,6 +789,22 @@ int adjoint_impl(lks_handle* h, double seed, cudaStream_t st) {
   CK(cudaGetLastError());
   if (h->launch_error) return LKS_ERR_CUDA;
   return LKS_OK;
+}
+
+// Room for the flagged words of the 2D coupling; without it the handle keeps to the other forms.
+void choose_coupling(lks_handle* h) {
+  if (h->g.flag_ctas == 0 || h->words) return;
+  const size_t need = (couple_flag_bytes(kFlagMaxCtas) + 255) & ~(size_t)255;
+  const bool room = !h->P.hbm_budget_bytes || h->bytes + need <= h->P.hbm_budget_bytes;
+  if (!room || cudaMalloc(&h->words, need) != cudaSuccess) {
+    cudaGetLastError();
+    h->words = nullptr;
+    h->no_words = true;
+    h->g.flag_ctas = h->g.flag_threads = 0;
+    return;
+  }
+  h->bytes += need;
+  h->allocs.push_back(h->words);
 }
 
 // Chooses the form of the exact reverse: the linear maps for bodies about one axis in the automatic
@@ -932,6 +957,8 @@ int refresh_box(lks_handle* h) {
   const int old[3] = {h->g.B[0], h->g.B[1], h->g.B[2]};
   setup_box(&h->g, h->P.design_radius, rotated);
   h->g.coop_fwd = h->g.coop_adj = 0;
+  h->g.flag_ctas = h->g.flag_threads = 0;
+  if (h->coop_mode == 2 && !h->no_words) setup_couple_flag(&h->g, h->prec == LKS_FP64);
   if (h->coop_mode != 0) setup_coop(&h->g, h->prec == LKS_FP64);
   if (h->coop_mode == 2 && (h->g.dim != 2 || box_tiles(h->g) <= h->g.coop_fwd))
     h->g.coop_fwd = h->g.coop_adj = 0;  // measured slower there: a grid barrier costs about twice a
@@ -1044,6 +1071,7 @@ int lks_set_initial_state(lks_handle* h, const double* p, const double* u, const
 int lks_forward(lks_handle* h, const double* gamma_dev, double* J_host, void* stream) {
   if (!h || !gamma_dev) return LKS_ERR_ARG;
   cudaStream_t st = (cudaStream_t)stream;
+  choose_coupling(h);
   const Geo& g = h->g;
   h->fwd_done = h->adj_done = h->exact_done = h->alks_done = false;
   if ((const void*)gamma_dev != (const void*)h->gamma)

@@ -33,6 +33,7 @@
 #include <climits>
 
 #include "lks_body_common.cuh"
+#include "lks_wait.cuh"
 
 namespace lks {
 
@@ -986,14 +987,6 @@ __global__ void k_ckpt_pack(Geo g, Slots<T> S, T* ckpt, long long cstride, int e
 // order and runs the same FP64 EOM (or its reverse) on thread 0, so all CTAs hold the same iterate
 // without a second barrier. The partials are double-buffered by the parity of the iteration: a
 // buffer is rewritten only two barriers after it was read.
-
-constexpr unsigned long long kSyncTimeoutNs = 1000000000ull;  // one second
-
-__device__ __forceinline__ unsigned long long globaltimer_ns() {
-  unsigned long long t;
-  asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
-  return t;
-}
 
 __device__ __forceinline__ unsigned ld_acquire_gpu(const unsigned* p) {
   unsigned v;

@@ -1,0 +1,715 @@
+// All N_itr coupling iterations of a 2D step in one launch whose CTAs exchange their force and
+// torque sums and the iterate through flagged words (the default in 2D; lks_body.cu holds the forms
+// with one launch per iteration and with grid barriers).
+//
+// An iteration is short (a gather over the box's cells, three sums, the EOM), so its time is the
+// latency of the sums' way through the chip. CTA 0 has no cells: the others publish their three sums
+// to it, it adds them up, runs the EOM and publishes the iterate. Values travel as 64-bit words that
+// carry the iteration's number beside 32 bits of payload, so the arrival of the data is the
+// synchronisation: one trip through L2 each way, and every waiting CTA polls one or two lines. (A form
+// in which every CTA polled the words of all others and ran the EOM itself needed one trip only, but
+// took 4.3 us an iteration without gather and EOM on 148 SMs: 57 lines polled by all of them.)
+// A word's number tells it from the one two iterations earlier in the same place (two places by the
+// iteration's parity): sums of iteration e + 2 are published after the iterate of e + 1 was read,
+// which CTA 0 publishes after it has read the sums of e; and likewise the other way. All sums are
+// taken in a fixed order (warps, CTA, then 32 lanes over the CTAs), so results do not vary between
+// runs.
+//
+// Warps are dealt over the box round robin, so the design-free corners of a rotating body's box are
+// shared evenly between the CTAs. The launch is cooperative (all CTAs resident); waits are bounded by
+// one second as those of the grid barriers.
+//
+// What bounds it: the gather's slowest warps and two trips through L2 per iteration. Forward march
+// measured on GB300, N_itr launches (or grid barriers) per step -> this kernel, us per step: 512x256
+// body of 128^2 60 -> 37; 1024x512, 256^2 (grid barriers before) 100 -> 58; FP64 80x40, 16^2 290 -> 58;
+// FP64 600x100, 20^2 500 -> 67.
+#include <climits>
+
+#include "lks_body_common.cuh"
+#include "lks_wait.cuh"
+
+namespace lks {
+
+namespace {
+
+constexpr int NVC = 3;  // force x, y and torque
+
+// Lanes per cell and the largest CTA. FP32: 2 lanes split a cell's candidate rows (the gather is bound
+// by issue: with 4 lanes the uneven rows and each lane's setup cost more than the extra warps hide).
+// FP64 issues one warp instruction per 64 cycles and scheduler, so 16 lanes take one to four
+// candidates each and a small box spreads over all SMs.
+template <typename T>
+struct FlagCta;
+template <>
+struct FlagCta<float> {
+  static constexpr int lanes = 2, max_threads = 640;
+};
+template <>
+struct FlagCta<double> {
+  static constexpr int lanes = 16, max_threads = 512;
+};
+
+// Sums over the design points of one cell, e = xi_m - xi(cell) the offset from the cell's image in
+// the design frame: phi, kappa, sum W e, sum W kappa e; then moved to the pivot (sum W r).
+template <typename T>
+__device__ __forceinline__ void to_pivot(T xb, T xc, T eb, T ec, T kb, T kc, Acc<T>& o) {
+  o.wr[0] = eb + xb * o.phi;
+  o.wr[1] = ec + xc * o.phi;
+  o.kr[0] = kb + xb * o.kap;
+  o.kr[1] = kc + xc * o.kap;
+  o.wr[2] = o.kr[2] = T(0);
+}
+
+// FP32. Lane cl takes the candidate rows cl, cl + 2, ...; within a row the interval of candidates
+// follows from the two support bounds (linear in the offset), widened, and the exact test decides.
+// Cosine kernel: with the rotation scaled by pi/2 the offsets are the cosines' arguments; the factor
+// 1/16 of the two weights is applied to the sums.
+__device__ __forceinline__ void gather2d(const Geo& g, const float* __restrict__ kref, const float (&d)[2], float cs,
+                                         float sn, int cl, bool active, Acc<float>& o) {
+  constexpr int LC = FlagCta<float>::lanes;
+  const float S = (float)g.s, pad = 1e-3f, tiny = 1e-6f;
+  const float xb = cs * d[0] + sn * d[1], xc = cs * d[1] - sn * d[0];
+  const float xib = xb + g.xicf[0], xic = xc + g.xicf[1];
+  const float h = S * (fabsf(cs) + fabsf(sn));
+  const int nx = g.nd[0];
+  const int ib0 = max(0, (int)ceilf(xib - h)), ib1 = min(nx - 1, (int)floorf(xib + h));
+  const int ic0 = max(0, (int)ceilf(xic - h)), ic1 = min(g.nd[1] - 1, (int)floorf(xic + h));
+  float phi = 0.0f, kap = 0.0f, sb = 0.0f, sc = 0.0f, kb = 0.0f, kc = 0.0f;
+  if (active && ib0 <= ib1) {
+    const bool cosine = g.wk == W_COS4, ball = g.rad4 != INT_MAX;
+    const float sw = cosine ? 1.57079632679f : 1.0f, Sw = cosine ? 3.14159265359f : 1.0f;
+    const float cw = sw * cs, nw = sw * sn;
+    const float ics = fabsf(cs) > tiny ? 1.0f / cs : 0.0f, isn = fabsf(sn) > tiny ? 1.0f / sn : 0.0f;
+    for (int ic = ic0 + cl; ic <= ic1; ic += LC) {
+      const float ec = (float)ic - xic;
+      float lo = -1e6f, hi = 1e6f;
+      if (ics != 0.0f) {
+        const float e1 = (sn * ec - S) * ics, e2 = (sn * ec + S) * ics;
+        lo = fmaxf(lo, fminf(e1, e2));
+        hi = fminf(hi, fmaxf(e1, e2));
+      } else if (fabsf(sn * ec) >= S + pad) {
+        continue;
+      }
+      if (isn != 0.0f) {
+        const float e1 = (-S - cs * ec) * isn, e2 = (S - cs * ec) * isn;
+        lo = fmaxf(lo, fminf(e1, e2));
+        hi = fminf(hi, fmaxf(e1, e2));
+      } else if (fabsf(cs * ec) >= S + pad) {
+        continue;
+      }
+      const int j0 = max(ib0, (int)ceilf(xib + lo - pad)), j1 = min(ib1, (int)floorf(xib + hi + pad));
+      if (j0 > j1) continue;
+      // a chord of the rotated support square is at most 4 sqrt 2 long: six candidates, all taken at
+      // once (masked) so that their loads and cosines overlap
+      const float* kr = kref + (long long)ic * nx;
+      float kv[6];
+#pragma unroll
+      for (int j = 0; j < 6; ++j) kv[j] = __ldg(kr + min(j0 + j, j1));
+      const float ob0 = -nw * ec, oc0 = cw * ec;
+      float ps = 0.0f, pk = 0.0f;
+#pragma unroll
+      for (int j = 0; j < 6; ++j) {
+        const int ib = j0 + j;
+        const float eb = (float)ib - xib;
+        const float ob = fmaf(cw, eb, ob0), oc = fmaf(nw, eb, oc0);
+        bool ok = ib <= j1 && fabsf(ob) < Sw && fabsf(oc) < Sw;
+        if (ball) ok = ok && dsq(ib, nx) + dsq(ic, g.nd[1]) <= g.rad4;
+        float w = cosine ? (1.0f + __cosf(ob)) * (1.0f + __cosf(oc)) : (1.0f - fabsf(ob)) * (1.0f - fabsf(oc));
+        w = ok ? w : 0.0f;
+        const float wk = w * kv[j];
+        ps += w;
+        pk += wk;
+        sb = fmaf(w, eb, sb);
+        kb = fmaf(wk, eb, kb);
+      }
+      phi += ps;
+      kap += pk;
+      sc = fmaf(ps, ec, sc);
+      kc = fmaf(pk, ec, kc);
+    }
+    const float f = cosine ? 0.0625f : 1.0f;
+    phi *= f;
+    kap *= f;
+    sb *= f;
+    sc *= f;
+    kb *= f;
+    kc *= f;
+  }
+#pragma unroll
+  for (int off = 1; off < LC; off <<= 1) {
+    phi += __shfl_xor_sync(0xffffffffu, phi, off);
+    kap += __shfl_xor_sync(0xffffffffu, kap, off);
+    sb += __shfl_xor_sync(0xffffffffu, sb, off);
+    sc += __shfl_xor_sync(0xffffffffu, sc, off);
+    kb += __shfl_xor_sync(0xffffffffu, kb, off);
+    kc += __shfl_xor_sync(0xffffffffu, kc, off);
+  }
+  o.phi = phi;
+  o.kap = kap;
+  to_pivot(xb, xc, sb, sc, kb, kc, o);
+}
+
+// FP64: lane (cl >> 2, cl & 3) takes every fourth row and column of the candidates' bounding
+// square; the test against the support is made in FP32 first (widened by more than its rounding),
+// so FP64 instructions are spent on accepted candidates only. The six sums of the 16 lanes are
+// combined by halving (each level exchanges half of the values: 8 additions, not 24).
+__device__ __forceinline__ void gather2d(const Geo& g, const double* __restrict__ kref, const double (&d)[2],
+                                         double cs, double sn, int cl, bool active, Acc<double>& o) {
+  const double S = (double)g.s;
+  const double xb = cs * d[0] + sn * d[1], xc = cs * d[1] - sn * d[0];
+  const double xib = xb + g.xic[0], xic = xc + g.xic[1];
+  const float csf = (float)cs, snf = (float)sn, pad = 2e-3f, Sp = (float)g.s + pad;
+  const float xibf = (float)xib, xicf = (float)xic;
+  const float h = Sp * (fabsf(csf) + fabsf(snf)) + pad;
+  const int ib0 = max(0, (int)ceilf(xibf - h)), ic0 = max(0, (int)ceilf(xicf - h));
+  const int ib1 = active ? min(g.nd[0] - 1, (int)floorf(xibf + h)) : -1;
+  const int ic1 = min(g.nd[1] - 1, (int)floorf(xicf + h));
+  double v[8];
+#pragma unroll
+  for (int i = 0; i < 8; ++i) v[i] = 0.0;
+  for (int ib = ib0 + (cl >> 2); ib <= ib1; ib += 4)
+    for (int ic = ic0 + (cl & 3); ic <= ic1; ic += 4) {
+      const float ebf = (float)ib - xibf, ecf = (float)ic - xicf;
+      if (fabsf(csf * ebf - snf * ecf) >= Sp || fabsf(snf * ebf + csf * ecf) >= Sp) continue;
+      if (dsq(ib, g.nd[0]) + dsq(ic, g.nd[1]) > g.rad4) continue;
+      const double eb = (double)ib - xib, ec = (double)ic - xic;
+      const double ob = cs * eb - sn * ec, oc = sn * eb + cs * ec;
+      if (fabs(ob) >= S || fabs(oc) >= S) continue;
+      const double w = wfun(g.wk, ob) * wfun(g.wk, oc), wk = w * kref[ib + ic * g.nd[0]];
+      v[0] += w;
+      v[1] += wk;
+      v[2] += w * eb;
+      v[3] += w * ec;
+      v[4] += wk * eb;
+      v[5] += wk * ec;
+    }
+  // halving over lane bits 3, 2, 1 (value index bits 2, 1, 0), then the pair of bit 0
+  const bool b3 = cl & 8, b2 = cl & 4, b1 = cl & 2;
+  double a[4], b[2], c;
+#pragma unroll
+  for (int i = 0; i < 4; ++i) a[i] = (b3 ? v[4 + i] : v[i]) + __shfl_xor_sync(0xffffffffu, b3 ? v[i] : v[4 + i], 8);
+#pragma unroll
+  for (int i = 0; i < 2; ++i) b[i] = (b2 ? a[2 + i] : a[i]) + __shfl_xor_sync(0xffffffffu, b2 ? a[i] : a[2 + i], 4);
+  c = (b1 ? b[1] : b[0]) + __shfl_xor_sync(0xffffffffu, b1 ? b[0] : b[1], 2);
+  c += __shfl_xor_sync(0xffffffffu, c, 1);
+  o.phi = __shfl_sync(0xffffffffu, c, 0, 16);
+  o.kap = __shfl_sync(0xffffffffu, c, 2, 16);
+  const double sb = __shfl_sync(0xffffffffu, c, 4, 16), sc = __shfl_sync(0xffffffffu, c, 6, 16);
+  const double kb = __shfl_sync(0xffffffffu, c, 8, 16), kc = __shfl_sync(0xffffffffu, c, 10, 16);
+  to_pivot(xb, xc, sb, sc, kb, kc, o);
+}
+
+// One value as two 64-bit words (number << 32 | payload) and back.
+struct Words {
+  unsigned long long a, b;
+};
+__device__ __forceinline__ void st_words(Words* p, Words w) {
+  asm volatile("st.relaxed.gpu.global.v2.u64 [%0], {%1, %2};" ::"l"(p), "l"(w.a), "l"(w.b) : "memory");
+}
+__device__ __forceinline__ Words ld_words(const Words* p) {
+  Words w;
+  asm volatile("ld.relaxed.gpu.global.v2.u64 {%0, %1}, [%2];" : "=l"(w.a), "=l"(w.b) : "l"(p) : "memory");
+  return w;
+}
+__device__ __forceinline__ Words pack(unsigned e, unsigned x, unsigned y) {
+  return Words{((unsigned long long)e << 32) | x, ((unsigned long long)e << 32) | y};
+}
+
+// The value of a whole warp's lanes (fixed order), and a CTA's or the grid's sum of one component.
+struct Df {
+  float hi, lo;
+  __device__ __forceinline__ void zero() { hi = lo = 0.0f; }
+  __device__ __forceinline__ void set(float v) { hi = v, lo = 0.0f; }
+  __device__ __forceinline__ void add(const Df& o) { df_add(hi, lo, o.hi, o.lo); }
+  __device__ __forceinline__ Df from_xor(int off) const {
+    return Df{__shfl_xor_sync(0xffffffffu, hi, off), __shfl_xor_sync(0xffffffffu, lo, off)};
+  }
+  __device__ __forceinline__ Words words(unsigned e) const { return pack(e, __float_as_uint(hi), __float_as_uint(lo)); }
+  __device__ __forceinline__ void read(const Words& w) {
+    hi = __uint_as_float((unsigned)w.a);
+    lo = __uint_as_float((unsigned)w.b);
+  }
+  __device__ __forceinline__ double value() const { return (double)hi + (double)lo; }
+};
+struct Dd {
+  double v;
+  __device__ __forceinline__ void zero() { v = 0.0; }
+  __device__ __forceinline__ void set(double x) { v = x; }
+  __device__ __forceinline__ void add(const Dd& o) { v += o.v; }
+  __device__ __forceinline__ Dd from_xor(int off) const { return Dd{__shfl_xor_sync(0xffffffffu, v, off)}; }
+  __device__ __forceinline__ Words words(unsigned e) const {
+    const unsigned long long b = (unsigned long long)__double_as_longlong(v);
+    return pack(e, (unsigned)b, (unsigned)(b >> 32));
+  }
+  __device__ __forceinline__ void read(const Words& w) {
+    v = __longlong_as_double((long long)((w.a & 0xffffffffull) | (w.b << 32)));
+  }
+  __device__ __forceinline__ double value() const { return v; }
+};
+template <typename T>
+struct SumOf;
+template <>
+struct SumOf<float> {
+  using type = Df;
+};
+template <>
+struct SumOf<double> {
+  using type = Dd;
+};
+template <int STRIDE, typename V>
+__device__ __forceinline__ void warp_total(V& v) {
+#pragma unroll
+  for (int off = 16; off >= STRIDE; off >>= 1) v.add(v.from_xor(off));
+}
+
+// EOM of an iteration, one component per warp (0, 1: an axis; 2: the rotation), in FP64. Every FP64
+// instruction of a warp costs 64 cycles, dependent or not, so prepare (while the other warps gather)
+// does what does not need the sums, and finish spends about a dozen. The cosine of the step's rotation
+// is taken on the even lanes and its sine on the odd ones by the same instructions with their own
+// coefficients. Range tests are made on the exponent in integers. All lanes of the warp call both.
+struct EomPart {
+  double c0, im, q0, f0, x0, y0;  // v = s im + c0; q = q0 + v; f0 = frac(q0); cos/sin(t-1) by lane
+  int xi0;
+  bool fr;
+  __device__ __forceinline__ void prepare(const Geo& g, const Moments& mom, const Dof& s0, const Dof& sk, int comp,
+                                          int lane) {
+    const double cs = sk.cs, sn = sk.sn, om = sk.s[7];
+    const double kx = cs * mom.K1[0] - sn * mom.K1[1], ky = sn * mom.K1[0] + cs * mom.K1[1];
+    double pre, v0;
+    if (comp < 2) {
+      pre = mom.K0 * sk.s[3 + comp] + om * (comp == 0 ? -ky : kx);
+      fr = (g.dof_mask & (1 << comp)) != 0;
+      v0 = s0.s[3 + comp];
+      im = g.inv_mass;
+      q0 = s0.s[comp];
+      const double fl = floor(q0);
+      xi0 = (int)fl;
+      f0 = q0 - fl;
+    } else {
+      pre = (kx * sk.s[4] - ky * sk.s[3]) + om * mom.K2p;
+      fr = (g.dof_mask & DOF_ROT) != 0;
+      v0 = s0.s[7];
+      im = g.inv_inertia;
+      q0 = s0.s[6];
+      x0 = (lane & 1) ? s0.sn : s0.cs;  // cos' = cs c - sn s, sin' = sn c + cs s
+      y0 = (lane & 1) ? s0.cs : -s0.sn;
+    }
+    c0 = fr ? v0 - pre * im : v0;
+    if (!fr) im = 0.0;
+  }
+  // s: the component's sum. Writes the iterate's entries to nx and publishes those the gather reads
+  // (see Pose); returns the status bits.
+  template <typename T>
+  __device__ __forceinline__ int finish(const Geo& g, double s, Dof* nx, unsigned long long* pose, unsigned e, int comp,
+                                        int lane) const;
+};
+
+// What the cells need of an iterate, and its words: FP32 per axis u^G, fraction and floor of x^G, then
+// cos, sin, omega (9 words); FP64 per axis u^G and x^G, then cos, sin, omega (14 words).
+template <typename T>
+struct Pose;
+template <>
+struct Pose<float> {
+  static constexpr int words = 9;
+  float cs, sn, om, ug[2], xf[2];
+  int xi[2];
+  __device__ __forceinline__ void set(const Dof& d) {
+    cs = d.csf, sn = d.snf, om = d.om;
+    for (int a = 0; a < 2; ++a) ug[a] = d.ug[a], xf[a] = d.xf[a], xi[a] = d.xi[a];
+  }
+  // word w of the iterate
+  __device__ __forceinline__ void put(int w, unsigned p, unsigned) {
+    const float f = __uint_as_float(p);
+    if (w < 6) {
+      const int a = w >= 3 ? 1 : 0, i = w - 3 * a;
+      if (i == 0) ug[a] = f;
+      if (i == 1) xf[a] = f;
+      if (i == 2) xi[a] = (int)p;
+    } else {
+      (w == 6 ? cs : w == 7 ? sn : om) = f;
+    }
+  }
+  __device__ __forceinline__ float rel(int a, int p) const { return (float)(p - xi[a]) - xf[a]; }
+};
+template <>
+struct Pose<double> {
+  static constexpr int words = 14;
+  double cs, sn, om, ug[2], x[2];
+  __device__ __forceinline__ void set(const Dof& d) {
+    cs = d.cs, sn = d.sn, om = d.s[7];
+    for (int a = 0; a < 2; ++a) ug[a] = d.s[3 + a], x[a] = d.s[a];
+  }
+  // the low word w (even) of the iterate, hi the next one
+  __device__ __forceinline__ void put(int w, unsigned p, unsigned hi) {
+    if (w & 1) return;
+    const double f = __hiloint2double((int)hi, (int)p);
+    if (w < 8) {
+      const int a = w >= 4 ? 1 : 0;
+      (w & 2 ? x[a] : ug[a]) = f;
+    } else {
+      (w == 8 ? cs : w == 10 ? sn : om) = f;
+    }
+  }
+  __device__ __forceinline__ double rel(int a, int p) const { return (double)p - x[a]; }
+};
+
+__device__ __forceinline__ void st_word(unsigned long long* p, unsigned e, unsigned payload) {
+  asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(((unsigned long long)e << 32) | payload) : "memory");
+}
+__device__ __forceinline__ unsigned long long ld_word(const unsigned long long* p) {
+  unsigned long long w;
+  asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(w) : "l"(p) : "memory");
+  return w;
+}
+
+template <typename T>
+__device__ __forceinline__ int EomPart::finish(const Geo& g, double s, Dof* nx, unsigned long long* pose, unsigned e,
+                                               int comp, int lane) const {
+  constexpr bool D64 = sizeof(T) == 8;
+  const double v = fma(s, im, c0);
+  const int hi = __double2hiint(v) & 0x7fffffff;
+  int st = 0;
+  if (hi >= 0x7ff00000 || (__double2hiint(s) & 0x7fffffff) >= 0x7ff00000) st = ST_NONFINITE;
+  if (comp < 2) {
+    const double q = fr ? q0 + v : q0;
+    if constexpr (D64) {
+      const double w = lane < 2 ? v : q;
+      if (lane < 4) st_word(pose + 4 * comp + lane, e, (unsigned)((lane & 1) ? __double2hiint(w) : __double2loint(w)));
+    }
+    if (hi >= 0x3ff00000 && fr && fabs(v) > (double)g.margin) st |= ST_BOX_OVERFLOW;
+    // floor and fraction of the position from those of t-1 (a crossing renews them)
+    double f = fr ? f0 + v : f0;
+    int xi = xi0;
+    const int hf = __double2hiint(f);
+    if (hf < 0 || hf >= 0x3ff00000) {
+      const double fl = floor(f);
+      xi += (int)fl;
+      f -= fl;
+    }
+    const float vf = (float)v, ff = (float)f;
+    if constexpr (!D64) {
+      const unsigned w = lane == 0 ? __float_as_uint(vf) : (lane == 1 ? __float_as_uint(ff) : (unsigned)xi);
+      if (lane < 3) st_word(pose + 3 * comp + lane, e, w);
+    }
+    if (lane == 0) {
+      nx->s[comp] = q;
+      nx->s[3 + comp] = v;
+      nx->xi[comp] = xi;
+      nx->xf[comp] = ff;
+      nx->ug[comp] = vf;
+    }
+    return st;
+  }
+  const bool sine = lane & 1;
+  const double x = fr ? v : 0.0;  // the step's rotation
+  const int hx = fr ? hi : 0;
+  double p;
+  if (hx > 0x3fd00000) {  // above 1/4
+    double sd, cd;
+    sincos(x, &sd, &cd);
+    p = sine ? sd : cd;
+  } else {
+    // sums of (-1)^k x^2k / (2k)! and x (-1)^k x^2k / (2k+1)!: up to |x| = 2^-10 three terms leave
+    // less than 2e-21, up to 1/64 five (1e-25), up to 1/4 nine (1e-27)
+    const double x2 = x * x;
+    p = 0.0;
+    if (hx > 0x3f500000) {
+      if (hx > 0x3f900000) {
+        p = sine ? 1.0 / 355687428096000.0 : 1.0 / 20922789888000.0;
+        p = fma(p, x2, sine ? -1.0 / 1307674368000.0 : -1.0 / 87178291200.0);
+        p = fma(p, x2, sine ? 1.0 / 6227020800.0 : 1.0 / 479001600.0);
+        p = fma(p, x2, sine ? -1.0 / 39916800.0 : -1.0 / 3628800.0);
+      }
+      p = fma(p, x2, sine ? 1.0 / 362880.0 : 1.0 / 40320.0);
+      p = fma(p, x2, sine ? -1.0 / 5040.0 : -1.0 / 720.0);
+    }
+    p = fma(p, x2, sine ? 1.0 / 120.0 : 1.0 / 24.0);
+    p = fma(p, x2, sine ? -1.0 / 6.0 : -1.0 / 2.0);
+    p = fma(p, x2, 1.0);
+    const double ps = p * x;
+    if (sine) p = ps;
+  }
+  const double other = __shfl_xor_sync(0xffffffffu, p, 1);
+  const double trig = fma(x0, sine ? other : p, y0 * (sine ? p : other));  // cos, sin by lane parity
+  const float tf = (float)trig, vf = (float)v;
+  if constexpr (D64) {
+    const double c = __shfl_sync(0xffffffffu, trig, 0), sn = __shfl_sync(0xffffffffu, trig, 1);
+    const double w = lane < 2 ? c : (lane < 4 ? sn : v);
+    if (lane < 6) st_word(pose + 8 + lane, e, (unsigned)((lane & 1) ? __double2hiint(w) : __double2loint(w)));
+  } else {
+    if (lane < 3) st_word(pose + 6 + lane, e, __float_as_uint(lane < 2 ? tf : vf));
+  }
+  if (lane == 0) {
+    nx->s[6] = fr ? q0 + v : q0;
+    nx->s[7] = v;
+    nx->om = vf;
+    nx->cs = trig;
+    nx->csf = tf;
+  } else if (lane == 1) {
+    nx->sn = trig;
+    nx->snf = tf;
+  }
+  return st;
+}
+
+// The exchange's words: sums [parity][component][CTA], then iterates [parity][16].
+__device__ __forceinline__ Words* sum_words(void* w, unsigned e, int comp, int cells) {
+  return static_cast<Words*>(w) + ((long long)(e & 1u) * NVC + comp) * cells;
+}
+__device__ __forceinline__ unsigned long long* pose_words(void* w, unsigned e, int cells) {
+  return reinterpret_cast<unsigned long long*>(static_cast<Words*>(w) + 2LL * NVC * cells) + (e & 1u) * 16;
+}
+
+// CTA 0: warp `comp` adds the CTAs' sums of its component and runs its part of the EOM.
+template <typename T>
+__device__ __forceinline__ void flag_root(const Geo& g, Ctrl* ctrl, Dof* row, const Moments* __restrict__ mom,
+                                          void* words, int cells, unsigned e0, bool skip, Dof (&sd)[2], int& gave_up) {
+  using V = typename SumOf<T>::type;
+  constexpr int DW = (int)(sizeof(Dof) / sizeof(double));
+  const int tid = threadIdx.x, comp = tid >> 5, lane = tid & 31, K = g.K;
+  if (comp >= NVC) return;
+  auto sync = [] { asm volatile("bar.sync 1, %0;" ::"n"(NVC * 32) : "memory"); };
+  double* sdw = reinterpret_cast<double*>(sd);
+  for (int k = 1; k <= K; ++k) {
+    const unsigned e = e0 + (unsigned)k;
+    EomPart eom;
+    eom.prepare(g, *mom, sd[0], sd[1], comp, lane);
+    const Words* place = sum_words(words, e, comp, cells);
+    V s;
+    s.zero();
+    WaitLimit limit;
+    bool ok = true;
+    for (int q0 = lane; q0 < cells && ok; q0 += 32 * 4) {
+      Words w[4];
+      bool have;
+      do {  // up to four words at a time in flight
+        have = true;
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+          if (q0 + 32 * j < cells) w[j] = ld_words(place + q0 + 32 * j);
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+          if (q0 + 32 * j < cells) have = have && (unsigned)(w[j].a >> 32) == e && (unsigned)(w[j].b >> 32) == e;
+        if (!have && limit.over(&ctrl->status)) ok = false;
+      } while (!have && ok);
+      if (ok)
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+          if (q0 + 32 * j < cells) {
+            V x;
+            x.read(w[j]);
+            s.add(x);
+          }
+    }
+    __syncwarp();
+    ok = __all_sync(0xffffffffu, ok);
+    if (!ok && lane == 0) gave_up = 1;
+    sync();  // every warp has read sd[1]
+    if (gave_up) return;
+    warp_total<1>(s);
+    // the skip hook (a test) publishes into the sums' unused parity-free end: no one reads it
+    unsigned long long* pose = skip ? pose_words(words, 0u, cells) + 32 : pose_words(words, e, cells);
+    const int st = eom.finish<T>(g, s.value(), &sd[1], pose, e, comp, lane);
+    if (st && lane == 0) atomicOr(&ctrl->status, st);
+    sync();
+    if (tid < DW) {
+      reinterpret_cast<double*>(row + k)[tid] = sdw[DW + tid];
+      if (k == K) reinterpret_cast<double*>(row + K + 1)[tid] = sdw[DW + tid];  // s(t): the next step's row 0
+    }
+  }
+}
+
+template <typename T>
+__global__ void __launch_bounds__(FlagCta<T>::max_threads, 1)
+    k_couple_flag(Geo g, Slots<T> S, Ctrl* ctrl, Dof* it, const T* __restrict__ kref, const Moments* __restrict__ mom,
+                  void* words, T* __restrict__ boxstore, int nbox, int di) {
+  using V = typename SumOf<T>::type;
+  constexpr int LC = FlagCta<T>::lanes, CPW = 32 / LC;  // lanes per cell, cells per warp
+  constexpr int DW = (int)(sizeof(Dof) / sizeof(double));
+  __shared__ V part[32 * NVC];
+  __shared__ Dof sd[2];  // CTA 0: s(t-1), the current iterate
+  __shared__ Pose<T> pose;
+  __shared__ int gave_up;
+  if (*(volatile int*)&ctrl->status & ST_SYNC_TIMEOUT) return;  // an earlier launch gave up
+  const int t = ctrl->t0 + di, base = ctrl->base, K = g.K;
+  Dof* row = it + (long long)(t - 1) * (K + 1);
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, nw = (int)(blockDim.x >> 5);
+  const int G = (int)gridDim.x - 1, cta = (int)blockIdx.x - 1;  // CTAs with cells
+  const unsigned e0 = (unsigned)((long long)(t - 1) * K);
+  if (tid < DW) {
+    const double v = reinterpret_cast<const double*>(row)[tid];
+    reinterpret_cast<double*>(sd)[tid] = v;
+    reinterpret_cast<double*>(sd)[DW + tid] = v;
+  }
+  if (tid == 0) gave_up = 0;
+  __syncthreads();
+  if (cta < 0) {
+    flag_root<T>(g, ctrl, row, mom, words, G, e0, (ctrl->sync_skip & 1) != 0, sd, gave_up);
+    return;
+  }
+  if (tid == 0) pose.set(sd[0]);
+  T* __restrict__ dst = slot_ptr(S, t, base);
+  int lo[3];
+  box_origin<2>(g, sd[0], lo[0], lo[1], lo[2]);
+  T* bs = boxstore ? boxstore + (long long)((t - base - 1) % nbox) * g.box_cells * 2 : nullptr;
+  const long long N = g.N;
+  const int BC = (int)g.box_cells, W = G * nw, sub = lane / LC, cl = lane % LC;
+  const int first = (warp * G + cta) * CPW;
+  // position, grid index and u* of this thread's first cell stay in registers through the iterations
+  struct Cell {
+    int px, py, n;  // n < 0: outside the grid
+  };
+  auto cell_of = [&](int bl) {
+    Cell c{0, 0, -1};
+    if (bl < BC) {
+      const int j1 = bl / g.B[0];
+      c.px = lo[0] + bl - j1 * g.B[0];
+      c.py = lo[1] + j1;
+      long long n;
+      if (cell_index<2>(g, c.px, c.py, 0, n)) c.n = (int)n;
+    }
+    return c;
+  };
+  const Cell cell0 = cell_of(first + sub);
+  T ust0[2] = {T(0), T(0)};
+  if (cell0.n >= 0) {
+    ust0[0] = dst[N + cell0.n];
+    ust0[1] = dst[2 * N + cell0.n];
+  }
+  __syncthreads();
+  for (int k = 1; k <= K; ++k) {
+    const bool last = k == K;
+    const unsigned e = e0 + (unsigned)k;
+    const Pose<T> P = pose;
+    T v[NVC] = {T(0), T(0), T(0)};
+    for (int c0 = first; c0 < BC; c0 += W * CPW) {  // uniform per warp
+      const int bl = c0 + sub;
+      const Cell cc = c0 == first ? cell0 : cell_of(bl);
+      const int n = cc.n;
+      const T d[2] = {P.rel(0, cc.px), P.rel(1, cc.py)};
+      Acc<T> A;
+      gather2d(g, kref, d, P.cs, P.sn, cl, bl < BC, A);
+      if (bl >= BC || cl != 0) continue;
+      if (A.phi == T(0)) {  // no design point in reach: u = u*
+        if (last && bs && n >= 0) {
+          bs[bl] = c0 == first ? ust0[0] : dst[N + n];
+          bs[g.box_cells + bl] = c0 == first ? ust0[1] : dst[2 * N + n];
+        }
+        continue;
+      }
+      if (n < 0 || forbidden<2>(g, cc.px, cc.py, 0)) atomicOr(&ctrl->status, ST_BODY_OUTSIDE);
+      if (n < 0) continue;
+      T dwr[3], L[3];
+      drot<2>(P.cs, P.sn, A.wr, dwr);
+      rot<2>(P.cs, P.sn, A.kr, L);
+      const T inv = T(1) / (T(1) + A.kap);
+      T u[2];
+#pragma unroll
+      for (int a = 0; a < 2; ++a) {
+        const T us = P.ug[a] * A.phi + P.om * dwr[a];
+        const T ustar = c0 == first ? ust0[a] : dst[(a + 1) * N + n];
+        u[a] = (ustar + A.kap * us) * inv;
+        v[a] += A.kap * u[a];
+        if (last) {
+          if (bs) bs[a * g.box_cells + bl] = ustar;
+          dst[(a + 1) * N + n] = u[a];
+        }
+      }
+      v[2] += L[0] * u[1] - L[1] * u[0];
+    }
+    __syncwarp();
+    // the lanes with cl = 0 hold the values: lane cl takes component cl of its cell (two components a
+    // lane in FP32), so the trees over the cells run side by side
+    constexpr int per = (NVC + LC - 1) / LC;
+#pragma unroll
+    for (int q = 0; q < per; ++q) {
+      T x = T(0);
+#pragma unroll
+      for (int i = 0; i < NVC; ++i) {
+        const T y = __shfl_sync(0xffffffffu, v[i], lane - cl);
+        if (i == cl + q * LC) x = y;
+      }
+      V s;
+      s.set(x);
+      warp_total<LC>(s);
+      if (lane + q * LC < NVC && lane < LC) part[warp * NVC + lane + q * LC] = s;
+    }
+    __syncthreads();
+    if (warp < NVC) {  // the CTA's sum of component `warp`
+      V s;
+      s.zero();
+      if (lane < nw) s = part[lane * NVC + warp];
+      warp_total<1>(s);
+      if (lane == 0) st_words(sum_words(words, e, warp, G) + cta, s.words(e));
+    }
+    if (last) return;
+    if (warp == NVC) {  // the next iterate
+      const unsigned long long* p = pose_words(words, e, G);
+      unsigned long long w = 0;
+      WaitLimit limit;
+      bool ok = true;
+      if (lane < Pose<T>::words)
+        while ((unsigned)((w = ld_word(p + lane)) >> 32) != e)
+          if (limit.over(&ctrl->status)) {
+            ok = false;
+            break;
+          }
+      __syncwarp();
+      const unsigned hi = __shfl_down_sync(0xffffffffu, (unsigned)w, 1);
+      if (lane < Pose<T>::words) {
+        if (ok)
+          pose.put(lane, (unsigned)w, hi);
+        else
+          gave_up = 1;
+      }
+    }
+    __syncthreads();
+    if (gave_up) return;
+  }
+}
+
+template <typename T>
+int flag_shape(const Geo& g, int* threads) {
+  int dev = 0, sms = 0, per_sm = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess) return 0;
+  if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms < 2) return 0;
+  const long long want = g.box_cells * FlagCta<T>::lanes;
+  // one CTA per SM, one SM for CTA 0: as few publishers as fill the chip, each with the threads its
+  // share needs
+  long long nt = (want + sms - 2) / (sms - 1);
+  nt = (nt + 31) / 32 * 32;
+  if (nt < 128) nt = 128;  // a warp per scheduler; three sum, the fourth waits for the iterate
+  if (nt > FlagCta<T>::max_threads) nt = FlagCta<T>::max_threads;
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_couple_flag<T>, (int)nt, 0) != cudaSuccess) return 0;
+  if (per_sm < 1) return 0;
+  const long long ctas = (want + nt - 1) / nt + 1;
+  *threads = (int)nt;
+  const long long cap = sms < kFlagMaxCtas ? sms : kFlagMaxCtas;
+  return (int)(ctas < cap ? ctas : cap);
+}
+
+}  // namespace
+
+void setup_couple_flag(Geo* g, bool fp64) {
+  g->flag_ctas = g->flag_threads = 0;
+  if (g->dim != 2 || g->box_cells >= (1LL << 27) || g->N >= (1LL << 31)) return;
+  g->flag_ctas = fp64 ? flag_shape<double>(*g, &g->flag_threads) : flag_shape<float>(*g, &g->flag_threads);
+  cudaGetLastError();  // a query that failed leaves the other forms in use
+}
+
+// the sums of the CTAs with cells, the iterates (two parities), and 16 words the test hook writes to
+size_t couple_flag_bytes(int ctas) { return 2 * (size_t)(ctas - 1) * NVC * sizeof(Words) + 48 * 8; }
+
+template <typename T>
+void launch_couple_flag(const Geo& g, const Slots<T>& S, Ctrl* ctrl, Dof* it, const T* kref, const Moments* mom,
+                        void* words, T* boxstore, int nbox, int di, cudaStream_t st) {
+  launch_coop(k_couple_flag<T>, dim3((unsigned)g.flag_ctas), dim3((unsigned)g.flag_threads), 0, st, g, S, ctrl, it, kref,
+              mom, words, boxstore, nbox, di);
+}
+
+template void launch_couple_flag<float>(const Geo&, const Slots<float>&, Ctrl*, Dof*, const float*, const Moments*,
+                                        void*, float*, int, int, cudaStream_t);
+template void launch_couple_flag<double>(const Geo&, const Slots<double>&, Ctrl*, Dof*, const double*, const Moments*,
+                                         void*, double*, int, int, cudaStream_t);
+
+}  // namespace lks

@@ -163,6 +163,7 @@ struct Geo {
   int hb[3];      // box half extent (ceil of the body's half extent)
   int margin;     // cells of drift allowed within one step
   long long box_cells;
+  int flag_ctas, flag_threads;  // 2D: shape of the flag-exchange coupling kernel (0: another form runs)
   int coop_fwd, coop_adj;  // CTAs of the cooperative coupling kernels (0: the per-iteration kernels)
 };
 

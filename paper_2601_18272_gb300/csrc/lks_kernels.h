@@ -119,6 +119,16 @@ void launch_adj_coop(const Geo& g, Ctrl* ctrl, const Dof* it, const T* kref, con
 // as the device holds at once (0 if the kernel cannot be resident); sets g->coop_fwd, g->coop_adj.
 void setup_coop(Geo* g, bool fp64);
 
+// The same in 2D with the sums exchanged through flagged words (lks_couple2d.cu): g.flag_ctas CTAs of
+// g.flag_threads threads, set by setup_couple_flag (0 if it does not apply). words:
+// couple_flag_bytes(CTAs) bytes (at most kFlagMaxCtas CTAs), zeroed before a march (the words carry the iteration's number in the run).
+constexpr int kFlagMaxCtas = 1024;
+void setup_couple_flag(Geo* g, bool fp64);
+size_t couple_flag_bytes(int ctas);
+template <typename T>
+void launch_couple_flag(const Geo& g, const Slots<T>& S, Ctrl* ctrl, Dof* it, const T* kref, const Moments* mom,
+                        void* words, T* boxstore, int nbox, int di, cudaStream_t st);
+
 // Recompute: Brinkman update with the stored iterate s^(K-1); writes u(t) and the box store of u*.
 template <typename T>
 void launch_apply(const Geo& g, const Slots<T>& S, const Ctrl* ctrl, const Dof* it, const T* kref, T* boxstore,
