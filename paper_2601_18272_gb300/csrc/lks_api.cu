@@ -1079,7 +1079,7 @@ int lks_forward(lks_handle* h, const double* gamma_dev, double* J_host, void* st
   Launcher L0{h, st, false};
   CK(cudaMemsetAsync((char*)h->ctrl + offsetof(Ctrl, prep_status), 0, sizeof(int), st));
   // design chain gamma -> gamma-bar (Sec. 3.2, 4.2), then kappa^ref of gamma-bar
-  L0.n("prep", 2, [&](cudaStream_t s) { launch_design_chain(g, h->gamma, h->cg1, h->cgtil, h->cgbar, h->cW, s); });
+  L0.n("prep", g.cyc > 1 ? 2 : 1, [&](cudaStream_t s) { launch_design_chain(g, h->gamma, h->cg1, h->cgtil, h->cgbar, h->cW, s); });
   if (h->prec == LKS_FP64)
     L0("prep", [&](cudaStream_t s) { launch_prep<double>(g, h->cgbar, h->P.kappa_max, h->P.q, (double*)h->kref, h->mom, h->partials, h->ctrl, s); });
   else
@@ -1202,9 +1202,8 @@ int lks_sensitivity(lks_handle* h, double* out, void* stream) {
   if (!h->adj_done) return LKS_ERR_ORDER;
   cudaStream_t st = (cudaStream_t)stream;
   // dJ/dgamma-bar at gamma-bar, then the transpose of the design chain
-  launch_sensitivity(h->g, h->cgbar, h->dkref, h->P.kappa_max, h->P.q, h->dv, st);
-  launch_design_chain_T(h->g, h->cgtil, h->cW, h->dv, h->dtmp, out, st);
-  h->launches += 4;
+  h->launches += launch_sensitivity(h->g, h->cgbar, h->dkref, h->P.kappa_max, h->P.q, h->cgtil, h->cW, h->dv, h->dtmp,
+                                    out, st);
   CK(cudaGetLastError());
   return LKS_OK;
 }
@@ -1243,20 +1242,17 @@ int lks_constraint(lks_handle* h, const double* gamma_dev, double* G_host, doubl
   if (!(h->P.v_min > 0.0)) return LKS_ERR_ARG;
   cudaStream_t st = (cudaStream_t)stream;
   const Geo& g = h->g;
-  launch_design_chain(g, gamma_dev, h->kg1, h->kgtil, h->kgbar, h->kW, st);
+  // everything is enqueued before the one wait: the gradient's scale needs the point count only,
+  // which it reads on the device
+  h->launches += launch_design_chain(g, gamma_dev, h->kg1, h->kgtil, h->kgbar, h->kW, st) + 1;
   launch_volume(g, h->kgbar, h->vol, st);
+  if (dGdgamma_dev)
+    h->launches += launch_volume_gradient(g, h->vol, h->P.v_min, h->kgtil, h->kW, h->dv, h->dtmp, dGdgamma_dev, st);
+  CK(cudaGetLastError());
   double vol[2];
   CK(cudaMemcpyAsync(vol, h->vol, sizeof(vol), cudaMemcpyDeviceToHost, st));
   CK(cudaStreamSynchronize(st));
-  const double scale = 1.0 / (h->P.v_min * vol[1]);
-  *G_host = vol[0] * scale - 1.0;
-  h->launches += 3;
-  if (dGdgamma_dev) {
-    launch_fill_domain(g, scale, h->dv, st);
-    launch_design_chain_T(g, h->kgtil, h->kW, h->dv, h->dtmp, dGdgamma_dev, st);
-    h->launches += 4;
-  }
-  CK(cudaGetLastError());
+  *G_host = vol[0] * (1.0 / (h->P.v_min * vol[1])) - 1.0;
   return LKS_OK;
 }
 

@@ -960,14 +960,6 @@ __global__ void k_adj_init(Geo g, Ctrl* ctrl, const Dof* it, int nt, const doubl
   lam_store(ctrl, nF, nT);
 }
 
-__global__ void k_sensitivity(int nd, const double* __restrict__ gamma, const double* __restrict__ dkref, double kmax,
-                              double q, double* __restrict__ out) {
-  const int m = blockIdx.x * blockDim.x + threadIdx.x;
-  if (m >= nd) return;
-  const double den = (1.0 - gamma[m]) + q;
-  out[m] = dkref[m] * kmax * q * (1.0 + q) / (den * den);
-}
-
 template <typename T>
 __global__ void k_ckpt_pack(Geo g, Slots<T> S, T* ckpt, long long cstride, int every, const Ctrl* ctrl, int di) {
   const int tn = ctrl->t0 + di;
@@ -1401,11 +1393,6 @@ void launch_adj_init(const Geo& g, Ctrl* ctrl, const Dof* it, int nt, const doub
                      const double* term_s, double* dkref, int nd, cudaStream_t st) {
   cudaMemsetAsync(dkref, 0, sizeof(double) * (size_t)nd, st);
   launch(k_adj_init, 1, 1, 0, st, g, ctrl, it, nt, objw, seed, term_s);
-}
-
-void launch_sensitivity(const Geo& g, const double* gamma, const double* dkref, double kappa_max, double q,
-                        double* out, cudaStream_t st) {
-  launch(k_sensitivity, (g.ND + 255) / 256, 256, 0, st, g.ND, gamma, dkref, kappa_max, q, out);
 }
 
 template <typename T>

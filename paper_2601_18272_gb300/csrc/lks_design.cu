@@ -14,6 +14,8 @@
 // Transpose: v3 = dJ/dgbar -> v2 = v3 dgbar/dgtil -> v1_j = sum_i w_ij v2_i / W_i (the weights are
 // symmetric, so this is the same gather as the filter applied to v2 / W) -> out_m = sum of v1 over
 // m's orbit when m is its own representative, else 0. Every output is one thread's fixed-order sum.
+#include <climits>
+
 #include "lks_kernels.h"
 
 namespace lks {
@@ -67,30 +69,92 @@ __global__ void __launch_bounds__(kDB) k_expand(Geo g, const double* __restrict_
   g1[m] = gamma[rep];
 }
 
-// Sum of w_ij src_j over the filter disc of i (points of the design domain); W = sum of w_ij.
-__device__ __forceinline__ void filter_sum(const Geo& g, const double* __restrict__ src, const int* i, double* acc,
-                                           double* W) {
+// Filter weights by squared distance, (R - sqrt(d2)) / R up to R (beyond: -1), and the weights' sum
+// over a whole disc, made once per block: the square root and the division took most of the
+// filter's FP64 instructions (each costs a warp 64 cycles) when every pair of points computed its own
+// (lks_constraint with its gradient on a 256^2 design, R = 3, with projection and cyclic order 4:
+// 350 -> 111 us, with the volume's sum in a cluster and one wait at the end).
+// Radii whose table would not fit keep that form.
+constexpr int kTab = 2048;
+// Table entries for radius R: every squared distance up to R^2, one more for its rounding.
+__device__ __forceinline__ int tab_size(double R) { return R < 1000.0 ? (int)floor(R * R) + 2 : INT_MAX; }
+struct FilterTab {
+  double w[kTab];
+  double full;  // sum over the whole disc, in the order of filter_sum
+};
+__device__ __forceinline__ double filter_weight(double R, int d2) {
+  const double dist = sqrt((double)d2);
+  return dist > R ? -1.0 : (R - dist) / R;
+}
+// All threads of the block call it; a block barrier follows it.
+__device__ __forceinline__ void make_table(const Geo& g, FilterTab& tab) {
+  const int rr = (int)floor(g.frad), n = tab_size(g.frad);
+  if (g.frad > 0.0 && n <= kTab) {
+    for (int d2 = threadIdx.x; d2 < n; d2 += kDB) tab.w[d2] = filter_weight(g.frad, d2);
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      double w = 0.0;
+      const int ez = (g.dim == 3) ? rr : 0;
+      for (int dz = -ez; dz <= ez; ++dz)
+        for (int dy = -rr; dy <= rr; ++dy)
+          for (int dx = -rr; dx <= rr; ++dx) {
+            const int d2 = dx * dx + dy * dy + dz * dz;
+            if (d2 < n && tab.w[d2] >= 0.0) w += tab.w[d2];
+          }
+      tab.full = w;
+    }
+  }
+}
+
+// Sum of w_ij src_j over the filter disc of i (points of the design domain).
+template <bool NEED_W>
+__device__ __forceinline__ double filter_sum(const Geo& g, const FilterTab& tab, const double* __restrict__ src,
+                                             const int* i, double* W) {
   const double R = g.frad;
-  const int rr = (int)floor(R);
+  const int rr = (int)floor(R), n = tab_size(R);
   const int ez = (g.dim == 3) ? rr : 0;
+  const bool ball = g.rad4 != INT_MAX, table = n <= kTab;
   double a = 0.0, w = 0.0;
-  for (int dz = -ez; dz <= ez; ++dz)
-    for (int dy = -rr; dy <= rr; ++dy)
-      for (int dx = -rr; dx <= rr; ++dx) {
-        const int j[3] = {i[0] + dx, i[1] + dy, i[2] + dz};
-        if (j[0] < 0 || j[0] >= g.nd[0] || j[1] < 0 || j[1] >= g.nd[1] || j[2] < 0 || j[2] >= g.nd[2]) continue;
-        const double dist = sqrt((double)(dx * dx + dy * dy + dz * dz));
-        if (dist > R || !in_domain(g, j)) continue;
-        const double wij = (R - dist) / R;
-        a += wij * src[design_index(g, j)];
-        w += wij;
+  const int x0 = max(-rr, -i[0]), x1 = min(rr, g.nd[0] - 1 - i[0]);
+  const int y0 = max(-rr, -i[1]), y1 = min(rr, g.nd[1] - 1 - i[1]);
+  const int z0 = max(-ez, -i[2]), z1 = min(ez, g.nd[2] - 1 - i[2]);
+  const bool whole = !ball && table && x0 == -rr && x1 == rr && y0 == -rr && y1 == rr && z0 == -ez && z1 == ez;
+  for (int dz = z0; dz <= z1; ++dz)
+    for (int dy = y0; dy <= y1; ++dy) {
+      const int r2 = dy * dy + dz * dz;
+      if (r2 >= n) continue;  // beyond R
+      const double* row = src + i[0] + (long long)g.nd[0] * (i[1] + dy + (long long)g.nd[1] * (i[2] + dz));
+      for (int dx = x0; dx <= x1; ++dx) {
+        const int d2 = dx * dx + r2;
+        const double wij = table ? (d2 < n ? tab.w[d2] : -1.0) : filter_weight(R, d2);
+        if (wij < 0.0) continue;
+        if (ball) {
+          const int j[3] = {i[0] + dx, i[1] + dy, i[2] + dz};
+          if (!in_domain(g, j)) continue;
+        }
+        a += wij * row[dx];
+        if (NEED_W && !whole) w += wij;
       }
-  *acc = a;
-  *W = w;
+    }
+  if (NEED_W) *W = whole ? tab.full : w;
+  return a;
+}
+
+// tanh(beta eta) and the projection's denominator, the same for every point: once per block.
+__device__ __forceinline__ void make_projection(const Geo& g, double (&pr)[2]) {
+  if (g.pbeta > 0.0) {
+    if (threadIdx.x == 32) pr[0] = tanh(g.pbeta * g.peta);
+    if (threadIdx.x == 64) pr[1] = tanh(g.pbeta * (1.0 - g.peta));
+  }
 }
 
 __global__ void __launch_bounds__(kDB) k_filter_project(Geo g, const double* __restrict__ g1, double* __restrict__ gtil,
                                                         double* __restrict__ gbar, double* __restrict__ W) {
+  __shared__ FilterTab tab;
+  __shared__ double pr[2];
+  make_projection(g, pr);
+  make_table(g, tab);
+  __syncthreads();
   const int m = blockIdx.x * kDB + threadIdx.x;
   if (m >= g.ND) return;
   int i[3];
@@ -101,41 +165,29 @@ __global__ void __launch_bounds__(kDB) k_filter_project(Geo g, const double* __r
     return;
   }
   double gt = g1[m], w = 1.0;
-  if (g.frad > 0.0) {
-    double a;
-    filter_sum(g, g1, i, &a, &w);
-    gt = a / w;
-  }
+  if (g.frad > 0.0) gt = filter_sum<true>(g, tab, g1, i, &w) / w;
   gtil[m] = gt;
   W[m] = w;
-  if (g.pbeta > 0.0) {
-    const double te = tanh(g.pbeta * g.peta);
-    gbar[m] = (te + tanh(g.pbeta * (gt - g.peta))) / (te + tanh(g.pbeta * (1.0 - g.peta)));
-  } else {
+  if (g.pbeta > 0.0)
+    gbar[m] = (pr[0] + tanh(g.pbeta * (gt - g.peta))) / (pr[0] + pr[1]);
+  else
     gbar[m] = gt;
-  }
 }
 
-// v <- v dgbar/dgtil / W (in place), zero outside the domain
-__global__ void __launch_bounds__(kDB) k_project_T(Geo g, const double* __restrict__ gtil, const double* __restrict__ W,
-                                                   double* __restrict__ v) {
-  const int m = blockIdx.x * kDB + threadIdx.x;
-  if (m >= g.ND) return;
-  int i[3];
-  design_ijk(g, m, i);
-  if (!in_domain(g, i)) {
-    v[m] = 0.0;
-    return;
-  }
-  double d = 1.0;
-  if (g.pbeta > 0.0) {
-    const double th = tanh(g.pbeta * (gtil[m] - g.peta));
-    d = g.pbeta * (1.0 - th * th) / (tanh(g.pbeta * g.peta) + tanh(g.pbeta * (1.0 - g.peta)));
-  }
-  v[m] = v[m] * d / W[m];
-}
-
-__global__ void __launch_bounds__(kDB) k_filter_T(Geo g, const double* __restrict__ v, double* __restrict__ out) {
+// out = dJ/dgbar dgbar/dgtil / W, zero outside the domain, with dJ/dgbar = dJ/dkappa^ref times
+// dkappa^ref/dgbar (Eq. brinkman_coefficient), or a constant over the domain (the volume's gradient,
+// 1 / (v_min * vol[1])).
+struct GradIn {
+  const double *gbar, *dkref;
+  double kmax, q;
+  const double* vol;  // dkref null
+  double v_min;
+};
+__global__ void __launch_bounds__(kDB) k_project_T(Geo g, GradIn in, const double* __restrict__ gtil,
+                                                   const double* __restrict__ W, double* __restrict__ out) {
+  __shared__ double pr[2];
+  make_projection(g, pr);
+  __syncthreads();
   const int m = blockIdx.x * kDB + threadIdx.x;
   if (m >= g.ND) return;
   int i[3];
@@ -144,13 +196,30 @@ __global__ void __launch_bounds__(kDB) k_filter_T(Geo g, const double* __restric
     out[m] = 0.0;
     return;
   }
-  if (g.frad > 0.0) {
-    double a, w;
-    filter_sum(g, v, i, &a, &w);
-    out[m] = a;
+  double v;
+  if (in.dkref) {
+    const double den = (1.0 - in.gbar[m]) + in.q;
+    v = in.dkref[m] * in.kmax * in.q * (1.0 + in.q) / (den * den);
   } else {
-    out[m] = v[m];
+    v = 1.0 / (in.v_min * in.vol[1]);
   }
+  double d = 1.0;
+  if (g.pbeta > 0.0) {
+    const double th = tanh(g.pbeta * (gtil[m] - g.peta));
+    d = g.pbeta * (1.0 - th * th) / (pr[0] + pr[1]);
+  }
+  out[m] = g.frad > 0.0 ? v * d / W[m] : v * d;
+}
+
+__global__ void __launch_bounds__(kDB) k_filter_T(Geo g, const double* __restrict__ v, double* __restrict__ out) {
+  __shared__ FilterTab tab;
+  make_table(g, tab);
+  __syncthreads();
+  const int m = blockIdx.x * kDB + threadIdx.x;
+  if (m >= g.ND) return;
+  int i[3];
+  design_ijk(g, m, i);
+  out[m] = in_domain(g, i) ? filter_sum<false>(g, tab, v, i, nullptr) : 0.0;
 }
 
 __global__ void __launch_bounds__(kDB) k_orbit_sum(Geo g, const double* __restrict__ v, double* __restrict__ out) {
@@ -169,58 +238,98 @@ __global__ void __launch_bounds__(kDB) k_orbit_sum(Geo g, const double* __restri
   out[m] = rep ? s : 0.0;
 }
 
-// One CTA: sum of gbar over the design domain in a fixed order, and the domain's point count.
-__global__ void __launch_bounds__(1024) k_volume(Geo g, const double* __restrict__ gbar, double* __restrict__ out) {
-  __shared__ double red[32 * 2];
+// Sum of gbar over the design domain in a fixed order, and the domain's point count: one cluster of
+// eight CTAs, whose sums the first one reads from the others' shared memory (one CTA alone was bound
+// by the latency of its loads).
+constexpr int kVolCtas = 8;
+__global__ void __cluster_dims__(kVolCtas, 1, 1) __launch_bounds__(1024) k_volume(Geo g, const double* __restrict__ gbar,
+                                                                                  double* __restrict__ out) {
+  __shared__ double red[32 * 2], mine[2];
+  const bool ball = g.rad4 != INT_MAX;
   double v[2] = {0.0, 0.0};
-  for (int m = threadIdx.x; m < g.ND; m += blockDim.x) {
-    int i[3];
-    design_ijk(g, m, i);
-    if (in_domain(g, i)) {
-      v[0] += gbar[m];
-      v[1] += 1.0;
+  const int stride = 1024 * kVolCtas;
+  for (int m = blockIdx.x * 1024 + threadIdx.x; m < g.ND; m += 4 * stride) {
+    double x[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) x[j] = m + j * stride < g.ND ? gbar[m + j * stride] : 0.0;
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      if (m + j * stride >= g.ND) continue;
+      if (ball) {
+        int i[3];
+        design_ijk(g, m + j * stride, i);
+        if (!in_domain(g, i)) continue;
+      }
+      v[0] += x[j];
+      if (ball) v[1] += 1.0;
     }
   }
   block_sum<2>(v, red);
   if (threadIdx.x == 0) {
-    out[0] = v[0];
-    out[1] = v[1];
+    mine[0] = v[0];
+    mine[1] = v[1];
   }
-}
-
-__global__ void __launch_bounds__(kDB) k_fill_domain(Geo g, double value, double* __restrict__ out) {
-  const int m = blockIdx.x * kDB + threadIdx.x;
-  if (m >= g.ND) return;
-  int i[3];
-  design_ijk(g, m, i);
-  out[m] = in_domain(g, i) ? value : 0.0;
+  auto cluster_sync = [] {
+    asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+  };
+  cluster_sync();
+  if (blockIdx.x == 0 && threadIdx.x < 2) {
+    const unsigned at = (unsigned)__cvta_generic_to_shared(&mine[threadIdx.x]);
+    double s = 0.0;
+    for (int c = 0; c < kVolCtas; ++c) {
+      unsigned ra;
+      double x;
+      asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(ra) : "r"(at), "r"(c));
+      asm volatile("ld.shared::cluster.f64 %0, [%1];" : "=d"(x) : "r"(ra) : "memory");
+      s += x;
+    }
+    out[threadIdx.x] = threadIdx.x == 1 && !ball ? (double)g.ND : s;
+  }
+  cluster_sync();  // no CTA leaves before its sums are read
 }
 
 inline unsigned nblk(const Geo& g) { return (unsigned)((g.ND + kDB - 1) / kDB); }
 
 }  // namespace
 
-bool design_chain_active(const Geo& g) { return g.cyc > 1 || g.frad > 0.0 || g.pbeta > 0.0; }
-
-void launch_design_chain(const Geo& g, const double* gamma, double* g1, double* gtil, double* gbar, double* W,
-                         cudaStream_t st) {
-  launch(k_expand, nblk(g), kDB, 0, st, g, gamma, g1);
-  launch(k_filter_project, nblk(g), kDB, 0, st, g, (const double*)g1, gtil, gbar, W);
+// The expansion is a copy without cyclic order: the filter then reads gamma itself.
+int launch_design_chain(const Geo& g, const double* gamma, double* g1, double* gtil, double* gbar, double* W,
+                        cudaStream_t st) {
+  const double* src = gamma;
+  if (g.cyc > 1) {
+    launch(k_expand, nblk(g), kDB, 0, st, g, gamma, g1);
+    src = g1;
+  }
+  launch(k_filter_project, nblk(g), kDB, 0, st, g, src, gtil, gbar, W);
+  return g.cyc > 1 ? 2 : 1;
 }
 
-void launch_design_chain_T(const Geo& g, const double* gtil, const double* W, double* v, double* tmp, double* out,
-                           cudaStream_t st) {
-  launch(k_project_T, nblk(g), kDB, 0, st, g, gtil, W, v);
-  launch(k_filter_T, nblk(g), kDB, 0, st, g, (const double*)v, tmp);
-  launch(k_orbit_sum, nblk(g), kDB, 0, st, g, (const double*)tmp, out);
+namespace {
+// Transpose of the chain: projection, filter and orbit sum, without the steps that are off.
+int chain_T(const Geo& g, const GradIn& in, const double* gtil, const double* W, double* v, double* tmp, double* out,
+            cudaStream_t st) {
+  const bool filter = g.frad > 0.0, cyclic = g.cyc > 1;
+  double* o1 = filter || cyclic ? v : out;
+  launch(k_project_T, nblk(g), kDB, 0, st, g, in, gtil, W, o1);
+  double* o2 = cyclic ? tmp : out;
+  if (filter) launch(k_filter_T, nblk(g), kDB, 0, st, g, (const double*)o1, o2);
+  if (cyclic) launch(k_orbit_sum, nblk(g), kDB, 0, st, g, (const double*)(filter ? o2 : o1), out);
+  return 1 + (filter ? 1 : 0) + (cyclic ? 1 : 0);
+}
+}  // namespace
+
+int launch_sensitivity(const Geo& g, const double* gbar, const double* dkref, double kappa_max, double q,
+                       const double* gtil, const double* W, double* v, double* tmp, double* out, cudaStream_t st) {
+  return chain_T(g, GradIn{gbar, dkref, kappa_max, q, nullptr, 0.0}, gtil, W, v, tmp, out, st);
 }
 
 void launch_volume(const Geo& g, const double* gbar, double* out2, cudaStream_t st) {
-  launch(k_volume, 1, 1024, 0, st, g, gbar, out2);
+  launch(k_volume, kVolCtas, 1024, 0, st, g, gbar, out2);
 }
 
-void launch_fill_domain(const Geo& g, double value, double* out, cudaStream_t st) {
-  launch(k_fill_domain, nblk(g), kDB, 0, st, g, value, out);
+int launch_volume_gradient(const Geo& g, const double* vol, double v_min, const double* gtil, const double* W, double* v,
+                           double* tmp, double* out, cudaStream_t st) {
+  return chain_T(g, GradIn{nullptr, nullptr, 0.0, 0.0, vol, v_min}, gtil, W, v, tmp, out, st);
 }
 
 }  // namespace lks

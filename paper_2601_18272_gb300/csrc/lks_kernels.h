@@ -179,17 +179,18 @@ template <typename T>
 void launch_support_sets(const Geo& g, const Dof& s, const T* kref, long long* out, cudaStream_t st);
 
 // Design chain (cyclic expansion, density filter, Heaviside projection) gamma -> gbar, keeping the
-// filtered field gtil and the filter normaliser W for the transpose; active unless every step is off.
-bool design_chain_active(const Geo& g);
-void launch_design_chain(const Geo& g, const double* gamma, double* g1, double* gtil, double* gbar, double* W,
-                         cudaStream_t st);
-// Transpose: out = (dgbar/dgamma)^T v; v and tmp are overwritten.
-void launch_design_chain_T(const Geo& g, const double* gtil, const double* W, double* v, double* tmp, double* out,
-                           cudaStream_t st);
+// filtered field gtil and the filter normaliser W for the transpose. Returns the kernels launched.
+int launch_design_chain(const Geo& g, const double* gamma, double* g1, double* gtil, double* gbar, double* W,
+                        cudaStream_t st);
+// dJ/dgamma: dJ/dgamma-bar = dJ/dkappa^ref * dkappa^ref/dgamma-bar at gamma-bar (Eq.
+// brinkman_coefficient) through the transpose of the chain; v and tmp are scratch.
+int launch_sensitivity(const Geo& g, const double* gbar, const double* dkref, double kappa_max, double q,
+                       const double* gtil, const double* W, double* v, double* tmp, double* out, cudaStream_t st);
 // out2[0] = sum of gbar over the design domain, out2[1] = the domain's point count.
 void launch_volume(const Geo& g, const double* gbar, double* out2, cudaStream_t st);
-// out = value on the design domain, 0 elsewhere.
-void launch_fill_domain(const Geo& g, double value, double* out, cudaStream_t st);
+// The gradient of out2[0] / (v_min out2[1]) through the transpose of the chain.
+int launch_volume_gradient(const Geo& g, const double* vol, double v_min, const double* gtil, const double* W, double* v,
+                           double* tmp, double* out, cudaStream_t st);
 
 // Initial state (double) -> slot(0); s0 -> it row 0; ctrl reset for a forward (t0 = 1, base 0).
 template <typename T>
@@ -206,10 +207,6 @@ void launch_adj_init(const Geo& g, Ctrl* ctrl, const Dof* it, int nt, const doub
 // A state slot (T) -> p0 [N], u0 [dim][N] as doubles.
 template <typename T>
 void launch_state_to_double(const Geo& g, const T* src, double* p0, double* u0, cudaStream_t st);
-
-// dJ/dgamma-bar = dJ/dkappa^ref * dkappa^ref/dgamma-bar at gamma-bar (Eq. brinkman_coefficient).
-void launch_sensitivity(const Geo& g, const double* gbar, const double* dkref, double kappa_max, double q,
-                        double* out, cudaStream_t st);
 
 // Reduced-precision checkpoint (FP32 fields) of the state at step ctrl->t0 + di into checkpoint
 // c = step / every: per-plane range keys[c][plane][2] and q[c][plane][N] in BF16 or FP16.
