@@ -63,6 +63,15 @@ template <typename T>
 void launch_stencil_adj(const Geo& g, const Slots<T>& S, T* Lb, long long lstride, const Ctrl* ctrl, int di,
                         cudaStream_t st);
 
+// 2D tiled forms for small grids (lks_stencil_tile.cu), called by the launchers above where they pay
+// against strips of the given number of rows.
+bool stencil_tile_pays(const Geo& g, int rows, bool fp64, bool transpose);
+template <typename T>
+void launch_stencil_tile_fwd(const Geo& g, const Slots<T>& S, const Ctrl* ctrl, int di, cudaStream_t st);
+template <typename T>
+void launch_stencil_tile_adj(const Geo& g, const Slots<T>& S, T* Lb, long long lstride, const Ctrl* ctrl, int di,
+                             cudaStream_t st);
+
 // 3D forms (D3Q15), called by the launchers above; prepare_stencil3d sets their shared-memory
 // attributes and must run once before the first launch (outside stream capture).
 template <typename T>

@@ -850,6 +850,7 @@ template <typename T>
 void launch_stencil_fwd(const Geo& g, const Slots<T>& S, const Ctrl* ctrl, int di, cudaStream_t st) {
   if (g.dim == 2) {
     const StripPlan sp = plan_strips(g);
+    if (stencil_tile_pays(g, g.n[1] / sp.nstrip, sizeof(T) == 8, false)) return launch_stencil_tile_fwd<T>(g, S, ctrl, di, st);
     const int warps = sp.ntx * sp.nstrip;
     const size_t smem = Ring<T>::bytes(3);
     if (vec_ok(g))
@@ -866,6 +867,7 @@ void launch_stencil_adj(const Geo& g, const Slots<T>& S, T* Lb, long long lstrid
                         cudaStream_t st) {
   if (g.dim == 2) {
     const StripPlan sp = plan_strips(g);
+    if (stencil_tile_pays(g, g.n[1] / sp.nstrip, sizeof(T) == 8, true)) return launch_stencil_tile_adj<T>(g, S, Lb, lstride, ctrl, di, st);
     const int warps = sp.ntx * sp.nstrip;
     const size_t smem = Ring<T>::bytes(5);
     if (vec_ok(g))
