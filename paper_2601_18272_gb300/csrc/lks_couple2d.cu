@@ -3,21 +3,10 @@
 // with one launch per iteration and with grid barriers).
 //
 // An iteration is short (a gather over the box's cells, three sums, the EOM), so its time is the
-// latency of the sums' way through the chip. CTA 0 has no cells: the others publish their three sums
-// to it, it adds them up, runs the EOM and publishes the iterate. Values travel as 64-bit words that
-// carry the iteration's number beside 32 bits of payload, so the arrival of the data is the
-// synchronisation: one trip through L2 each way, and every waiting CTA polls one or two lines. (A form
-// in which every CTA polled the words of all others and ran the EOM itself needed one trip only, but
-// took 4.3 us an iteration without gather and EOM on 148 SMs: 57 lines polled by all of them.)
-// A word's number tells it from the one two iterations earlier in the same place (two places by the
-// iteration's parity): sums of iteration e + 2 are published after the iterate of e + 1 was read,
-// which CTA 0 publishes after it has read the sums of e; and likewise the other way. All sums are
-// taken in a fixed order (warps, CTA, then 32 lanes over the CTAs), so results do not vary between
-// runs.
+// latency of the sums' way through the chip (lks_flag.cuh: how they travel).
 //
 // Warps are dealt over the box round robin, so the design-free corners of a rotating body's box are
-// shared evenly between the CTAs. The launch is cooperative (all CTAs resident); waits are bounded by
-// one second as those of the grid barriers.
+// shared evenly between the CTAs. The launch is cooperative (all CTAs resident).
 //
 // What bounds it: the gather's slowest warps and two trips through L2 per iteration. Forward march
 // measured on GB300, N_itr launches (or grid barriers) per step -> this kernel, us per step: 512x256
@@ -25,8 +14,7 @@
 // FP64 600x100, 20^2 500 -> 67.
 #include <climits>
 
-#include "lks_body_common.cuh"
-#include "lks_wait.cuh"
+#include "lks_flag.cuh"
 
 namespace lks {
 
@@ -199,326 +187,6 @@ __device__ __forceinline__ void gather2d(const Geo& g, const double* __restrict_
   to_pivot(xb, xc, sb, sc, kb, kc, o);
 }
 
-// One value as two 64-bit words (number << 32 | payload) and back.
-struct Words {
-  unsigned long long a, b;
-};
-__device__ __forceinline__ void st_words(Words* p, Words w) {
-  asm volatile("st.relaxed.gpu.global.v2.u64 [%0], {%1, %2};" ::"l"(p), "l"(w.a), "l"(w.b) : "memory");
-}
-__device__ __forceinline__ Words ld_words(const Words* p) {
-  Words w;
-  asm volatile("ld.relaxed.gpu.global.v2.u64 {%0, %1}, [%2];" : "=l"(w.a), "=l"(w.b) : "l"(p) : "memory");
-  return w;
-}
-__device__ __forceinline__ Words pack(unsigned e, unsigned x, unsigned y) {
-  return Words{((unsigned long long)e << 32) | x, ((unsigned long long)e << 32) | y};
-}
-
-// The value of a whole warp's lanes (fixed order), and a CTA's or the grid's sum of one component.
-struct Df {
-  float hi, lo;
-  __device__ __forceinline__ void zero() { hi = lo = 0.0f; }
-  __device__ __forceinline__ void set(float v) { hi = v, lo = 0.0f; }
-  __device__ __forceinline__ void add(const Df& o) { df_add(hi, lo, o.hi, o.lo); }
-  __device__ __forceinline__ Df from_xor(int off) const {
-    return Df{__shfl_xor_sync(0xffffffffu, hi, off), __shfl_xor_sync(0xffffffffu, lo, off)};
-  }
-  __device__ __forceinline__ Words words(unsigned e) const { return pack(e, __float_as_uint(hi), __float_as_uint(lo)); }
-  __device__ __forceinline__ void read(const Words& w) {
-    hi = __uint_as_float((unsigned)w.a);
-    lo = __uint_as_float((unsigned)w.b);
-  }
-  __device__ __forceinline__ double value() const { return (double)hi + (double)lo; }
-};
-struct Dd {
-  double v;
-  __device__ __forceinline__ void zero() { v = 0.0; }
-  __device__ __forceinline__ void set(double x) { v = x; }
-  __device__ __forceinline__ void add(const Dd& o) { v += o.v; }
-  __device__ __forceinline__ Dd from_xor(int off) const { return Dd{__shfl_xor_sync(0xffffffffu, v, off)}; }
-  __device__ __forceinline__ Words words(unsigned e) const {
-    const unsigned long long b = (unsigned long long)__double_as_longlong(v);
-    return pack(e, (unsigned)b, (unsigned)(b >> 32));
-  }
-  __device__ __forceinline__ void read(const Words& w) {
-    v = __longlong_as_double((long long)((w.a & 0xffffffffull) | (w.b << 32)));
-  }
-  __device__ __forceinline__ double value() const { return v; }
-};
-template <typename T>
-struct SumOf;
-template <>
-struct SumOf<float> {
-  using type = Df;
-};
-template <>
-struct SumOf<double> {
-  using type = Dd;
-};
-template <int STRIDE, typename V>
-__device__ __forceinline__ void warp_total(V& v) {
-#pragma unroll
-  for (int off = 16; off >= STRIDE; off >>= 1) v.add(v.from_xor(off));
-}
-
-// EOM of an iteration, one component per warp (0, 1: an axis; 2: the rotation), in FP64. Every FP64
-// instruction of a warp costs 64 cycles, dependent or not, so prepare (while the other warps gather)
-// does what does not need the sums, and finish spends about a dozen. The cosine of the step's rotation
-// is taken on the even lanes and its sine on the odd ones by the same instructions with their own
-// coefficients. Range tests are made on the exponent in integers. All lanes of the warp call both.
-struct EomPart {
-  double c0, im, q0, f0, x0, y0;  // v = s im + c0; q = q0 + v; f0 = frac(q0); cos/sin(t-1) by lane
-  int xi0;
-  bool fr;
-  __device__ __forceinline__ void prepare(const Geo& g, const Moments& mom, const Dof& s0, const Dof& sk, int comp,
-                                          int lane) {
-    const double cs = sk.cs, sn = sk.sn, om = sk.s[7];
-    const double kx = cs * mom.K1[0] - sn * mom.K1[1], ky = sn * mom.K1[0] + cs * mom.K1[1];
-    double pre, v0;
-    if (comp < 2) {
-      pre = mom.K0 * sk.s[3 + comp] + om * (comp == 0 ? -ky : kx);
-      fr = (g.dof_mask & (1 << comp)) != 0;
-      v0 = s0.s[3 + comp];
-      im = g.inv_mass;
-      q0 = s0.s[comp];
-      const double fl = floor(q0);
-      xi0 = (int)fl;
-      f0 = q0 - fl;
-    } else {
-      pre = (kx * sk.s[4] - ky * sk.s[3]) + om * mom.K2p;
-      fr = (g.dof_mask & DOF_ROT) != 0;
-      v0 = s0.s[7];
-      im = g.inv_inertia;
-      q0 = s0.s[6];
-      x0 = (lane & 1) ? s0.sn : s0.cs;  // cos' = cs c - sn s, sin' = sn c + cs s
-      y0 = (lane & 1) ? s0.cs : -s0.sn;
-    }
-    c0 = fr ? v0 - pre * im : v0;
-    if (!fr) im = 0.0;
-  }
-  // s: the component's sum. Writes the iterate's entries to nx and publishes those the gather reads
-  // (see Pose); returns the status bits.
-  template <typename T>
-  __device__ __forceinline__ int finish(const Geo& g, double s, Dof* nx, unsigned long long* pose, unsigned e, int comp,
-                                        int lane) const;
-};
-
-// What the cells need of an iterate, and its words: FP32 per axis u^G, fraction and floor of x^G, then
-// cos, sin, omega (9 words); FP64 per axis u^G and x^G, then cos, sin, omega (14 words).
-template <typename T>
-struct Pose;
-template <>
-struct Pose<float> {
-  static constexpr int words = 9;
-  float cs, sn, om, ug[2], xf[2];
-  int xi[2];
-  __device__ __forceinline__ void set(const Dof& d) {
-    cs = d.csf, sn = d.snf, om = d.om;
-    for (int a = 0; a < 2; ++a) ug[a] = d.ug[a], xf[a] = d.xf[a], xi[a] = d.xi[a];
-  }
-  // word w of the iterate
-  __device__ __forceinline__ void put(int w, unsigned p, unsigned) {
-    const float f = __uint_as_float(p);
-    if (w < 6) {
-      const int a = w >= 3 ? 1 : 0, i = w - 3 * a;
-      if (i == 0) ug[a] = f;
-      if (i == 1) xf[a] = f;
-      if (i == 2) xi[a] = (int)p;
-    } else {
-      (w == 6 ? cs : w == 7 ? sn : om) = f;
-    }
-  }
-  __device__ __forceinline__ float rel(int a, int p) const { return (float)(p - xi[a]) - xf[a]; }
-};
-template <>
-struct Pose<double> {
-  static constexpr int words = 14;
-  double cs, sn, om, ug[2], x[2];
-  __device__ __forceinline__ void set(const Dof& d) {
-    cs = d.cs, sn = d.sn, om = d.s[7];
-    for (int a = 0; a < 2; ++a) ug[a] = d.s[3 + a], x[a] = d.s[a];
-  }
-  // the low word w (even) of the iterate, hi the next one
-  __device__ __forceinline__ void put(int w, unsigned p, unsigned hi) {
-    if (w & 1) return;
-    const double f = __hiloint2double((int)hi, (int)p);
-    if (w < 8) {
-      const int a = w >= 4 ? 1 : 0;
-      (w & 2 ? x[a] : ug[a]) = f;
-    } else {
-      (w == 8 ? cs : w == 10 ? sn : om) = f;
-    }
-  }
-  __device__ __forceinline__ double rel(int a, int p) const { return (double)p - x[a]; }
-};
-
-__device__ __forceinline__ void st_word(unsigned long long* p, unsigned e, unsigned payload) {
-  asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(((unsigned long long)e << 32) | payload) : "memory");
-}
-__device__ __forceinline__ unsigned long long ld_word(const unsigned long long* p) {
-  unsigned long long w;
-  asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(w) : "l"(p) : "memory");
-  return w;
-}
-
-template <typename T>
-__device__ __forceinline__ int EomPart::finish(const Geo& g, double s, Dof* nx, unsigned long long* pose, unsigned e,
-                                               int comp, int lane) const {
-  constexpr bool D64 = sizeof(T) == 8;
-  const double v = fma(s, im, c0);
-  const int hi = __double2hiint(v) & 0x7fffffff;
-  int st = 0;
-  if (hi >= 0x7ff00000 || (__double2hiint(s) & 0x7fffffff) >= 0x7ff00000) st = ST_NONFINITE;
-  if (comp < 2) {
-    const double q = fr ? q0 + v : q0;
-    if constexpr (D64) {
-      const double w = lane < 2 ? v : q;
-      if (lane < 4) st_word(pose + 4 * comp + lane, e, (unsigned)((lane & 1) ? __double2hiint(w) : __double2loint(w)));
-    }
-    if (hi >= 0x3ff00000 && fr && fabs(v) > (double)g.margin) st |= ST_BOX_OVERFLOW;
-    // floor and fraction of the position from those of t-1 (a crossing renews them)
-    double f = fr ? f0 + v : f0;
-    int xi = xi0;
-    const int hf = __double2hiint(f);
-    if (hf < 0 || hf >= 0x3ff00000) {
-      const double fl = floor(f);
-      xi += (int)fl;
-      f -= fl;
-    }
-    const float vf = (float)v, ff = (float)f;
-    if constexpr (!D64) {
-      const unsigned w = lane == 0 ? __float_as_uint(vf) : (lane == 1 ? __float_as_uint(ff) : (unsigned)xi);
-      if (lane < 3) st_word(pose + 3 * comp + lane, e, w);
-    }
-    if (lane == 0) {
-      nx->s[comp] = q;
-      nx->s[3 + comp] = v;
-      nx->xi[comp] = xi;
-      nx->xf[comp] = ff;
-      nx->ug[comp] = vf;
-    }
-    return st;
-  }
-  const bool sine = lane & 1;
-  const double x = fr ? v : 0.0;  // the step's rotation
-  const int hx = fr ? hi : 0;
-  double p;
-  if (hx > 0x3fd00000) {  // above 1/4
-    double sd, cd;
-    sincos(x, &sd, &cd);
-    p = sine ? sd : cd;
-  } else {
-    // sums of (-1)^k x^2k / (2k)! and x (-1)^k x^2k / (2k+1)!: up to |x| = 2^-10 three terms leave
-    // less than 2e-21, up to 1/64 five (1e-25), up to 1/4 nine (1e-27)
-    const double x2 = x * x;
-    p = 0.0;
-    if (hx > 0x3f500000) {
-      if (hx > 0x3f900000) {
-        p = sine ? 1.0 / 355687428096000.0 : 1.0 / 20922789888000.0;
-        p = fma(p, x2, sine ? -1.0 / 1307674368000.0 : -1.0 / 87178291200.0);
-        p = fma(p, x2, sine ? 1.0 / 6227020800.0 : 1.0 / 479001600.0);
-        p = fma(p, x2, sine ? -1.0 / 39916800.0 : -1.0 / 3628800.0);
-      }
-      p = fma(p, x2, sine ? 1.0 / 362880.0 : 1.0 / 40320.0);
-      p = fma(p, x2, sine ? -1.0 / 5040.0 : -1.0 / 720.0);
-    }
-    p = fma(p, x2, sine ? 1.0 / 120.0 : 1.0 / 24.0);
-    p = fma(p, x2, sine ? -1.0 / 6.0 : -1.0 / 2.0);
-    p = fma(p, x2, 1.0);
-    const double ps = p * x;
-    if (sine) p = ps;
-  }
-  const double other = __shfl_xor_sync(0xffffffffu, p, 1);
-  const double trig = fma(x0, sine ? other : p, y0 * (sine ? p : other));  // cos, sin by lane parity
-  const float tf = (float)trig, vf = (float)v;
-  if constexpr (D64) {
-    const double c = __shfl_sync(0xffffffffu, trig, 0), sn = __shfl_sync(0xffffffffu, trig, 1);
-    const double w = lane < 2 ? c : (lane < 4 ? sn : v);
-    if (lane < 6) st_word(pose + 8 + lane, e, (unsigned)((lane & 1) ? __double2hiint(w) : __double2loint(w)));
-  } else {
-    if (lane < 3) st_word(pose + 6 + lane, e, __float_as_uint(lane < 2 ? tf : vf));
-  }
-  if (lane == 0) {
-    nx->s[6] = fr ? q0 + v : q0;
-    nx->s[7] = v;
-    nx->om = vf;
-    nx->cs = trig;
-    nx->csf = tf;
-  } else if (lane == 1) {
-    nx->sn = trig;
-    nx->snf = tf;
-  }
-  return st;
-}
-
-// The exchange's words: sums [parity][component][CTA], then iterates [parity][16].
-__device__ __forceinline__ Words* sum_words(void* w, unsigned e, int comp, int cells) {
-  return static_cast<Words*>(w) + ((long long)(e & 1u) * NVC + comp) * cells;
-}
-__device__ __forceinline__ unsigned long long* pose_words(void* w, unsigned e, int cells) {
-  return reinterpret_cast<unsigned long long*>(static_cast<Words*>(w) + 2LL * NVC * cells) + (e & 1u) * 16;
-}
-
-// CTA 0: warp `comp` adds the CTAs' sums of its component and runs its part of the EOM.
-template <typename T>
-__device__ __forceinline__ void flag_root(const Geo& g, Ctrl* ctrl, Dof* row, const Moments* __restrict__ mom,
-                                          void* words, int cells, unsigned e0, bool skip, Dof (&sd)[2], int& gave_up) {
-  using V = typename SumOf<T>::type;
-  constexpr int DW = (int)(sizeof(Dof) / sizeof(double));
-  const int tid = threadIdx.x, comp = tid >> 5, lane = tid & 31, K = g.K;
-  if (comp >= NVC) return;
-  auto sync = [] { asm volatile("bar.sync 1, %0;" ::"n"(NVC * 32) : "memory"); };
-  double* sdw = reinterpret_cast<double*>(sd);
-  for (int k = 1; k <= K; ++k) {
-    const unsigned e = e0 + (unsigned)k;
-    EomPart eom;
-    eom.prepare(g, *mom, sd[0], sd[1], comp, lane);
-    const Words* place = sum_words(words, e, comp, cells);
-    V s;
-    s.zero();
-    WaitLimit limit;
-    bool ok = true;
-    for (int q0 = lane; q0 < cells && ok; q0 += 32 * 4) {
-      Words w[4];
-      bool have;
-      do {  // up to four words at a time in flight
-        have = true;
-#pragma unroll
-        for (int j = 0; j < 4; ++j)
-          if (q0 + 32 * j < cells) w[j] = ld_words(place + q0 + 32 * j);
-#pragma unroll
-        for (int j = 0; j < 4; ++j)
-          if (q0 + 32 * j < cells) have = have && (unsigned)(w[j].a >> 32) == e && (unsigned)(w[j].b >> 32) == e;
-        if (!have && limit.over(&ctrl->status)) ok = false;
-      } while (!have && ok);
-      if (ok)
-#pragma unroll
-        for (int j = 0; j < 4; ++j)
-          if (q0 + 32 * j < cells) {
-            V x;
-            x.read(w[j]);
-            s.add(x);
-          }
-    }
-    __syncwarp();
-    ok = __all_sync(0xffffffffu, ok);
-    if (!ok && lane == 0) gave_up = 1;
-    sync();  // every warp has read sd[1]
-    if (gave_up) return;
-    warp_total<1>(s);
-    // the skip hook (a test) publishes into the sums' unused parity-free end: no one reads it
-    unsigned long long* pose = skip ? pose_words(words, 0u, cells) + 32 : pose_words(words, e, cells);
-    const int st = eom.finish<T>(g, s.value(), &sd[1], pose, e, comp, lane);
-    if (st && lane == 0) atomicOr(&ctrl->status, st);
-    sync();
-    if (tid < DW) {
-      reinterpret_cast<double*>(row + k)[tid] = sdw[DW + tid];
-      if (k == K) reinterpret_cast<double*>(row + K + 1)[tid] = sdw[DW + tid];  // s(t): the next step's row 0
-    }
-  }
-}
-
 template <typename T>
 __global__ void __launch_bounds__(FlagCta<T>::max_threads, 1)
     k_couple_flag(Geo g, Slots<T> S, Ctrl* ctrl, Dof* it, const T* __restrict__ kref, const Moments* __restrict__ mom,
@@ -528,7 +196,7 @@ __global__ void __launch_bounds__(FlagCta<T>::max_threads, 1)
   constexpr int DW = (int)(sizeof(Dof) / sizeof(double));
   __shared__ V part[32 * NVC];
   __shared__ Dof sd[2];  // CTA 0: s(t-1), the current iterate
-  __shared__ Pose<T> pose;
+  __shared__ Pose<T, 2> pose;
   __shared__ int gave_up;
   if (*(volatile int*)&ctrl->status & ST_SYNC_TIMEOUT) return;  // an earlier launch gave up
   const int t = ctrl->t0 + di, base = ctrl->base, K = g.K;
@@ -544,7 +212,7 @@ __global__ void __launch_bounds__(FlagCta<T>::max_threads, 1)
   if (tid == 0) gave_up = 0;
   __syncthreads();
   if (cta < 0) {
-    flag_root<T>(g, ctrl, row, mom, words, G, e0, (ctrl->sync_skip & 1) != 0, sd, gave_up);
+    flag_root<T, 2, 2>(g, ctrl, row, mom, words, G, e0, (ctrl->sync_skip & 1) != 0, sd, gave_up);
     return;
   }
   if (tid == 0) pose.set(sd[0]);
@@ -580,7 +248,7 @@ __global__ void __launch_bounds__(FlagCta<T>::max_threads, 1)
   for (int k = 1; k <= K; ++k) {
     const bool last = k == K;
     const unsigned e = e0 + (unsigned)k;
-    const Pose<T> P = pose;
+    const Pose<T, 2> P = pose;
     T v[NVC] = {T(0), T(0), T(0)};
     for (int c0 = first; c0 < BC; c0 += W * CPW) {  // uniform per warp
       const int bl = c0 + sub;
@@ -635,34 +303,8 @@ __global__ void __launch_bounds__(FlagCta<T>::max_threads, 1)
       if (lane + q * LC < NVC && lane < LC) part[warp * NVC + lane + q * LC] = s;
     }
     __syncthreads();
-    if (warp < NVC) {  // the CTA's sum of component `warp`
-      V s;
-      s.zero();
-      if (lane < nw) s = part[lane * NVC + warp];
-      warp_total<1>(s);
-      if (lane == 0) st_words(sum_words(words, e, warp, G) + cta, s.words(e));
-    }
+    flag_exchange<T, 2>(words, e, cta, G, last, &ctrl->status, part, pose, gave_up);
     if (last) return;
-    if (warp == NVC) {  // the next iterate
-      const unsigned long long* p = pose_words(words, e, G);
-      unsigned long long w = 0;
-      WaitLimit limit;
-      bool ok = true;
-      if (lane < Pose<T>::words)
-        while ((unsigned)((w = ld_word(p + lane)) >> 32) != e)
-          if (limit.over(&ctrl->status)) {
-            ok = false;
-            break;
-          }
-      __syncwarp();
-      const unsigned hi = __shfl_down_sync(0xffffffffu, (unsigned)w, 1);
-      if (lane < Pose<T>::words) {
-        if (ok)
-          pose.put(lane, (unsigned)w, hi);
-        else
-          gave_up = 1;
-      }
-    }
     __syncthreads();
     if (gave_up) return;
   }
@@ -692,17 +334,21 @@ int flag_shape(const Geo& g, int* threads) {
 
 void setup_couple_flag(Geo* g, bool fp64) {
   g->flag_ctas = g->flag_threads = 0;
-  if (g->dim != 2 || g->box_cells >= (1LL << 27) || g->N >= (1LL << 31)) return;
-  g->flag_ctas = fp64 ? flag_shape<double>(*g, &g->flag_threads) : flag_shape<float>(*g, &g->flag_threads);
+  if (g->dim == 3) {
+    setup_couple_axis3d(g, fp64);
+  } else if (g->box_cells < (1LL << 27) && g->N < (1LL << 31)) {
+    g->flag_ctas = fp64 ? flag_shape<double>(*g, &g->flag_threads) : flag_shape<float>(*g, &g->flag_threads);
+  }
   cudaGetLastError();  // a query that failed leaves the other forms in use
 }
 
-// the sums of the CTAs with cells, the iterates (two parities), and 16 words the test hook writes to
-size_t couple_flag_bytes(int ctas) { return 2 * (size_t)(ctas - 1) * NVC * sizeof(Words) + 48 * 8; }
+// The sums of the CTAs with cells (up to four components), the iterates of both parities and the hook's.
+size_t couple_flag_bytes(int ctas) { return 2 * (size_t)(ctas - 1) * 4 * sizeof(Words) + 3 * kPoseWords * 8; }
 
 template <typename T>
 void launch_couple_flag(const Geo& g, const Slots<T>& S, Ctrl* ctrl, Dof* it, const T* kref, const Moments* mom,
                         void* words, T* boxstore, int nbox, int di, cudaStream_t st) {
+  if (g.dim == 3) return launch_couple_axis3d<T>(g, S, ctrl, it, kref, mom, words, boxstore, nbox, di, st);
   launch_coop(k_couple_flag<T>, dim3((unsigned)g.flag_ctas), dim3((unsigned)g.flag_threads), 0, st, g, S, ctrl, it, kref,
               mom, words, boxstore, nbox, di);
 }

@@ -128,7 +128,7 @@ void launch_adj_coop(const Geo& g, Ctrl* ctrl, const Dof* it, const T* kref, con
 // as the device holds at once (0 if the kernel cannot be resident); sets g->coop_fwd, g->coop_adj.
 void setup_coop(Geo* g, bool fp64);
 
-// The same in 2D with the sums exchanged through flagged words (lks_couple2d.cu): g.flag_ctas CTAs of
+// The same with the sums exchanged through flagged words (2D and 3D about one axis): g.flag_ctas CTAs of
 // g.flag_threads threads, set by setup_couple_flag (0 if it does not apply). words:
 // couple_flag_bytes(CTAs) bytes (at most kFlagMaxCtas CTAs), zeroed before a march (the words carry the iteration's number in the run).
 constexpr int kFlagMaxCtas = 1024;
@@ -137,6 +137,18 @@ size_t couple_flag_bytes(int ctas);
 template <typename T>
 void launch_couple_flag(const Geo& g, const Slots<T>& S, Ctrl* ctrl, Dof* it, const T* kref, const Moments* mom,
                         void* words, T* boxstore, int nbox, int di, cudaStream_t st);
+
+// 3D forms about one rotation axis (lks_axis3d.cu). setup and launch of the coupling are reached
+// through setup_couple_flag and launch_couple_flag, the coefficient and design kernels through
+// launch_rev_coef and launch_rev_design.
+bool axis3d_fits(const Geo& g);
+void setup_couple_axis3d(Geo* g, bool fp64);
+template <typename T>
+void launch_couple_axis3d(const Geo& g, const Slots<T>& S, Ctrl* ctrl, Dof* it, const T* kref, const Moments* mom,
+                          void* words, T* boxstore, int nbox, int di, cudaStream_t st);
+template <typename T>
+void launch_apply_axis3d(const Geo& g, const Slots<T>& S, const Ctrl* ctrl, const Dof* it, const T* kref, T* boxstore,
+                         int nbox, int di, cudaStream_t st);
 
 // Recompute: Brinkman update with the stored iterate s^(K-1); writes u(t) and the box store of u*.
 template <typename T>
@@ -181,6 +193,16 @@ void launch_rev_step(const Geo& g, const RevBuffers& R, Ctrl* ctrl, const Dof* i
 template <typename T>
 void launch_rev_design(const Geo& g, const RevBuffers& R, Ctrl* ctrl, const Dof* it, int nsteps, int di,
                        cudaStream_t st);
+
+// Their 3D forms; coef_axis3d_fits: the whole design grid is the design domain.
+bool coef_axis3d_fits(const Geo& g);
+int coef_axis3d_ctas(const Geo& g, bool fp64);
+template <typename T>
+void launch_coef_axis3d(const Geo& g, const RevBuffers& R, const Ctrl* ctrl, const Dof* it, const T* kref, const T* boxstore,
+                        int nbox, int nsteps, int di, cudaStream_t st);
+template <typename T>
+void launch_design_axis3d(const Geo& g, const RevBuffers& R, Ctrl* ctrl, const Dof* it, int nsteps, int di,
+                          cudaStream_t st);
 
 // Test export: the design points the coupling's gather accepts for each cell of the box of the
 // iterate s, as out[box cell][5] = (count, least index or -1, largest index, sum, sum of squares).

@@ -30,135 +30,14 @@
 // are left in a step's chain; the rest runs over whole chunks of steps. Gradients measured on GB300,
 // before -> after: 512x256 / 128^2, 200 steps 30.2 -> 21.1 ms; 1024x512 / 256^2, 100 steps 30.2 -> 22.3
 // ms; 80x40 / 16^2 FP64, 400 steps 256 -> 135 ms; 128x64x64 / 48^3, 40 steps 26.3 -> 21.9 ms.
-#include "lks_body_common.cuh"
+#include <algorithm>
+#include <climits>
+
+#include "lks_reverse.cuh"
 
 namespace lks {
 
 namespace {
-
-constexpr int kRevThreads = 256;
-constexpr int kRevMaxItr = 64;     // iterations k_rev_apply's shared memory holds (432 bytes each)
-constexpr int kRevMaxCtas = 304;  // k_rev_const, k_rev_apply: every CTA of the latter sums the former's partials
-
-// Planes of a step's slab (box cells each). Per iteration: kappa/(1+kappa), L/(1+kappa) in the plane,
-// u, kappa du/dkappa, and the dJ/dT coefficient of dJ/dkappa (k_rev_apply puts dJ/dkappa there).
-// Then for iteration N_itr: 1/(1+kappa), du/dkappa, du/d(x^G, theta), du/du^G and du/domega parts.
-template <int D>
-struct RevPlanes {
-  static constexpr int beta = 0, iL = 1, u = 3, kd = 3 + D, eps = 3 + 2 * D, per_itr = 4 + 2 * D;
-  static constexpr int inv = 0, del = 1, Q = 1 + D, bphi = Q + (D + 1) * D, bP = bphi + 1, consts = bP + 2;
-};
-// Sums of k_rev_coef: rows x^G and theta by columns lam_F and lam_T, then the u^G and omega rows.
-template <int D>
-struct RevSums {
-  static constexpr int uF = (D + 1) * (D + 1), uT = uF + 1, oF = uT + 2, oT = oF + 2, N = oT + 1;
-};
-template <int D>
-__host__ __device__ constexpr int rev_nconst() { return 2 * D + 2; }  // c: x^G[D], theta, u^G[D], omega
-
-// Block sums of NV per-thread values with few instructions: the values go through shared memory
-// (rows of kRevThreads), 8 threads sum each row's eighths in order and combine them with shuffles.
-// A shuffle tree over all threads costs NV * 5 levels in every warp: with 15 to 22 values that was
-// as much as the gather itself. FP32 values are summed as double-float pairs.
-template <int NV>
-struct RowBuf {
-  static constexpr int pitch = kRevThreads + 1;
-};
-template <int NV>
-__device__ __forceinline__ void row_sums(const float (&v)[NV], float* buf, float2* out) {
-  constexpr int pitch = RowBuf<NV>::pitch;
-  const int tid = threadIdx.x;
-  __syncthreads();
-#pragma unroll
-  for (int i = 0; i < NV; ++i) buf[i * pitch + tid] = v[i];
-  __syncthreads();
-  const int row = tid >> 3, seg = tid & 7;
-  static_assert(NV * 8 <= kRevThreads, "eight threads per value");
-  if ((tid & ~31) < NV * 8) {  // whole warps (shuffles below)
-    float hi = 0.0f, lo = 0.0f;
-    if (row < NV) {
-      const float* p = buf + row * pitch + seg;
-#pragma unroll 8
-      for (int j = 0; j < kRevThreads / 8; ++j) {
-        const float b = p[8 * j], s = hi + b, bb = s - hi;
-        lo += (hi - (s - bb)) + (b - bb);
-        hi = s;
-      }
-    }
-#pragma unroll
-    for (int off = 4; off > 0; off >>= 1)
-      df_add(hi, lo, __shfl_down_sync(0xffffffffu, hi, off, 8), __shfl_down_sync(0xffffffffu, lo, off, 8));
-    if (row < NV && seg == 0) out[row] = make_float2(hi, lo);
-  }
-}
-template <int NV>
-__device__ __forceinline__ void row_sums(const double (&v)[NV], double* buf, double* out) {
-  constexpr int pitch = RowBuf<NV>::pitch;
-  const int tid = threadIdx.x;
-  __syncthreads();
-#pragma unroll
-  for (int i = 0; i < NV; ++i) buf[i * pitch + tid] = v[i];
-  __syncthreads();
-  const int row = tid >> 3, seg = tid & 7;
-  static_assert(NV * 8 <= kRevThreads, "eight threads per value");
-  if ((tid & ~31) < NV * 8) {
-    double s = 0.0;
-    if (row < NV) {
-      const double* p = buf + row * pitch + seg;
-#pragma unroll 8
-      for (int j = 0; j < kRevThreads / 8; ++j) s += p[8 * j];
-    }
-#pragma unroll
-    for (int off = 4; off > 0; off >>= 1) s += __shfl_down_sync(0xffffffffu, s, off, 8);
-    if (row < NV && seg == 0) out[row] = s;
-  }
-}
-// Row `row` of partials [n][nv] summed by 8 threads in a fixed order (result in seg 0's thread).
-__device__ __forceinline__ double part_sum(const float2* p, int n, int nv, int row, int seg) {
-  float hi = 0.0f, lo = 0.0f;
-#pragma unroll 4
-  for (int q = seg; q < n; q += 8) {
-    const float2 b = __ldcg(p + (long long)q * nv + row);
-    df_add(hi, lo, b.x, b.y);
-  }
-#pragma unroll
-  for (int off = 4; off > 0; off >>= 1)
-    df_add(hi, lo, __shfl_down_sync(0xffffffffu, hi, off, 8), __shfl_down_sync(0xffffffffu, lo, off, 8));
-  return (double)hi + (double)lo;
-}
-__device__ __forceinline__ double part_sum(const double* p, int n, int nv, int row, int seg) {
-  double s = 0.0;
-#pragma unroll 4
-  for (int q = seg; q < n; q += 8) s += __ldcg(p + (long long)q * nv + row);
-#pragma unroll
-  for (int off = 4; off > 0; off >>= 1) s += __shfl_down_sync(0xffffffffu, s, off, 8);
-  return s;
-}
-
-// w(r) and w'(r) inside the support.
-__device__ __forceinline__ void w_dw(int wk, float r, float* w, float* dw) {
-  *w = wfun(wk, r);
-  *dw = dwfun(wk, r);
-}
-__device__ __forceinline__ void w_dw(int wk, double r, double* w, double* dw) {
-  if (wk == W_BILINEAR) {
-    *w = wfun(wk, r);
-    *dw = dwfun(wk, r);
-    return;
-  }
-  double s, c;
-  sincospi(0.5 * r, &s, &c);
-  *w = 0.25 * (1.0 + c);
-  *dw = -0.125 * 3.141592653589793 * s;
-}
-
-// Sums over the design points within the support of one cell: index 0 with W, 1 + e with dW/dx_e
-// (e the world axis); q: sums with the rotation derivative W_b l_c - W_c l_b times l_b, l_c.
-template <typename T>
-struct Moments1 {
-  T phi[4], kap[4], Pb[4], Pc[4], Lb[4], Lc[4];
-  T qPb, qPc, qLb, qLc;
-};
 
 template <typename T, int D, int AX>
 __device__ __forceinline__ void gather_moments(const Geo& g, const T* __restrict__ kref, const T (&d)[3], T cs, T sn,
@@ -274,9 +153,6 @@ __device__ __forceinline__ void gather_moments(const Geo& g, const T* __restrict
   }
 }
 
-// Step of slab i of the chunk that starts di steps below ctrl->t0.
-__device__ __forceinline__ int rev_step(const Ctrl* ctrl, int di, int i) { return ctrl->t0 - di - i; }
-
 template <typename T, int D, int AX>
 __global__ void __launch_bounds__(kRevThreads) k_rev_coef(Geo g, const Ctrl* ctrl, const Dof* it,
                                                           const T* __restrict__ kref, const T* __restrict__ boxstore,
@@ -284,7 +160,6 @@ __global__ void __launch_bounds__(kRevThreads) k_rev_coef(Geo g, const Ctrl* ctr
                                                           typename Partial<T>::type* __restrict__ mpart, int di) {
   using RP = RevPlanes<D>;
   using RS = RevSums<D>;
-  constexpr int b = Axes<AX>::B, c = Axes<AX>::C;
   extern __shared__ __align__(16) unsigned char rev_smem[];
   const int K = g.K, k = (int)blockIdx.y + 1, i = blockIdx.z;
   const int t = rev_step(ctrl, di, i), base = ctrl->base;
@@ -315,74 +190,7 @@ __global__ void __launch_bounds__(kRevThreads) k_rev_coef(Geo g, const Ctrl* ctr
       A.qPb = A.qPc = A.qLb = A.qLc = T(0);
     }
     const T* bs = boxstore + (long long)((t - base - 1) % nbox) * BC * D;
-    const T kap = A.kap[0], inv = T(1) / (T(1) + kap), beta = kap * inv, om = V.om;
-    T us[3], u[3], del[3];
-#pragma unroll
-    for (int a = 0; a < D; ++a) {
-      us[a] = V.ug[a] * A.phi[0];
-      if (a == b) us[a] -= om * A.Pc[0];
-      if (a == c) us[a] += om * A.Pb[0];
-      u[a] = ing ? (bs[a * BC + bl] + kap * us[a]) * inv : T(0);  // no stored u* off the grid
-      del[a] = (us[a] - u[a]) * inv;
-    }
-    T* P = slabs + (long long)i * slab + bl;
-    T* Pk = P + (long long)(k - 1) * RP::per_itr * BC;
-    Pk[RP::beta * BC] = beta;
-    Pk[RP::iL * BC] = inv * A.Lb[0];
-    Pk[(RP::iL + 1) * BC] = inv * A.Lc[0];
-#pragma unroll
-    for (int a = 0; a < D; ++a) {
-      Pk[(RP::u + a) * BC] = u[a];
-      Pk[(RP::kd + a) * BC] = kap * del[a];
-    }
-    Pk[RP::eps * BC] = A.Lb[0] * del[c] - A.Lc[0] * del[b];
-    const T bphi = beta * A.phi[0], bPb = beta * A.Pb[0], bPc = beta * A.Pc[0];
-    T* Pc = P + (long long)K * RP::per_itr * BC;
-    if (k == K) {
-      Pc[RP::inv * BC] = inv;
-#pragma unroll
-      for (int a = 0; a < D; ++a) Pc[(RP::del + a) * BC] = del[a];
-      Pc[RP::bphi * BC] = bphi;
-      Pc[RP::bP * BC] = bPb;
-      Pc[(RP::bP + 1) * BC] = bPc;
-    }
-    // rows x^G_e (derivative -dW/dx_e) and theta (W_b l_c - W_c l_b, and l turning with the body)
-#pragma unroll
-    for (int e = 0; e <= D; ++e) {
-      T dphi, dk, dPb, dPc, dLb, dLc;
-      if (e < D) {
-        dphi = -A.phi[1 + e];
-        dk = -A.kap[1 + e];
-        dPb = -A.Pb[1 + e];
-        dPc = -A.Pc[1 + e];
-        dLb = -A.Lb[1 + e];
-        dLc = -A.Lc[1 + e];
-      } else {
-        dphi = A.Pc[1 + b] - A.Pb[1 + c];
-        dk = A.Lc[1 + b] - A.Lb[1 + c];
-        dPb = A.qPb - A.Pc[0];
-        dPc = A.qPc + A.Pb[0];
-        dLb = A.qLb - A.Lc[0];
-        dLc = A.qLc + A.Lb[0];
-      }
-      T du[3];
-#pragma unroll
-      for (int a = 0; a < D; ++a) {
-        T dus = V.ug[a] * dphi;
-        if (a == b) dus -= om * dPc;
-        if (a == c) dus += om * dPb;
-        du[a] = del[a] * dk + beta * dus;
-        if (k == K) Pc[(RP::Q + e * D + a) * BC] = du[a];
-        v[e * (D + 1) + a] = kap * du[a] + u[a] * dk;
-      }
-      v[e * (D + 1) + D] = A.Lb[0] * du[c] - A.Lc[0] * du[b] + dLb * u[c] - dLc * u[b];
-    }
-    v[RS::uF] = kap * bphi;
-    v[RS::uT] = -A.Lc[0] * bphi;
-    v[RS::uT + 1] = A.Lb[0] * bphi;
-    v[RS::oF] = -kap * bPc;
-    v[RS::oF + 1] = kap * bPb;
-    v[RS::oT] = A.Lb[0] * bPb + A.Lc[0] * bPc;
+    rev_cell<T, D, AX>(g, V, A, ing, bs, bl, slabs + (long long)i * slab + bl, k, v);
   }
   row_sums<RS::N>(v, reinterpret_cast<T*>(rev_smem),
                   mpart + (((long long)i * K + (k - 1)) * gridDim.x + blockIdx.x) * RS::N);
@@ -619,67 +427,36 @@ __global__ void __launch_bounds__(kRevThreads) k_rev_apply(Geo g, Ctrl* ctrl, co
   }
 }
 
-// Kernel weights of the 2s window cells from floor(x) - s + 1, at the fraction fr of x.
-__device__ __forceinline__ void window_weights(const Geo& g, float fr, float (&w)[4]) {
-  if (g.wk == W_BILINEAR) {
-    w[0] = 1.0f - fr;
-    w[1] = fr;
-    w[2] = w[3] = 0.0f;
-    return;
-  }
-  const float c = __cosf(1.57079632679f * fr), s = __sinf(1.57079632679f * fr);
-  w[0] = 0.25f * (1.0f - s);
-  w[1] = 0.25f * (1.0f + c);
-  w[2] = 0.25f * (1.0f + s);
-  w[3] = 0.25f * (1.0f - c);
-}
-__device__ __forceinline__ void window_weights(const Geo& g, double fr, double (&w)[4]) {
-  if (g.wk == W_BILINEAR) {
-    w[0] = 1.0 - fr;
-    w[1] = fr;
-    w[2] = w[3] = 0.0;
-    return;
-  }
-  double s, c;
-  sincospi(0.5 * fr, &s, &c);
-  w[0] = 0.25 * (1.0 - s);
-  w[1] = 0.25 * (1.0 + c);
-  w[2] = 0.25 * (1.0 + s);
-  w[3] = 0.25 * (1.0 - c);
-}
-
-// LN lanes per design point, one row (2D) or plane (3D) of the window each; split blockIdx.y takes
-// the chunk's steps blockIdx.y, blockIdx.y + gridDim.y, ... and keeps its own dJ/dkappa^ref.
-template <typename T, int D, int AX>
+// 2D: LN lanes per design point, one row of the window each; split blockIdx.y takes the chunk's steps
+// blockIdx.y, blockIdx.y + gridDim.y, ... and keeps its own dJ/dkappa^ref. (3D: k_design_axis3d.)
+template <typename T>
 __global__ void __launch_bounds__(kRevThreads) k_rev_design(Geo g, Ctrl* ctrl, const Dof* it,
                                                             const T* __restrict__ slabs, long long slab,
                                                             const T* __restrict__ lamh, double* __restrict__ dkp,
                                                             int nsteps, int di) {
-  using RP = RevPlanes<D>;
-  constexpr int b = Axes<AX>::B, c = Axes<AX>::C;
+  using RP = RevPlanes<2>;
   const int K = g.K, lane = threadIdx.x % LN;
   const int m = (int)((blockIdx.x * (unsigned)kRevThreads + threadIdx.x) / LN);
   const int mm = m < g.ND ? m : 0;
-  const int ix = mm % g.nd[0], iy = (mm / g.nd[0]) % g.nd[1], iz = mm / (g.nd[0] * g.nd[1]);
-  const bool valid = m < g.ND && dsq(ix, g.nd[0]) + dsq(iy, g.nd[1]) + dsq(iz, g.nd[2]) <= g.rad4;
-  const T r[3] = {(T)ix - pivot<T>(g, 0), (T)iy - pivot<T>(g, 1), D == 3 ? (T)iz - pivot<T>(g, 2) : T(0)};
-  const int S2 = 2 * g.s;
+  const int ix = mm % g.nd[0], iy = mm / g.nd[0];
+  const bool valid = m < g.ND && dsq(ix, g.nd[0]) + dsq(iy, g.nd[1]) <= g.rad4;
+  const T r[3] = {(T)ix - pivot<T>(g, 0), (T)iy - pivot<T>(g, 1), T(0)};
+  const int S2 = 2 * g.s, B0 = g.B[0], B1 = g.B[1];
   const long long BC = g.box_cells;
-  const int B0 = g.B[0], B1 = g.B[1], B2 = (D == 3) ? g.B[2] : 1;
   bool inside = true;
   double acc = 0.0;
   for (int i = blockIdx.y; i < nsteps; i += gridDim.y) {
     const Dof* row = it + (long long)(rev_step(ctrl, di, i) - 1) * (K + 1);
     int lo[3];
-    box_origin<D>(g, row[0], lo[0], lo[1], lo[2]);
+    box_origin<2>(g, row[0], lo[0], lo[1], lo[2]);
     for (int k = K; k >= 1; --k) {
       const DofView<T> V(row[k - 1]);
-      T l[3], dl[3], usr[3], fr[3], w[3][4];
-      int f[3] = {0, 0, 0};
-      rot<AX>(V.cs, V.sn, r, l);
-      drot<AX>(V.cs, V.sn, r, dl);
+      T l[3], dl[3], usr[2], fr[2], w[2][4];
+      int f[2] = {0, 0};
+      rot<2>(V.cs, V.sn, r, l);
+      drot<2>(V.cs, V.sn, r, dl);
 #pragma unroll
-      for (int a = 0; a < D; ++a) {
+      for (int a = 0; a < 2; ++a) {
         usr[a] = V.ug[a] + V.om * dl[a];
         V.split(a, l[a], &f[a], &fr[a]);
         window_weights(g, fr[a], w[a]);
@@ -687,52 +464,40 @@ __global__ void __launch_bounds__(kRevThreads) k_rev_design(Geo g, Ctrl* ctrl, c
       }
       // the window's cells with weight 0 (fr = 0 puts the last one on the support's edge) need not
       // lie in the box
-      constexpr int E = (D == 3) ? 2 : 1;
       T we = T(0);
 #pragma unroll
       for (int q = 0; q < 4; ++q)
-        if (q == lane) we = w[E][q];
+        if (q == lane) we = w[1][q];
       const bool here = valid && lane < S2 && we != T(0);
-      const int pe = f[E] + lane;
-      if (here && (f[0] < 0 || f[0] + S2 - 1 - (fr[0] == T(0)) >= B0 || pe < 0 || pe >= (D == 3 ? B2 : B1) ||
-                   (D == 3 && (f[1] < 0 || f[1] + S2 - 1 - (fr[1] == T(0)) >= B1))))
-        inside = false;
-      T uref[3] = {T(0), T(0), T(0)}, slk = T(0);
+      const int pe = f[1] + lane;
+      if (here && (f[0] < 0 || f[0] + S2 - 1 - (fr[0] == T(0)) >= B0 || pe < 0 || pe >= B1)) inside = false;
+      T uref[2] = {T(0), T(0)}, slk = T(0);
       if (here && inside) {
-        const T* P = slabs + (long long)i * slab + (long long)(k - 1) * RP::per_itr * BC;
-        const T* Pu = P + RP::u * BC;
-        const T* Pl = P + RP::eps * BC;
+        const T* P = slabs + (long long)i * slab + (long long)(k - 1) * RP::per_itr * BC + f[0] + B0 * pe;
 #pragma unroll
-        for (int q1 = 0; q1 < (D == 3 ? 4 : 1); ++q1) {
-          if (D == 3 && (q1 >= S2 || w[1][q1] == T(0))) continue;
-          const T w1 = D == 3 ? we * w[1][q1] : we;
-          const int rowb = D == 3 ? f[0] + B0 * (f[1] + q1 + B1 * pe) : f[0] + B0 * pe;
+        for (int q = 0; q < 4; ++q) {
+          if (q >= S2 || w[0][q] == T(0)) continue;
+          const T W = w[0][q] * we;
+          slk += W * __ldg(P + RP::eps * BC + q);
 #pragma unroll
-          for (int q0 = 0; q0 < 4; ++q0) {
-            if (q0 >= S2 || w[0][q0] == T(0)) continue;
-            const T W = w[0][q0] * w1;
-            const int o = rowb + q0;
-            slk += W * __ldg(Pl + o);
-#pragma unroll
-            for (int a = 0; a < D; ++a) uref[a] += W * __ldg(Pu + a * BC + o);
-          }
+          for (int a = 0; a < 2; ++a) uref[a] += W * __ldg(P + (RP::u + a) * BC + q);
         }
       }
 #pragma unroll
       for (int off = 1; off < LN; off <<= 1) {
         slk += __shfl_xor_sync(0xffffffffu, slk, off);
 #pragma unroll
-        for (int a = 0; a < D; ++a) uref[a] += __shfl_xor_sync(0xffffffffu, uref[a], off);
+        for (int a = 0; a < 2; ++a) uref[a] += __shfl_xor_sync(0xffffffffu, uref[a], off);
       }
       if (valid && lane == 0) {
         const T* lam = lamh + ((long long)i * K + (k - 1)) * 4;
         T dk = slk;
 #pragma unroll
-        for (int a = 0; a < D; ++a) {
+        for (int a = 0; a < 2; ++a) {
           uref[a] -= usr[a];
           dk += lam[a] * uref[a];
         }
-        dk += lam[3] * (l[b] * uref[c] - l[c] * uref[b]);
+        dk += lam[3] * (l[0] * uref[1] - l[1] * uref[0]);
         acc += (double)dk;
       }
     }
@@ -770,9 +535,14 @@ template <typename T, int D, int AX>
 void coef_ax(const Geo& g, const RevBuffers& R, Ctrl* ctrl, const Dof* it, const T* kref, const Moments* mom,
              const T* boxstore, int nbox, int nsteps, int di, cudaStream_t st) {
   using PT = typename Partial<T>::type;
-  const unsigned nc = (unsigned)((g.box_cells + kRevThreads - 1) / kRevThreads);
-  launch(k_rev_coef<T, D, AX>, dim3(nc, g.K, nsteps), kRevThreads, rev_row_bytes<T, D>(RevSums<D>::N), st, g,
-         (const Ctrl*)ctrl, it, kref, boxstore, nbox, (T*)R.slabs, R.slab, (PT*)R.mpart, di);
+  unsigned nc = (unsigned)((g.box_cells + kRevThreads - 1) / kRevThreads);
+  if (D == 3 && coef_axis3d_fits(g)) {
+    nc = (unsigned)coef_axis3d_ctas(g, sizeof(T) == 8);
+    launch_coef_axis3d<T>(g, R, ctrl, it, kref, boxstore, nbox, nsteps, di, st);
+  } else {
+    launch(k_rev_coef<T, D, AX>, dim3(nc, g.K, nsteps), kRevThreads, rev_row_bytes<T, D>(RevSums<D>::N), st, g,
+           (const Ctrl*)ctrl, it, kref, boxstore, nbox, (T*)R.slabs, R.slab, (PT*)R.mpart, di);
+  }
   launch(k_rev_mat<T, D, AX>, dim3(g.K, nsteps), kRevThreads, 0, st, g, (const Ctrl*)ctrl, it, mom, (const PT*)R.mpart,
          (int)nc, (RevMat*)R.mats, di);
 }
@@ -786,13 +556,6 @@ void step_ax(const Geo& g, const RevBuffers& R, Ctrl* ctrl, const Dof* it, T* Lb
   launch(k_rev_apply<T, D, AX>, nc + 1, kRevThreads, (size_t)g.K * (sizeof(RevMat) + 4 * (sizeof(double) + sizeof(T))), st, g, ctrl, it,
          (T*)R.slabs, R.slab, Lb, lstride, (const PT*)R.cpart, (int)nc, (const RevMat*)R.mats, (T*)R.lamh, di, i);
 }
-template <typename T, int D, int AX>
-void design_ax(const Geo& g, const RevBuffers& R, Ctrl* ctrl, const Dof* it, int nsteps, int di, cudaStream_t st) {
-  const unsigned nb = (unsigned)(((long long)g.ND * LN + kRevThreads - 1) / kRevThreads);
-  launch(k_rev_design<T, D, AX>, dim3(nb, R.splits), kRevThreads, 0, st, g, ctrl, it, (const T*)R.slabs, R.slab,
-         (const T*)R.lamh, R.dkp, nsteps, di);
-}
-
 #define LKS_REV_DISPATCH(F, ...)                  \
   do {                                            \
     if (g.dim == 2) F<T, 2, 2>(__VA_ARGS__);      \
@@ -804,7 +567,7 @@ void design_ax(const Geo& g, const RevBuffers& R, Ctrl* ctrl, const Dof* it, int
 }  // namespace
 
 bool reverse_affine_fits(const Geo& g) {
-  return g.ax != AX_FREE && g.box_cells < (1LL << 29) && g.K <= kRevMaxItr;
+  return (g.dim == 2 || axis3d_fits(g)) && g.box_cells < (1LL << 29) && g.K <= kRevMaxItr;
 }
 
 size_t reverse_layout(const Geo& g, bool fp64, int max_steps, RevBuffers* R) {
@@ -813,17 +576,20 @@ size_t reverse_layout(const Geo& g, bool fp64, int max_steps, RevBuffers* R) {
   const long long planes = D == 2 ? K * RevPlanes<2>::per_itr + RevPlanes<2>::consts
                                   : K * RevPlanes<3>::per_itr + RevPlanes<3>::consts;
   const long long nm = D == 2 ? RevSums<2>::N : RevSums<3>::N;
-  const long long nc = (g.box_cells + kRevThreads - 1) / kRevThreads;
+  long long nc = (g.box_cells + kRevThreads - 1) / kRevThreads;
+  if (D == 3 && coef_axis3d_fits(g)) nc = std::max(nc, (long long)coef_axis3d_ctas(g, fp64));
   R->slab = planes * g.box_cells;
   // steps per chunk: as many slabs as about half of the L2 holds, so that the planes written by one
   // kernel are read from L2 by the next; at least one, at most the segment
   const long long want = (64LL << 20) / (R->slab * esz);
   R->steps = (int)(want < 1 ? 1 : (want < max_steps ? want : max_steps));
   if (R->steps > 64) R->steps = 64;
-  // splits of the design kernel over the chunk's steps: about 2^17 threads
-  long long sp = (1LL << 17) / ((long long)g.ND * LN);
+  // splits of the design kernel over the chunk's steps (3D: steps and iterations): about 2^17 threads in
+  // 2D, 2^15 of the 3D form's, each of which takes eight points
+  long long sp = D == 2 ? (1LL << 17) / ((long long)g.ND * LN) : (1LL << 18) / g.ND;
   sp = sp < 1 ? 1 : (sp > 16 ? 16 : sp);
-  R->splits = (int)(sp < R->steps ? sp : R->steps);
+  const long long items = D == 2 ? R->steps : R->steps * K;
+  R->splits = (int)(sp < items ? sp : items);
   size_t off = 0;
   auto take = [&](long long bytes) {
     const size_t at = off;
@@ -870,7 +636,10 @@ void launch_rev_step(const Geo& g, const RevBuffers& R, Ctrl* ctrl, const Dof* i
 template <typename T>
 void launch_rev_design(const Geo& g, const RevBuffers& R, Ctrl* ctrl, const Dof* it, int nsteps, int di,
                        cudaStream_t st) {
-  LKS_REV_DISPATCH(design_ax, g, R, ctrl, it, nsteps, di, st);
+  if (g.dim == 3) return launch_design_axis3d<T>(g, R, ctrl, it, nsteps, di, st);
+  const unsigned nb = (unsigned)(((long long)g.ND * LN + kRevThreads - 1) / kRevThreads);
+  launch(k_rev_design<T>, dim3(nb, R.splits), kRevThreads, 0, st, g, ctrl, it, (const T*)R.slabs, R.slab,
+         (const T*)R.lamh, R.dkp, nsteps, di);
 }
 
 #define LKS_REV_INST(T)                                                                                             \
