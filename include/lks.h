@@ -276,10 +276,10 @@ LKS_API int lks_debug_copy_skip(lks_handle* h, int skip);
 /* How the handle runs each step's N_itr coupling iterations (Sec. 3.1) and their reverse: mode 1 as
  * one persistent cooperative launch per step (grid barriers between the iterations) when the device
  * holds its grid, mode 0 as one launch per iteration (with the finish kernels), mode 2 (the default)
- * by the problem: in 2D the forward runs as one cooperative launch per step whose CTAs exchange their
- * sums through flagged words (bounded waits of one second, LKS_ERR_TIMEOUT), in 3D as one launch per
- * iteration; the reverse about one rotation axis runs by linear maps of the iterations (no waits),
- * with free rotation as one launch per iteration. The words and the maps' buffers are allocated by the
+ * by the problem: about one rotation axis the forward runs as one cooperative launch per step whose
+ * CTAs exchange their sums through flagged words (bounded waits of one second, LKS_ERR_TIMEOUT) and
+ * the reverse by linear maps of the iterations (no waits); with free rotation both run as one launch
+ * per iteration. The words and the maps' buffers are allocated by the
  * first lks_forward and lks_adjoint if hbm_budget_bytes and the device have room; without it 2D bodies
  * whose box has more tiles than the persistent grid has CTAs take the persistent launch and the others
  * one launch per iteration. Mode -1 only asks. Returns 1 if the grid-barrier kernels are chosen (in

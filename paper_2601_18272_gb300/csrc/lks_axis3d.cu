@@ -8,6 +8,10 @@
 // column loads ZC + 3 values of kappa, forms ZC axial sums from them and adds those to the planes'
 // sums. A cell's gather of 64 pairs costs it about 16 (1 load, 7 multiply-adds), where the form with
 // one cell per four lanes (lks_device.cuh) ran every candidate test and weight again for every plane.
+// Loads are issued one design column ahead (the kernels wait on L2 otherwise: a quarter of their time).
+// Measured on GB300, FP32, per step of the 128x64x64 / 48^3 body: coupling 250 -> 73 us (five iterations),
+// recompute 27 -> 11, reverse sums 107 -> 73, dJ/dkappa^ref 95 -> 43 (against one cell per four lanes and
+// one design point per four lanes).
 //
 //   k_couple_axis3d  the N_itr coupling iterations of a step, sums and iterate exchanged through
 //                    flagged words (lks_flag.cuh), one cooperative launch
@@ -162,6 +166,20 @@ __device__ __forceinline__ void design_strides(const Geo& g, int& sb, int& sc, i
   sa = s[Axes<AX>::A];
 }
 
+// Z + 3 values of kappa of a listed column from the axial window's first tap, zero off the design grid.
+// The window is the same for a warp's lanes, so the test for one inside the grid does not diverge.
+template <typename T, int Z>
+__device__ __forceinline__ void load_window(const T* __restrict__ kc, int ia0, int na, int sa, T (&kv)[Z + kPadPts]) {
+  const T* p = kc + (long long)ia0 * sa;
+  if (ia0 >= 0 && ia0 + Z + kPadPts <= na) {
+#pragma unroll
+    for (int m = 0; m < Z + kPadPts; ++m) kv[m] = __ldg(p + m * sa);
+  } else {
+#pragma unroll
+    for (int m = 0; m < Z + kPadPts; ++m) kv[m] = (ia0 + m >= 0 && ia0 + m < na) ? __ldg(p + m * sa) : T(0);
+  }
+}
+
 // Sums of ZC planes of one in-plane position: phi, kappa, P = sum W l, L = sum W kappa l (in the plane).
 template <typename T, int Z>
 struct PlaneSums {
@@ -178,16 +196,21 @@ __device__ __forceinline__ void plane_sums(const Geo& g, const T* __restrict__ k
   T f2 = T(0), pb2 = T(0), pc2 = T(0);
 #pragma unroll
   for (int j = 0; j < Z; ++j) o.phi[j] = o.kap[j] = o.Pb[j] = o.Pc[j] = o.Lb[j] = o.Lc[j] = T(0);
+  auto column_at = [&](unsigned e) { return kref + (int)(e & 0xffffu) * sb + (int)(e >> 16) * sc; };
+  // the next column's kappa is loaded while this one's is used
+  T kn[Z + kPadPts];
+  unsigned en = n > 0 ? list[0][lane] : 0;
+  if (n > 0) load_window<T, Z>(column_at(en), ax.ia0, g.nd[a], sa, kn);
   for (int i = 0; i < n; ++i) {
-    const Column<T, AX> q(g, list[i][lane], xib, xic, cs, sn, d);
-    const T w2 = wfun(g.wk, q.ob) * wfun(g.wk, q.oc);
-    const T* kc = kref + q.ib * sb + q.ic * sc;
+    const Column<T, AX> q(g, en, xib, xic, cs, sn, d);
     T kv[Z + kPadPts];
 #pragma unroll
-    for (int m = 0; m < Z + kPadPts; ++m) {
-      const int ia = ax.ia0 + m;
-      kv[m] = (ia >= 0 && ia < g.nd[a]) ? __ldg(kc + (long long)ia * sa) : T(0);
+    for (int m = 0; m < Z + kPadPts; ++m) kv[m] = kn[m];
+    if (i + 1 < n) {
+      en = list[i + 1][lane];
+      load_window<T, Z>(column_at(en), ax.ia0, g.nd[a], sa, kn);
     }
+    const T w2 = wfun(g.wk, q.ob) * wfun(g.wk, q.oc);
     const T wb = w2 * q.lb, wc = w2 * q.lc;
     int left = 0;
     if (BALL) left = g.rad4 - dsq(q.ib, g.nd[b]) - dsq(q.ic, g.nd[c]);
@@ -229,6 +252,54 @@ __device__ __forceinline__ void plane_sums(const Geo& g, const T* __restrict__ k
       o.Pc[j] = pc2 * s1;
     }
 }
+
+// Grid indices of a lane's Z cells: the in-plane part once, the axial one stepped (wrapped on a periodic
+// axis). ok: bit j set if cell j is in the box and on the grid; forb: it may not be touched by the body.
+template <int AX, int Z>
+struct LaneCells {
+  long long n0;
+  int pa, na, sa;  // first axial coordinate (wrapped if periodic), extent, stride
+  unsigned box, ok, forb;
+  bool per;
+  __device__ __forceinline__ LaneCells(const Geo& g, const int (&lo)[3], const LanePos& lp) {
+    constexpr int b = Axes<AX>::B, c = Axes<AX>::C, a = Axes<AX>::A;
+    const int st[3] = {1, g.n[0], g.n[0] * g.n[1]};
+    bool in = lp.ok, fb = false;
+    n0 = 0;
+#pragma unroll
+    for (int e = 0; e < 3; ++e) {
+      if (e == a) continue;
+      int p = lo[e] + lp.j[e];
+      if (g.bc[e] == BC_PERIODIC) {
+        p = wrapi(p, g.n[e]);
+      } else {
+        fb = fb || p < 2 || p > g.n[e] - 3;
+        in = in && p >= 0 && p < g.n[e];
+      }
+      n0 += (long long)p * st[e];
+    }
+    per = g.bc[a] == BC_PERIODIC;
+    na = g.n[a];
+    sa = st[a];
+    pa = lo[a] + lp.j[a];
+    if (per) pa = wrapi(pa, na);
+    box = ok = forb = 0;
+#pragma unroll
+    for (int j = 0; j < Z; ++j) {
+      const bool ib = lp.ok && lp.j[a] + j < g.B[a];
+      if (ib) box |= 1u << j;
+      if (ib && in && (per || (pa + j >= 0 && pa + j < na))) ok |= 1u << j;
+      if (fb || (!per && (pa + j < 2 || pa + j > na - 3))) forb |= 1u << j;
+    }
+    (void)b;
+    (void)c;
+  }
+  __device__ __forceinline__ long long at(int j) const {
+    int p = pa + j;
+    if (per && p >= na) p -= na;  // (the box fits the axis, so a chunk wraps at most once)
+    return n0 + (long long)p * sa;
+  }
+};
 
 // us of a cell from its sums.
 template <typename T, int AX, typename U>
@@ -295,33 +366,41 @@ __global__ void __launch_bounds__(512, 1)
       const int n = column_list<T, AX>(g, d, P.cs, P.sn, lp.ok, list, lane);
       PlaneSums<T, Z> A;
       plane_sums<T, AX, BALL, Z>(g, kref, d, P.cs, P.sn, n, list, lane, A);
-      if (!lp.ok) continue;
+      const LaneCells<AX, Z> lc(g, lo, lp);
+      unsigned work = 0;  // cells the body reaches (the others keep u = u*)
+#pragma unroll
+      for (int j = 0; j < Z; ++j)
+        if (A.phi[j] > T(0)) work |= 1u << j;
+      if (work & (lc.forb | (lc.box & ~lc.ok))) atomicOr(&ctrl->status, ST_BODY_OUTSIDE);
+      work &= lc.ok;
+      const unsigned stored = last && bs ? lc.ok : work;
+      const long long bl0 = lp.j[0] + (long long)g.B[0] * (lp.j[1] + (long long)g.B[1] * lp.j[2]);
+      const int sbx = a3 == 0 ? 1 : (a3 == 1 ? g.B[0] : g.B[0] * g.B[1]);
+      T us[Z][3];
+#pragma unroll
+      for (int j = 0; j < Z; ++j)
+#pragma unroll
+        for (int a = 0; a < 3; ++a) us[j][a] = (stored >> j & 1u) ? dst[(a + 1) * N + lc.at(j)] : T(0);
 #pragma unroll
       for (int j = 0; j < Z; ++j) {
-        int jj[3] = {lp.j[0], lp.j[1], lp.j[2]};
-        jj[a3] += j;
-        if (jj[a3] >= g.B[a3]) continue;
-        if (A.phi[j] == T(0) && !(last && bs)) continue;  // no design point in reach: u = u*
-        const int px = lo[0] + jj[0], py = lo[1] + jj[1], pz = lo[2] + jj[2];
-        long long m;
-        const bool ing = cell_index<3>(g, px, py, pz, m);
-        if (A.phi[j] > T(0) && (!ing || forbidden<3>(g, px, py, pz))) atomicOr(&ctrl->status, ST_BODY_OUTSIDE);
-        if (!ing) continue;
         const T inv = T(1) / (T(1) + A.kap[j]);
-        const long long bl = jj[0] + (long long)g.B[0] * (jj[1] + (long long)g.B[1] * jj[2]);
         T uu[3];
 #pragma unroll
         for (int a = 0; a < 3; ++a) {
-          const T us = solid_velocity<T, AX>(a, P.ug, P.om, A.phi[j], A.Pb[j], A.Pc[j]);
-          const T ustar = dst[(a + 1) * N + m];
-          uu[a] = (ustar + A.kap[j] * us) * inv;
-          run_add(v[a], A.kap[j] * uu[a]);
-          if (last) {
-            if (bs) bs[a * g.box_cells + bl] = ustar;
-            dst[(a + 1) * N + m] = uu[a];
-          }
+          const T sv = solid_velocity<T, AX>(a, P.ug, P.om, A.phi[j], A.Pb[j], A.Pc[j]);
+          uu[a] = (us[j][a] + A.kap[j] * sv) * inv;
         }
-        run_add(v[3], A.Lb[j] * uu[c] - A.Lc[j] * uu[b]);
+        if (work >> j & 1u) {
+#pragma unroll
+          for (int a = 0; a < 3; ++a) run_add(v[a], A.kap[j] * uu[a]);
+          run_add(v[3], A.Lb[j] * uu[c] - A.Lc[j] * uu[b]);
+          if (last)
+#pragma unroll
+            for (int a = 0; a < 3; ++a) dst[(a + 1) * N + lc.at(j)] = uu[a];
+        }
+        if (last && bs && (stored >> j & 1u))
+#pragma unroll
+          for (int a = 0; a < 3; ++a) bs[a * g.box_cells + bl0 + (long long)j * sbx] = us[j][a];
       }
     }
     __syncwarp();
@@ -360,21 +439,24 @@ __global__ void __launch_bounds__(kApplyWarps * 32) k_apply_axis3d(Geo g, Slots<
   const int n = column_list<T, AX>(g, d, P.cs, P.sn, lp.ok, lists[warp], lane);
   PlaneSums<T, Z> A;
   plane_sums<T, AX, BALL, Z>(g, kref, d, P.cs, P.sn, n, lists[warp], lane, A);
-  if (!lp.ok) return;
+  const LaneCells<AX, Z> lc(g, lo, lp);
+  const long long bl0 = lp.j[0] + (long long)g.B[0] * (lp.j[1] + (long long)g.B[1] * lp.j[2]);
+  const int sbx = a3 == 0 ? 1 : (a3 == 1 ? g.B[0] : g.B[0] * g.B[1]);
+  T us[Z][3];
+#pragma unroll
+  for (int j = 0; j < Z; ++j)
+#pragma unroll
+    for (int a = 0; a < 3; ++a) us[j][a] = (lc.ok >> j & 1u) ? dst[(a + 1) * g.N + lc.at(j)] : T(0);
 #pragma unroll
   for (int j = 0; j < Z; ++j) {
-    int jj[3] = {lp.j[0], lp.j[1], lp.j[2]};
-    jj[a3] += j;
-    long long m;
-    if (jj[a3] >= g.B[a3] || !cell_index<3>(g, lo[0] + jj[0], lo[1] + jj[1], lo[2] + jj[2], m)) continue;
+    if (!(lc.ok >> j & 1u)) continue;
     const T inv = T(1) / (T(1) + A.kap[j]);
-    const long long bl = jj[0] + (long long)g.B[0] * (jj[1] + (long long)g.B[1] * jj[2]);
+    const bool body = A.phi[j] > T(0);
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
-      const T us = solid_velocity<T, AX>(a, P.ug, P.om, A.phi[j], A.Pb[j], A.Pc[j]);
-      const T ustar = dst[(a + 1) * g.N + m];
-      bs[a * g.box_cells + bl] = ustar;
-      dst[(a + 1) * g.N + m] = (ustar + A.kap[j] * us) * inv;
+      const T sv = solid_velocity<T, AX>(a, P.ug, P.om, A.phi[j], A.Pb[j], A.Pc[j]);
+      bs[a * g.box_cells + bl0 + (long long)j * sbx] = us[j][a];
+      if (body) dst[(a + 1) * g.N + lc.at(j)] = (us[j][a] + A.kap[j] * sv) * inv;
     }
   }
 }
@@ -423,18 +505,22 @@ __global__ void __launch_bounds__(kRevThreads) k_coef_axis3d(Geo g, const Ctrl* 
       for (int e = 0; e < 4; ++e) s[j][e][0] = s[j][e][1] = s[j][e][2] = T(0);
       sq[j][0] = sq[j][1] = T(0);
     }
+    auto column_at = [&](unsigned e) { return kref + (int)(e & 0xffffu) * sb + (int)(e >> 16) * sc; };
+    T kn[Z + kPadPts];
+    unsigned en = n > 0 ? list[0][lane] : 0;
+    if (n > 0) load_window<T, Z>(column_at(en), ax.ia0, g.nd[a3], sa, kn);
     for (int q0 = 0; q0 < n; ++q0) {
-      const Column<T, AX> q(g, list[q0][lane], xib, xic, P.cs, P.sn, d);
+      const Column<T, AX> q(g, en, xib, xic, P.cs, P.sn, d);
+      T kv[Z + kPadPts];
+#pragma unroll
+      for (int m = 0; m < Z + kPadPts; ++m) kv[m] = kn[m];
+      if (q0 + 1 < n) {
+        en = list[q0 + 1][lane];
+        load_window<T, Z>(column_at(en), ax.ia0, g.nd[a3], sa, kn);
+      }
       T wb, dwb, wc, dwc;
       w_dw(g.wk, -q.ob, &wb, &dwb);
       w_dw(g.wk, -q.oc, &wc, &dwc);
-      const T* kc = kref + q.ib * sb + q.ic * sc;
-      T kv[Z + kPadPts];
-#pragma unroll
-      for (int m = 0; m < Z + kPadPts; ++m) {
-        const int ia = ax.ia0 + m;
-        kv[m] = (ia >= 0 && ia < g.nd[a3]) ? __ldg(kc + (long long)ia * sa) : T(0);
-      }
       const T w[3] = {wb * wc, dwb * wc, wb * dwc};
       const T rt = w[1] * q.lc - w[2] * q.lb, rb = rt * q.lb, rc = rt * q.lc;
       T wl[3][2];
@@ -573,26 +659,38 @@ __global__ void __launch_bounds__(128) k_design_axis3d(Geo g, Ctrl* ctrl, const 
     T sum[Z][4];  // u, dJ/dkappa_n
 #pragma unroll
     for (int j = 0; j < Z; ++j) sum[j][0] = sum[j][1] = sum[j][2] = sum[j][3] = T(0);
-#pragma unroll 1
-    for (int qc = 0; qc < S2; ++qc) {
+    const int top = min(np + S2 - 1, g.B[a3] - f[a3]);  // planes of the window that are read
+    auto weight = [&](int q2) {  // in-plane weight of window cell q2 = qb + S2 qc
+      const int qc = q2 / S2, qb = q2 - qc * S2;
       const T wc = qc == 0 ? w[c][0] : (qc == 1 ? w[c][1] : (qc == 2 ? w[c][2] : w[c][3]));
+      return wc * (qb == 0 ? w[b][0] : (qb == 1 ? w[b][1] : (qb == 2 ? w[b][2] : w[b][3])));
+    };
+    auto load = [&](int q2, int fl, bool on, T (&x)[Z + kPadPts]) {
+      const int qc = q2 / S2, qb = q2 - qc * S2;
+      const T* F = Pk + (fl < 3 ? RP::u + fl : RP::eps) * BC + (o0 + qb * st[b] + qc * st[c]);
+#pragma unroll
+      for (int m = 0; m < Z + kPadPts; ++m) x[m] = on && m < top ? __ldg(F + m * st[a3]) : T(0);
+    };
+    // each field's values are loaded while the one before is used
+    T w2 = weight(0), wn = T(0), x[Z + kPadPts], xn[Z + kPadPts];
+    load(0, 0, w2 != T(0), x);
 #pragma unroll 1
-      for (int qb = 0; qb < S2; ++qb) {
-        const T w2 = wc * (qb == 0 ? w[b][0] : (qb == 1 ? w[b][1] : (qb == 2 ? w[b][2] : w[b][3])));
-        if (w2 == T(0)) continue;
-        const int o1 = o0 + qb * st[b] + qc * st[c];
+    for (int q2 = 0; q2 < S2 * S2; ++q2) {
+      const bool more = q2 + 1 < S2 * S2;
+      wn = more ? weight(q2 + 1) : T(0);
 #pragma unroll
-        for (int fl = 0; fl < 4; ++fl) {
-          const T* F = Pk + (fl < 3 ? RP::u + fl : RP::eps) * BC + o1;
-          T x[Z + kPadPts];
+      for (int fl = 0; fl < 4; ++fl) {
+        if (fl < 3)
+          load(q2, fl + 1, w2 != T(0), xn);
+        else
+          load(more ? q2 + 1 : q2, 0, wn != T(0), xn);
 #pragma unroll
-          for (int m = 0; m < Z + kPadPts; ++m)
-            x[m] = (m < np + S2 - 1 && f[a3] + m < g.B[a3]) ? __ldg(F + m * st[a3]) : T(0);
+        for (int j = 0; j < Z; ++j)
+          sum[j][fl] += w2 * (w[a3][0] * x[j] + w[a3][1] * x[j + 1] + w[a3][2] * x[j + 2] + w[a3][3] * x[j + 3]);
 #pragma unroll
-          for (int j = 0; j < Z; ++j)
-            sum[j][fl] += w2 * (w[a3][0] * x[j] + w[a3][1] * x[j + 1] + w[a3][2] * x[j + 2] + w[a3][3] * x[j + 3]);
-        }
+        for (int m = 0; m < Z + kPadPts; ++m) x[m] = xn[m];
       }
+      w2 = wn;
     }
     const T* lam = lamh + ((long long)i * K + (k - 1)) * 4;
 #pragma unroll

@@ -585,8 +585,8 @@ size_t reverse_layout(const Geo& g, bool fp64, int max_steps, RevBuffers* R) {
   R->steps = (int)(want < 1 ? 1 : (want < max_steps ? want : max_steps));
   if (R->steps > 64) R->steps = 64;
   // splits of the design kernel over the chunk's steps (3D: steps and iterations): about 2^17 threads in
-  // 2D, 2^15 of the 3D form's, each of which takes eight points
-  long long sp = D == 2 ? (1LL << 17) / ((long long)g.ND * LN) : (1LL << 18) / g.ND;
+  // 2D, 2^17 of the 3D form's, each of which takes eight points
+  long long sp = D == 2 ? (1LL << 17) / ((long long)g.ND * LN) : (1LL << 20) / g.ND;
   sp = sp < 1 ? 1 : (sp > 16 ? 16 : sp);
   const long long items = D == 2 ? R->steps : R->steps * K;
   R->splits = (int)(sp < items ? sp : items);
