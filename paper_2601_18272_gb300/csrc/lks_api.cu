@@ -25,6 +25,7 @@
 #include <vector>
 
 #include "../../include/lks.h"
+#include "lks_free.cuh"
 #include "lks_geo.h"
 #include "lks_kernels.h"
 
@@ -1039,6 +1040,8 @@ int lks_create(const lks_problem* P, lks_handle** out) {
     lks_destroy(h);
     return r;
   }
+  h->g.free_tiled = g.ax == AX_FREE && h->prec == LKS_FP32 && g.wk == W_COS4 && prepare_free3d() ? 1 : 0;
+  cudaGetLastError();
   refresh_box(h);  // the default state starts unrotated: always fits
   *out = h;
   return LKS_OK;

@@ -33,6 +33,7 @@
 #include <climits>
 
 #include "lks_body_common.cuh"
+#include "lks_free.cuh"
 #include "lks_wait.cuh"
 
 namespace lks {
@@ -1366,6 +1367,9 @@ void launch_apply(const Geo& g, const Slots<T>& S, const Ctrl* ctrl, const Dof* 
 template <typename T>
 void launch_adj_cell(const Geo& g, const Ctrl* ctrl, const Dof* it, const T* kref, const T* boxstore, int nbox, T* Lb,
                      long long lstride, T* acc, T* scratch, int k, int di, cudaStream_t st) {
+  if constexpr (sizeof(T) == 4)
+    if (g.free_tiled)
+      return launch_adj_cell_free(g, ctrl, it, kref, boxstore, nbox, Lb, lstride, acc, scratch, k, di, st);
   LKS_BOX_DISPATCH(k_adj_cell, box_grid(g), box_threads(g), g, ctrl, it, kref, boxstore, nbox, Lb, lstride, acc,
                    scratch, k, di);
 }
@@ -1373,8 +1377,16 @@ void launch_adj_cell(const Geo& g, const Ctrl* ctrl, const Dof* it, const T* kre
 template <typename T>
 void launch_adj_design(const Geo& g, Ctrl* ctrl, const Dof* it, const T* kref, const T* scratch, double* dkref,
                        void* partials, int k, int di, cudaStream_t st) {
-  const unsigned nb = (unsigned)design_ctas(g);
-  LKS_BOX_DISPATCH(k_adj_design, nb, kDesignBlock, g, ctrl, it, kref, scratch, dkref, partials, k, di);
+  unsigned nb = (unsigned)design_ctas(g);
+  bool done = false;
+  if constexpr (sizeof(T) == 4) {
+    if (g.free_tiled) {
+      nb = (unsigned)free_design_ctas(g);
+      launch_adj_design_free(g, ctrl, it, kref, scratch, dkref, partials, k, di, st);
+      done = true;
+    }
+  }
+  if (!done) LKS_BOX_DISPATCH(k_adj_design, nb, kDesignBlock, g, ctrl, it, kref, scratch, dkref, partials, k, di);
   if (g.ax == AX_FREE)
     launch(k_design_finish<T, true>, 1, kFinishThreads, 0, st, g, ctrl, it, (const void*)partials, (int)nb, k, di);
   else
