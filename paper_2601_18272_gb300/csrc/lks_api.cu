@@ -304,7 +304,8 @@ struct lks_handle {
   double host_s0[kNdofFree];
   size_t bytes = 0;
   std::vector<void*> allocs;
-  cudaStream_t cap = nullptr;
+  cudaStream_t cap = nullptr, cap2 = nullptr;  // capture streams: the chain, and a branch beside it
+  cudaEvent_t fork_ev = nullptr, coef_ev[2] = {nullptr, nullptr};
   std::map<std::string, cudaGraphExec_t> graphs;
   std::map<std::string, int> graph_kernels;
   bool box_rot_ok = true;  // buffers hold the rotated box
@@ -564,6 +565,58 @@ void enqueue_recompute(lks_handle* h, Launcher& L, const Slots<T>& S, int nsteps
   }
 }
 
+// The reverse by linear maps: chunks of steps, each with its planes and matrices (coef), its chain of
+// steps and its dJ/dkappa^ref (design). Coef depends on the forward only and design on the chunk's
+// chain only, so in a captured graph they run on a branch of their own: coef(c + 2) follows design(c),
+// whose buffers it takes; the chain of c waits for coef(c), design(c) for the chain of c. The chain's
+// kernels are small and bound by latency. (512x256, 200 steps: see lks_reverse.cu.)
+template <typename T>
+void enqueue_rev_steps(lks_handle* h, Launcher& L, const Slots<T>& S, int nsteps) {
+  const Geo& g = h->g;
+  const int per = h->rev.steps, nc = (nsteps + per - 1) / per;
+  auto steps_of = [&](int c) { return std::min(per, nsteps - c * per); };
+  const bool fork = L.capturing && nc > 1;
+  Launcher side = L;
+  side.kernels = 0;
+  if (fork) side.st = h->cap2;
+  Launcher& B = fork ? side : L;  // the branch
+  auto coef = [&](int c) {
+    B.n("adj_cell", 2, [&](cudaStream_t s) {
+      launch_rev_coef<T>(g, h->rev.set(c), h->ctrl, h->it, (const T*)h->kref, h->mom, (const T*)h->boxstore, h->nbox,
+                         steps_of(c), c * per, s);
+    });
+    if (fork) cudaEventRecord(h->coef_ev[c & 1], B.st);
+  };
+  auto design = [&](int c) {
+    B("adj_design", [&](cudaStream_t s) { launch_rev_design<T>(g, h->rev.set(c), h->ctrl, h->it, steps_of(c), c * per, s); });
+  };
+  auto after = [&](cudaStream_t from, cudaStream_t to) {  // what follows on `to` waits for `from`
+    if (!fork) return;
+    cudaEventRecord(h->fork_ev, from);
+    cudaStreamWaitEvent(to, h->fork_ev, 0);
+  };
+  after(L.st, B.st);
+  coef(0);
+  for (int c = 0; c < nc; ++c) {
+    if (fork && c == 0) coef(1);
+    if (fork) cudaStreamWaitEvent(L.st, h->coef_ev[c & 1], 0);
+    const RevBuffers R = h->rev.set(c);
+    for (int i = 0; i < steps_of(c); ++i) {
+      L.n("adj_body", 2, [&](cudaStream_t s) {
+        launch_rev_step<T>(g, R, h->ctrl, h->it, (T*)h->L, h->slot_elems, i, c * per, s);
+      });
+      L("stencil_adj", [&](cudaStream_t s) {
+        launch_stencil_adj<T>(g, S, (T*)h->L, h->slot_elems, h->ctrl, c * per + i, s);
+      });
+    }
+    after(L.st, B.st);
+    design(c);
+    if (c + (fork ? 2 : 1) < nc) coef(c + (fork ? 2 : 1));
+  }
+  after(B.st, L.st);
+  if (fork) L.kernels += side.kernels;
+}
+
 template <typename T>
 void enqueue_adj_steps(lks_handle* h, Launcher& L, const Slots<T>& S, int nsteps) {
   const Geo& g = h->g;
@@ -580,20 +633,7 @@ void enqueue_adj_steps(lks_handle* h, Launcher& L, const Slots<T>& S, int nsteps
     return;
   }
   if (h->rev_on) {
-    const RevBuffers& R = h->rev;
-    for (int c = 0; c < nsteps; c += R.steps) {
-      const int n = std::min(R.steps, nsteps - c);
-      L.n("adj_cell", 2, [&](cudaStream_t s) {
-        launch_rev_coef<T>(g, R, h->ctrl, h->it, (const T*)h->kref, h->mom, (const T*)h->boxstore, h->nbox, n, c, s);
-      });
-      for (int i = 0; i < n; ++i) {
-        L.n("adj_body", 2, [&](cudaStream_t s) {
-          launch_rev_step<T>(g, R, h->ctrl, h->it, (T*)h->L, h->slot_elems, i, c, s);
-        });
-        L("stencil_adj", [&](cudaStream_t s) { launch_stencil_adj<T>(g, S, (T*)h->L, h->slot_elems, h->ctrl, c + i, s); });
-      }
-      L("adj_design", [&](cudaStream_t s) { launch_rev_design<T>(g, R, h->ctrl, h->it, n, c, s); });
-    }
+    enqueue_rev_steps<T>(h, L, S, nsteps);
     return;
   }
   for (int i = 0; i < nsteps; ++i) {
@@ -1030,7 +1070,14 @@ int lks_create(const lks_problem* P, lks_handle** out) {
   const Geo& g = h->g;
   int r = (h->prec == LKS_FP64) ? allocate<double>(h) : allocate<float>(h);
   if (r == LKS_OK) r = set_default_initial_state(h);
-  if (r == LKS_OK && cudaStreamCreateWithFlags(&h->cap, cudaStreamNonBlocking) != cudaSuccess) r = LKS_ERR_CUDA;
+  int low = 0, high = 0;  // the chain's kernels go before the branch's (graph nodes keep the priority)
+  cudaDeviceGetStreamPriorityRange(&low, &high);
+  if (r == LKS_OK && (cudaStreamCreateWithPriority(&h->cap, cudaStreamNonBlocking, high) != cudaSuccess ||
+                      cudaStreamCreateWithPriority(&h->cap2, cudaStreamNonBlocking, low) != cudaSuccess ||
+                      cudaEventCreateWithFlags(&h->fork_ev, cudaEventDisableTiming) != cudaSuccess ||
+                      cudaEventCreateWithFlags(&h->coef_ev[0], cudaEventDisableTiming) != cudaSuccess ||
+                      cudaEventCreateWithFlags(&h->coef_ev[1], cudaEventDisableTiming) != cudaSuccess))
+    r = LKS_ERR_CUDA;
   if (r == LKS_OK && g.dim == 3) {
     if (h->prec == LKS_FP64) prepare_stencil3d<double>();
     else prepare_stencil3d<float>();
@@ -1461,6 +1508,9 @@ void lks_destroy(lks_handle* h) {
   for (void* p : h->allocs) cudaFree(p);
   cudaFree(h->rev.block);
   if (h->cap) cudaStreamDestroy(h->cap);
+  if (h->cap2) cudaStreamDestroy(h->cap2);
+  for (cudaEvent_t e : {h->fork_ev, h->coef_ev[0], h->coef_ev[1]})
+    if (e) cudaEventDestroy(e);
   delete h;
 }
 

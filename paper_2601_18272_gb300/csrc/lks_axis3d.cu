@@ -795,8 +795,12 @@ bool axis3d_fits(const Geo& g) {
          g.box_cells < (1LL << 29);
 }
 
+// Small boxes leave each SM one warp, whose list and window loads then make the iteration's time: up to
+// 40,000 cells (FP64, where the per-iteration kernels are slower per cell, 10,000) those are as fast or
+// faster. Forward us per step at 5 iterations, per-iteration -> this: FP32 18^3 cells 85 -> 91, 32^3 99 ->
+// 99, 52 x 52 x 38 178 -> 114, 56^3 248 -> 108; FP64 20^3 635 -> 700, 28 x 28 x 22 936 -> 626.
 void setup_couple_axis3d(Geo* g, bool fp64) {
-  if (!axis3d_fits(*g)) return;
+  if (!axis3d_fits(*g) || g->box_cells <= (fp64 ? 10000 : 40000)) return;
   if (fp64)
     shape_any<double>(g);
   else

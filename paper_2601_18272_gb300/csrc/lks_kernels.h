@@ -2,6 +2,8 @@
 // include/lks.h).
 #pragma once
 
+#include <initializer_list>
+
 #include "lks_device.cuh"
 
 namespace lks {
@@ -176,6 +178,15 @@ struct RevBuffers {
   long long slab = 0;  // values per step's slab
   int steps = 0;       // slabs: steps per chunk
   int splits = 0;      // partial dJ/dkappa^ref of the design kernel
+  // a second set of the chunk's buffers (slabs, mpart, mats, lamh): the next chunk's planes are made and
+  // the last one's dJ/dkappa^ref is summed beside the chain of this one
+  size_t other = 0;    // bytes from a buffer of the first set to its twin
+  RevBuffers set(int i) const {
+    RevBuffers r = *this;
+    if (i & 1)
+      for (void** q : {&r.slabs, &r.mpart, &r.mats, &r.lamh}) *q = (char*)*q + other;
+    return r;
+  }
 };
 bool reverse_affine_fits(const Geo& g);
 size_t reverse_layout(const Geo& g, bool fp64, int max_steps, RevBuffers* R);

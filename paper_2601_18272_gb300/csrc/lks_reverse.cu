@@ -27,7 +27,8 @@
 // What it replaces: 3 N_itr dependent launches a step (cell, design and one-CTA finish kernel per
 // iteration), bound by their latency on 2D boxes (about 5 us each for 35 k cells) and in FP64 by the
 // few warps a small box gives each launch. Only k_rev_const, k_rev_apply and the transposed stencil
-// are left in a step's chain; the rest runs over whole chunks of steps. Gradients measured on GB300,
+// are left in a step's chain; the rest runs over whole chunks of steps, on a branch of its own beside the
+// chain (lks_api.cu: that took the gradients below by another 2 % (2D, small body) to 8 % (3D)). Gradients measured on GB300,
 // before -> after: 512x256 / 128^2, 200 steps 30.2 -> 21.1 ms; 1024x512 / 256^2, 100 steps 30.2 -> 22.3
 // ms; 80x40 / 16^2 FP64, 400 steps 256 -> 135 ms; 128x64x64 / 48^3, 40 steps 26.3 -> 21.9 ms.
 #include <algorithm>
@@ -579,11 +580,10 @@ size_t reverse_layout(const Geo& g, bool fp64, int max_steps, RevBuffers* R) {
   long long nc = (g.box_cells + kRevThreads - 1) / kRevThreads;
   if (D == 3 && coef_axis3d_fits(g)) nc = std::max(nc, (long long)coef_axis3d_ctas(g, fp64));
   R->slab = planes * g.box_cells;
-  // steps per chunk: as many slabs as about half of the L2 holds, so that the planes written by one
-  // kernel are read from L2 by the next; at least one, at most the segment
-  const long long want = (64LL << 20) / (R->slab * esz);
-  R->steps = (int)(want < 1 ? 1 : (want < max_steps ? want : max_steps));
-  if (R->steps > 64) R->steps = 64;
+  // steps per chunk: two chunks' slabs in about half of the L2, so that the planes written by one kernel
+  // are read from L2 by the next; at least one, and several chunks a segment to overlap them
+  const long long want = (32LL << 20) / (R->slab * esz), part = (max_steps + 3) / 4;
+  R->steps = (int)std::max(1LL, std::min({want, part, 64LL}));
   // splits of the design kernel over the chunk's steps (3D: steps and iterations): about 2^17 threads in
   // 2D, 2^17 of the 3D form's, each of which takes eight points
   long long sp = D == 2 ? (1LL << 17) / ((long long)g.ND * LN) : (1LL << 20) / g.ND;
@@ -599,8 +599,10 @@ size_t reverse_layout(const Geo& g, bool fp64, int max_steps, RevBuffers* R) {
   const size_t slabs = take(R->steps * R->slab * esz);
   const size_t mpart = take(R->steps * K * nc * nm * 8);
   const size_t mats = take(R->steps * K * (long long)sizeof(RevMat));
-  const size_t cpart = take((long long)kRevMaxCtas * 8 * 8);
   const size_t lamh = take(R->steps * K * 4 * esz);
+  R->other = off;
+  off *= 2;
+  const size_t cpart = take((long long)kRevMaxCtas * 8 * 8);
   const size_t dkp = take((long long)R->splits * g.ND * 8);
   if (R->block) {
     char* p = (char*)R->block;

@@ -40,6 +40,8 @@ def _cases():
                           bc=(BC_INFLOW_OUTFLOW, BC_WALL, BC_WALL)), 0.3, 0.002, 0.0
     yield "ball", body3d(nx=28, ny=27, nz=26, nd=11, centre=(12.6, 12.2, 12.9), rot_axis=1, nt=2), 0.4, 0.002, 4.0
     yield "large", body3d(nx=84, ny=79, nz=66, nd=41, centre=(40.3, 39.1, 32.6), rot_axis=2, nt=2, n_itr=2), 0.6, 1e-4, 0.0
+    yield "large-axis0", body3d(nx=66, ny=84, nz=79, nd=39, centre=(32.6, 40.3, 39.1), rot_axis=0, nt=2, n_itr=2), 0.6, 1e-4, 0.0
+    yield "large-ball", body3d(nx=84, ny=66, nz=79, nd=41, centre=(40.3, 32.6, 39.1), rot_axis=1, nt=2, n_itr=2), 0.6, 1e-4, 17.2
 
 
 CASES = list(_cases())
