@@ -19,6 +19,8 @@
 //
 // Algorithmic traffic per cell: read p, u (3 values), write p*, u* (3 values): 24 B in FP32;
 // the transpose reads the adjoint (3) and u(t-1) (2) and writes 3 values: 32 B.
+#include <algorithm>
+
 #include "lks_kernels.h"
 #include "lks_stencil_common.cuh"
 
@@ -822,18 +824,20 @@ __global__ void __launch_bounds__(SW * 32) k_stencil2d_adj(Geo g, Slots<T> S, T*
 
 // Column tiles and row strips: W output columns per warp (60, or a little less so that the
 // columns nx-2 and nx-1 of a non-periodic x axis share a warp; always even so column pairs start
-// on an even column), strips of rows sized so the grid has about 32 warps per SM scheduler (short
-// strips recompute two halo rows each, but more warps hide the shuffle and shared-memory
-// latencies; measured on 8192x4096, predictor / transpose in % of HBM: 8 warps 59 / 50, 16 warps
-// 71 / 65, 32 warps 76 / 72, 48 warps 74 / 73). Small grids are capped by the two-row minimum.
-StripPlan plan_strips(const Geo& g) {
+// on an even column). Strips: short ones recompute halo rows (L + 4 rows for L), few ones leave the
+// shuffle and shared-memory latencies uncovered. FP32: 14 rows, within 8 to 32 warps per SM scheduler.
+// Measured, predictor / transpose in us at 8, 16, 32 warps per scheduler: 2048x1024 21 / 32, 22 / 35,
+// 28 / 44; 3000x1500 34 / 54, 34 / 52, 41 / 60; 4096x2048 59 / 89, 53 / 78, 58 / 80; 8192x4096 197 / 313,
+// 165 / 242, 154 / 217. FP64: 32 warps. Small grids are capped by the two-row minimum.
+StripPlan plan_strips(const Geo& g, bool fp64) {
   StripPlan sp;
   sp.W = 60;
   if (g.bc[0] != BC_PERIODIC)
     while ((g.n[0] - 1) % sp.W == 0) sp.W -= 2;
   sp.ntx = (g.n[0] + sp.W - 1) / sp.W;
-  const int want = 32 * 152 * 4;  // warps
-  int ns = (want + sp.ntx - 1) / sp.ntx;
+  const int sched = 152 * 4;
+  int ns = (32 * sched + sp.ntx - 1) / sp.ntx;
+  if (!fp64) ns = std::max(8 * sched / sp.ntx, std::min(ns, g.n[1] / 14));
   const int maxs = g.n[1] / 2;  // at least two rows per strip (a wall row is built from the next)
   if (ns > maxs) ns = maxs;
   sp.nstrip = ns < 1 ? 1 : ns;
@@ -849,7 +853,7 @@ bool vec_ok(const Geo& g) { return g.n[0] % 2 == 0; }
 template <typename T>
 void launch_stencil_fwd(const Geo& g, const Slots<T>& S, const Ctrl* ctrl, int di, cudaStream_t st) {
   if (g.dim == 2) {
-    const StripPlan sp = plan_strips(g);
+    const StripPlan sp = plan_strips(g, sizeof(T) == 8);
     if (stencil_tile_pays(g, g.n[1] / sp.nstrip, sizeof(T) == 8, false)) return launch_stencil_tile_fwd<T>(g, S, ctrl, di, st);
     const int warps = sp.ntx * sp.nstrip;
     const size_t smem = Ring<T>::bytes(3);
@@ -866,7 +870,7 @@ template <typename T>
 void launch_stencil_adj(const Geo& g, const Slots<T>& S, T* Lb, long long lstride, const Ctrl* ctrl, int di,
                         cudaStream_t st) {
   if (g.dim == 2) {
-    const StripPlan sp = plan_strips(g);
+    const StripPlan sp = plan_strips(g, sizeof(T) == 8);
     if (stencil_tile_pays(g, g.n[1] / sp.nstrip, sizeof(T) == 8, true)) return launch_stencil_tile_adj<T>(g, S, Lb, lstride, ctrl, di, st);
     const int warps = sp.ntx * sp.nstrip;
     const size_t smem = Ring<T>::bytes(5);

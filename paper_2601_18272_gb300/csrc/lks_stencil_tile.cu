@@ -259,12 +259,13 @@ void adj_shape(const Geo& g, const Slots<T>& S, T* Lb, long long lstride, const 
 
 // Tiles pay while the strips of the other form are short: a strip of L rows works on L + 4. FP64
 // (instruction count decides): below 12 rows; 600x100 predictor / transpose 24 / 41 -> 17 / 18 us,
-// 80x40 25 / 42 -> 7 / 7. FP32: the transpose below 6 rows (512x256 11 -> 7, 1024x512 19 -> 15 us); the
-// predictor's shorter chain loses only on small grids (512x256 7 -> 6, but 1024x512 12.5 -> 13 us).
-// (Events around each launch, less their 3.5 us.)
+// 80x40 25 / 42 -> 7 / 7. FP32 (the tile's loads cost more): only where strips have two or three rows,
+// and the predictor, whose chain is shorter, only on the smallest grids: 512x256 7 / 11 -> 6 / 7,
+// 1024x512 12.4 / 18 -> 13 / 13.5, 2048x1024 21 / 32 -> 40 / 44 us. (Events around each launch, less
+// their 3.5 us.)
 bool stencil_tile_pays(const Geo& g, int rows, bool fp64, bool transpose) {
   if (fp64) return rows < 12;
-  return rows < 6 && (transpose || g.N <= (1LL << 18));
+  return rows < 4 && g.N <= (transpose ? 1LL << 20 : 1LL << 18);
 }
 
 template <typename T>

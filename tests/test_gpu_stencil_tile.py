@@ -56,7 +56,7 @@ def test_tiles_match_oracle(nx, ny, bx, by):
 def test_strips_match_tiles():
     kw = dict(nd=10, nt=5, n_itr=3, bc=(PER, PER, PER))
     P, g = body2d(nx=96, ny=80, centre=(48.3, 40.2), **kw)
-    Q, _ = body2d(nx=3702, ny=2001, centre=(1848.3, 1000.2), **kw)  # rows of 6.4 per strip
+    Q, _ = body2d(nx=3702, ny=2001, centre=(1848.3, 1000.2), **kw)  # strips of 14 rows
     a, b = _gradient(P, g, None, 32), _gradient(Q, g, None, 32)
     assert _rel(b[1], a[1]) < 2e-4
     np.testing.assert_allclose(b[2][:, 3:], a[2][:, 3:], rtol=0, atol=2e-5 * np.abs(a[2][:, 3:]).max())
