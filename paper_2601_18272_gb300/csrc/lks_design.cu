@@ -15,6 +15,7 @@
 // symmetric, so this is the same gather as the filter applied to v2 / W) -> out_m = sum of v1 over
 // m's orbit when m is its own representative, else 0. Every output is one thread's fixed-order sum.
 #include <climits>
+#include <cmath>
 
 #include "lks_kernels.h"
 
@@ -70,40 +71,37 @@ __global__ void __launch_bounds__(kDB) k_expand(Geo g, const double* __restrict_
 }
 
 // Filter weights by squared distance, (R - sqrt(d2)) / R up to R (beyond: -1), and the weights' sum
-// over a whole disc, made once per block: the square root and the division took most of the
-// filter's FP64 instructions (each costs a warp 64 cycles) when every pair of points computed its own
-// (lks_constraint with its gradient on a 256^2 design, R = 3, with projection and cyclic order 4:
-// 350 -> 111 us, with the volume's sum in a cluster and one wait at the end).
-// Radii whose table would not fit keep that form.
-constexpr int kTab = 2048;
-// Table entries for radius R: every squared distance up to R^2, one more for its rounding.
-__device__ __forceinline__ int tab_size(double R) { return R < 1000.0 ? (int)floor(R * R) + 2 : INT_MAX; }
+// over a whole disc in the order of filter_sum. The square root and the division took most of the
+// filter's FP64 instructions (each costs a warp 64 cycles) when every pair of points computed its own;
+// the host makes the table (the same IEEE operations) and passes it as an argument, whose uniform index
+// costs no shared load (lks_constraint with its gradient on a 256^2 design, R = 3, with projection and
+// cyclic order 4: 350 us per pair, 111 with a table per block, which each block waited for, 96 so). Radii whose
+// table does not fit compute each pair's.
+constexpr int kTab = 128;
 struct FilterTab {
-  double w[kTab];
-  double full;  // sum over the whole disc, in the order of filter_sum
+  int n;  // entries (0: no table)
+  double full, w[kTab];
 };
-__device__ __forceinline__ double filter_weight(double R, int d2) {
+__host__ __device__ inline double filter_weight(double R, int d2) {
   const double dist = sqrt((double)d2);
   return dist > R ? -1.0 : (R - dist) / R;
 }
-// All threads of the block call it; a block barrier follows it.
-__device__ __forceinline__ void make_table(const Geo& g, FilterTab& tab) {
-  const int rr = (int)floor(g.frad), n = tab_size(g.frad);
-  if (g.frad > 0.0 && n <= kTab) {
-    for (int d2 = threadIdx.x; d2 < n; d2 += kDB) tab.w[d2] = filter_weight(g.frad, d2);
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      double w = 0.0;
-      const int ez = (g.dim == 3) ? rr : 0;
-      for (int dz = -ez; dz <= ez; ++dz)
-        for (int dy = -rr; dy <= rr; ++dy)
-          for (int dx = -rr; dx <= rr; ++dx) {
-            const int d2 = dx * dx + dy * dy + dz * dz;
-            if (d2 < n && tab.w[d2] >= 0.0) w += tab.w[d2];
-          }
-      tab.full = w;
-    }
-  }
+FilterTab make_table(const Geo& g) {
+  FilterTab t;
+  t.n = 0;
+  t.full = 0.0;
+  const double R = g.frad;
+  if (!(R > 0.0) || R * R + 2.0 > (double)kTab) return t;
+  const int rr = (int)std::floor(R), ez = g.dim == 3 ? rr : 0;
+  t.n = (int)std::floor(R * R) + 2;  // every squared distance up to R^2, one more for its rounding
+  for (int d2 = 0; d2 < t.n; ++d2) t.w[d2] = filter_weight(R, d2);
+  for (int dz = -ez; dz <= ez; ++dz)
+    for (int dy = -rr; dy <= rr; ++dy)
+      for (int dx = -rr; dx <= rr; ++dx) {
+        const int d2 = dx * dx + dy * dy + dz * dz;
+        if (d2 < t.n && t.w[d2] >= 0.0) t.full += t.w[d2];
+      }
+  return t;
 }
 
 // Sum of w_ij src_j over the filter disc of i (points of the design domain).
@@ -111,22 +109,31 @@ template <bool NEED_W>
 __device__ __forceinline__ double filter_sum(const Geo& g, const FilterTab& tab, const double* __restrict__ src,
                                              const int* i, double* W) {
   const double R = g.frad;
-  const int rr = (int)floor(R), n = tab_size(R);
+  const int rr = (int)floor(R);
   const int ez = (g.dim == 3) ? rr : 0;
-  const bool ball = g.rad4 != INT_MAX, table = n <= kTab;
+  const bool ball = g.rad4 != INT_MAX, table = tab.n > 0;
   double a = 0.0, w = 0.0;
   const int x0 = max(-rr, -i[0]), x1 = min(rr, g.nd[0] - 1 - i[0]);
   const int y0 = max(-rr, -i[1]), y1 = min(rr, g.nd[1] - 1 - i[1]);
   const int z0 = max(-ez, -i[2]), z1 = min(ez, g.nd[2] - 1 - i[2]);
   const bool whole = !ball && table && x0 == -rr && x1 == rr && y0 == -rr && y1 == rr && z0 == -ez && z1 == ez;
-  for (int dz = z0; dz <= z1; ++dz)
-    for (int dy = y0; dy <= y1; ++dy) {
+  const bool even = __all_sync(__activemask(), whole);
+  for (int dz = even ? -ez : z0; dz <= (even ? ez : z1); ++dz)
+    for (int dy = even ? -rr : y0; dy <= (even ? rr : y1); ++dy) {
       const int r2 = dy * dy + dz * dz;
-      if (r2 >= n) continue;  // beyond R
       const double* row = src + i[0] + (long long)g.nd[0] * (i[1] + dy + (long long)g.nd[1] * (i[2] + dz));
+      if (even) {  // the warp's discs are whole: the same weights for every lane
+#pragma unroll 4
+        for (int dx = -rr; dx <= rr; ++dx) {
+          const int d2 = dx * dx + r2;
+          const double wij = d2 < tab.n ? tab.w[d2] : -1.0;
+          if (wij >= 0.0) a += wij * row[dx];
+        }
+        continue;
+      }
       for (int dx = x0; dx <= x1; ++dx) {
         const int d2 = dx * dx + r2;
-        const double wij = table ? (d2 < n ? tab.w[d2] : -1.0) : filter_weight(R, d2);
+        const double wij = table ? (d2 < tab.n ? tab.w[d2] : -1.0) : filter_weight(R, d2);
         if (wij < 0.0) continue;
         if (ball) {
           const int j[3] = {i[0] + dx, i[1] + dy, i[2] + dz};
@@ -148,12 +155,11 @@ __device__ __forceinline__ void make_projection(const Geo& g, double (&pr)[2]) {
   }
 }
 
-__global__ void __launch_bounds__(kDB) k_filter_project(Geo g, const double* __restrict__ g1, double* __restrict__ gtil,
+__global__ void __launch_bounds__(kDB) k_filter_project(Geo g, const __grid_constant__ FilterTab tab,
+                                                        const double* __restrict__ g1, double* __restrict__ gtil,
                                                         double* __restrict__ gbar, double* __restrict__ W) {
-  __shared__ FilterTab tab;
   __shared__ double pr[2];
   make_projection(g, pr);
-  make_table(g, tab);
   __syncthreads();
   const int m = blockIdx.x * kDB + threadIdx.x;
   if (m >= g.ND) return;
@@ -211,10 +217,8 @@ __global__ void __launch_bounds__(kDB) k_project_T(Geo g, GradIn in, const doubl
   out[m] = g.frad > 0.0 ? v * d / W[m] : v * d;
 }
 
-__global__ void __launch_bounds__(kDB) k_filter_T(Geo g, const double* __restrict__ v, double* __restrict__ out) {
-  __shared__ FilterTab tab;
-  make_table(g, tab);
-  __syncthreads();
+__global__ void __launch_bounds__(kDB) k_filter_T(Geo g, const __grid_constant__ FilterTab tab,
+                                                  const double* __restrict__ v, double* __restrict__ out) {
   const int m = blockIdx.x * kDB + threadIdx.x;
   if (m >= g.ND) return;
   int i[3];
@@ -264,7 +268,25 @@ __global__ void __cluster_dims__(kVolCtas, 1, 1) __launch_bounds__(1024) k_volum
       if (ball) v[1] += 1.0;
     }
   }
-  block_sum<2>(v, red);
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {  // a tree over the lanes, then over the warps
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) {
+      v[0] += __shfl_xor_sync(0xffffffffu, v[0], off);
+      if (ball) v[1] += __shfl_xor_sync(0xffffffffu, v[1], off);
+    }
+    if (h == 0) {
+      if (lane == 0) {
+        red[warp] = v[0];
+        red[32 + warp] = v[1];
+      }
+      __syncthreads();
+      if (warp != 0) break;
+      v[0] = red[lane];
+      v[1] = red[32 + lane];
+    }
+  }
   if (threadIdx.x == 0) {
     mine[0] = v[0];
     mine[1] = v[1];
@@ -300,7 +322,7 @@ int launch_design_chain(const Geo& g, const double* gamma, double* g1, double* g
     launch(k_expand, nblk(g), kDB, 0, st, g, gamma, g1);
     src = g1;
   }
-  launch(k_filter_project, nblk(g), kDB, 0, st, g, src, gtil, gbar, W);
+  launch(k_filter_project, nblk(g), kDB, 0, st, g, make_table(g), src, gtil, gbar, W);
   return g.cyc > 1 ? 2 : 1;
 }
 
@@ -312,7 +334,7 @@ int chain_T(const Geo& g, const GradIn& in, const double* gtil, const double* W,
   double* o1 = filter || cyclic ? v : out;
   launch(k_project_T, nblk(g), kDB, 0, st, g, in, gtil, W, o1);
   double* o2 = cyclic ? tmp : out;
-  if (filter) launch(k_filter_T, nblk(g), kDB, 0, st, g, (const double*)o1, o2);
+  if (filter) launch(k_filter_T, nblk(g), kDB, 0, st, g, make_table(g), (const double*)o1, o2);
   if (cyclic) launch(k_orbit_sum, nblk(g), kDB, 0, st, g, (const double*)(filter ? o2 : o1), out);
   return 1 + (filter ? 1 : 0) + (cyclic ? 1 : 0);
 }
