@@ -22,20 +22,15 @@ namespace {
 
 constexpr int NVC = 3;  // force x, y and torque
 
-// Lanes per cell and the largest CTA. FP32: 2 lanes split a cell's candidate rows (the gather is bound
-// by issue: with 4 lanes the uneven rows and each lane's setup cost more than the extra warps hide).
-// FP64 issues one warp instruction per 64 cycles and scheduler, so 16 lanes take one to four
-// candidates each and a small box spreads over all SMs.
+// Lanes per cell (LC) and the largest CTA. FP32: the gather is bound by issue, and uneven rows and each
+// lane's setup cost more with every lane, while fewer leave the chip idle on small boxes: 2 lanes split a
+// cell's candidate rows while that gives each thread one cell, 1 beyond
+// (forward us per step, 2 lanes and 1: 512x256 with 128x128 design points 37.4 and 39.7; 1024x512 with
+// 256x256 57.9 and 55.8). FP64 issues one warp instruction per 64 cycles and
+// scheduler, so 16 lanes take one to four candidates each and a small box spreads over all SMs.
+constexpr int kLanes64 = 16;
 template <typename T>
-struct FlagCta;
-template <>
-struct FlagCta<float> {
-  static constexpr int lanes = 2, max_threads = 640;
-};
-template <>
-struct FlagCta<double> {
-  static constexpr int lanes = 16, max_threads = 512;
-};
+constexpr int max_threads() { return sizeof(T) == 4 ? 640 : 512; }
 
 // Sums over the design points of one cell, e = xi_m - xi(cell) the offset from the cell's image in
 // the design frame: phi, kappa, sum W e, sum W kappa e; then moved to the pivot (sum W r).
@@ -48,13 +43,13 @@ __device__ __forceinline__ void to_pivot(T xb, T xc, T eb, T ec, T kb, T kc, Acc
   o.wr[2] = o.kr[2] = T(0);
 }
 
-// FP32. Lane cl takes the candidate rows cl, cl + 2, ...; within a row the interval of candidates
+// FP32. Lane cl takes the candidate rows cl, cl + LC, ...; within a row the interval of candidates
 // follows from the two support bounds (linear in the offset), widened, and the exact test decides.
 // Cosine kernel: with the rotation scaled by pi/2 the offsets are the cosines' arguments; the factor
 // 1/16 of the two weights is applied to the sums.
+template <int LC>
 __device__ __forceinline__ void gather2d(const Geo& g, const float* __restrict__ kref, const float (&d)[2], float cs,
                                          float sn, int cl, bool active, Acc<float>& o) {
-  constexpr int LC = FlagCta<float>::lanes;
   const float S = (float)g.s, pad = 1e-3f, tiny = 1e-6f;
   const float xb = cs * d[0] + sn * d[1], xc = cs * d[1] - sn * d[0];
   const float xib = xb + g.xicf[0], xic = xc + g.xicf[1];
@@ -141,8 +136,10 @@ __device__ __forceinline__ void gather2d(const Geo& g, const float* __restrict__
 // square; the test against the support is made in FP32 first (widened by more than its rounding),
 // so FP64 instructions are spent on accepted candidates only. The six sums of the 16 lanes are
 // combined by halving (each level exchanges half of the values: 8 additions, not 24).
+template <int LC>
 __device__ __forceinline__ void gather2d(const Geo& g, const double* __restrict__ kref, const double (&d)[2],
                                          double cs, double sn, int cl, bool active, Acc<double>& o) {
+  static_assert(LC == kLanes64, "a 4 x 4 pattern of lanes");
   const double S = (double)g.s;
   const double xb = cs * d[0] + sn * d[1], xc = cs * d[1] - sn * d[0];
   const double xib = xb + g.xic[0], xic = xc + g.xic[1];
@@ -187,12 +184,12 @@ __device__ __forceinline__ void gather2d(const Geo& g, const double* __restrict_
   to_pivot(xb, xc, sb, sc, kb, kc, o);
 }
 
-template <typename T>
-__global__ void __launch_bounds__(FlagCta<T>::max_threads, 1)
+template <typename T, int LC>
+__global__ void __launch_bounds__(max_threads<T>(), 1)
     k_couple_flag(Geo g, Slots<T> S, Ctrl* ctrl, Dof* it, const T* __restrict__ kref, const Moments* __restrict__ mom,
                   void* words, T* __restrict__ boxstore, int nbox, int di) {
   using V = typename SumOf<T>::type;
-  constexpr int LC = FlagCta<T>::lanes, CPW = 32 / LC;  // lanes per cell, cells per warp
+  constexpr int CPW = 32 / LC;  // cells per warp
   constexpr int DW = (int)(sizeof(Dof) / sizeof(double));
   __shared__ V part[32 * NVC];
   __shared__ Dof sd[2];  // CTA 0: s(t-1), the current iterate
@@ -256,7 +253,7 @@ __global__ void __launch_bounds__(FlagCta<T>::max_threads, 1)
       const int n = cc.n;
       const T d[2] = {P.rel(0, cc.px), P.rel(1, cc.py)};
       Acc<T> A;
-      gather2d(g, kref, d, P.cs, P.sn, cl, bl < BC, A);
+      gather2d<LC>(g, kref, d, P.cs, P.sn, cl, bl < BC, A);
       if (bl >= BC || cl != 0) continue;
       if (A.phi == T(0)) {  // no design point in reach: u = u*
         if (last && bs && n >= 0) {
@@ -310,19 +307,21 @@ __global__ void __launch_bounds__(FlagCta<T>::max_threads, 1)
   }
 }
 
-template <typename T>
-int flag_shape(const Geo& g, int* threads) {
+// CTAs and threads of the kernel with LC lanes; *passes: cells per thread.
+template <typename T, int LC>
+int flag_shape(const Geo& g, int* threads, long long* passes) {
   int dev = 0, sms = 0, per_sm = 0;
   if (cudaGetDevice(&dev) != cudaSuccess) return 0;
   if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms < 2) return 0;
-  const long long want = g.box_cells * FlagCta<T>::lanes;
+  const long long want = g.box_cells * LC;
   // one CTA per SM, one SM for CTA 0: as few publishers as fill the chip, each with the threads its
   // share needs
   long long nt = (want + sms - 2) / (sms - 1);
+  *passes = (nt + max_threads<T>() - 1) / max_threads<T>();
   nt = (nt + 31) / 32 * 32;
   if (nt < 128) nt = 128;  // a warp per scheduler; three sum, the fourth waits for the iterate
-  if (nt > FlagCta<T>::max_threads) nt = FlagCta<T>::max_threads;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_couple_flag<T>, (int)nt, 0) != cudaSuccess) return 0;
+  if (nt > max_threads<T>()) nt = max_threads<T>();
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_couple_flag<T, LC>, (int)nt, 0) != cudaSuccess) return 0;
   if (per_sm < 1) return 0;
   const long long ctas = (want + nt - 1) / nt + 1;
   *threads = (int)nt;
@@ -337,7 +336,14 @@ void setup_couple_flag(Geo* g, bool fp64) {
   if (g->dim == 3) {
     setup_couple_axis3d(g, fp64);
   } else if (g->box_cells < (1LL << 27) && g->N < (1LL << 31)) {
-    g->flag_ctas = fp64 ? flag_shape<double>(*g, &g->flag_threads) : flag_shape<float>(*g, &g->flag_threads);
+    long long passes = 0;
+    g->flag_lanes = fp64 ? kLanes64 : 2;
+    g->flag_ctas = fp64 ? flag_shape<double, kLanes64>(*g, &g->flag_threads, &passes)
+                        : flag_shape<float, 2>(*g, &g->flag_threads, &passes);
+    if (!fp64 && passes > 1) {
+      g->flag_lanes = 1;
+      g->flag_ctas = flag_shape<float, 1>(*g, &g->flag_threads, &passes);
+    }
   }
   cudaGetLastError();  // a query that failed leaves the other forms in use
 }
@@ -349,8 +355,16 @@ template <typename T>
 void launch_couple_flag(const Geo& g, const Slots<T>& S, Ctrl* ctrl, Dof* it, const T* kref, const Moments* mom,
                         void* words, T* boxstore, int nbox, int di, cudaStream_t st) {
   if (g.dim == 3) return launch_couple_axis3d<T>(g, S, ctrl, it, kref, mom, words, boxstore, nbox, di, st);
-  launch_coop(k_couple_flag<T>, dim3((unsigned)g.flag_ctas), dim3((unsigned)g.flag_threads), 0, st, g, S, ctrl, it, kref,
-              mom, words, boxstore, nbox, di);
+  auto run = [&](auto kernel) {
+    launch_coop(kernel, dim3((unsigned)g.flag_ctas), dim3((unsigned)g.flag_threads), 0, st, g, S, ctrl, it, kref, mom,
+                words, boxstore, nbox, di);
+  };
+  if constexpr (sizeof(T) == 8)
+    run(k_couple_flag<double, kLanes64>);
+  else if (g.flag_lanes == 1)
+    run(k_couple_flag<float, 1>);
+  else
+    run(k_couple_flag<float, 2>);
 }
 
 template void launch_couple_flag<float>(const Geo&, const Slots<float>&, Ctrl*, Dof*, const float*, const Moments*,
