@@ -333,14 +333,23 @@ int g_last_cuda_error = 0;
     }                                         \
   } while (0)
 
+int give_back_optional(lks_handle* h, bool* gave);
+
+// A buffer the call cannot do without: the optional ones make room for it when the budget or the device
+// has none left.
 int dalloc(lks_handle* h, void** p, size_t bytes) {
   if (bytes == 0) bytes = 16;
   bytes = (bytes + 255) & ~(size_t)255;
-  if (h->P.hbm_budget_bytes && h->bytes + bytes > h->P.hbm_budget_bytes) return LKS_ERR_BUDGET;
-  cudaError_t e = cudaMalloc(p, bytes);
-  if (e != cudaSuccess) {
-    cudaGetLastError();
-    return LKS_ERR_OOM;
+  for (;;) {
+    const bool over = h->P.hbm_budget_bytes && h->bytes + bytes > h->P.hbm_budget_bytes;
+    if (!over) {
+      if (cudaMalloc(p, bytes) == cudaSuccess) break;
+      cudaGetLastError();
+    }
+    bool gave = false;
+    const int r = give_back_optional(h, &gave);
+    if (r != LKS_OK) return r;
+    if (!gave) return over ? LKS_ERR_BUDGET : LKS_ERR_OOM;
   }
   h->bytes += bytes;
   h->allocs.push_back(*p);
@@ -845,13 +854,36 @@ void choose_coupling(lks_handle* h) {
     return;
   }
   h->bytes += need;
-  h->allocs.push_back(h->words);
+}
+
+// Frees a buffer the handle can do without and the graphs that name it: the reverse's linear maps (a later
+// lks_adjoint takes them again where it finds room), then the flagged words (the other forms run from
+// then on).
+int give_back_optional(lks_handle* h, bool* gave) {
+  *gave = h->rev.block || h->words;
+  if (!*gave) return LKS_OK;
+  CK(cudaDeviceSynchronize());
+  clear_graphs(h);
+  if (h->rev.block) {
+    CK(cudaFree(h->rev.block));
+    h->rev.block = nullptr;
+    h->bytes -= h->rev_bytes;
+    h->rev_bytes = 0;
+    h->rev_on = false;
+    return LKS_OK;
+  }
+  CK(cudaFree(h->words));
+  h->words = nullptr;
+  h->bytes -= (couple_flag_bytes(kFlagMaxCtas) + 255) & ~(size_t)255;
+  h->no_words = true;
+  h->g.flag_ctas = h->g.flag_threads = 0;
+  return LKS_OK;
 }
 
 // Chooses the form of the exact reverse: the linear maps for bodies about one axis in the automatic
 // coupling mode, when the workspace limit and the device have room for their buffers; else the
 // per-iteration or persistent kernels.
-int choose_reverse(lks_handle* h) {
+int choose_reverse(lks_handle* h, cudaStream_t st) {
   h->rev_on = false;
   if (h->coop_mode != 2 || !reverse_affine_fits(h->g)) return LKS_OK;
   const int seg = h->P.ckpt_policy == LKS_CKPT_BINOMIAL ? 1
@@ -859,6 +891,9 @@ int choose_reverse(lks_handle* h) {
   RevBuffers R;
   const size_t need = reverse_layout(h->g, h->prec == LKS_FP64, seg, &R);
   if (need > h->rev_bytes) {  // the first call, or a larger body box since (its graphs are gone)
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    CK(cudaStreamIsCapturing(st, &cs));
+    if (cs != cudaStreamCaptureStatusNone) return LKS_OK;  // no allocation while the caller captures
     if (h->P.hbm_budget_bytes && h->bytes - h->rev_bytes + need > h->P.hbm_budget_bytes) return LKS_OK;
     if (h->rev.block) {
       CK(cudaDeviceSynchronize());
@@ -1158,7 +1193,7 @@ int lks_adjoint(lks_handle* h, double seed, void* stream) {
   if (!h->fwd_done) return LKS_ERR_ORDER;
   cudaStream_t st = (cudaStream_t)stream;
   h->adj_done = h->exact_done = false;
-  TRY(choose_reverse(h));
+  TRY(choose_reverse(h, st));
   int r = (h->prec == LKS_FP64) ? adjoint_impl<double>(h, seed, st) : adjoint_impl<float>(h, seed, st);
   if (r != LKS_OK) return r;
   // a grid barrier or tile copy whose wait timed out is reported through the status word
@@ -1506,6 +1541,7 @@ void lks_destroy(lks_handle* h) {
       cudaEventDestroy(p.b);
     }
   for (void* p : h->allocs) cudaFree(p);
+  cudaFree(h->words);
   cudaFree(h->rev.block);
   if (h->cap) cudaStreamDestroy(h->cap);
   if (h->cap2) cudaStreamDestroy(h->cap2);
