@@ -10,8 +10,8 @@
 //
 // What bounds it: the gather's slowest warps and two trips through L2 per iteration. Forward march
 // measured on GB300, N_itr launches (or grid barriers) per step -> this kernel, us per step: 512x256
-// body of 128^2 60 -> 37; 1024x512, 256^2 (grid barriers before) 100 -> 58; FP64 80x40, 16^2 290 -> 58;
-// FP64 600x100, 20^2 500 -> 67.
+// body of 128^2 60 -> 37; 1024x512, 256^2 (grid barriers before) 100 -> 56; FP64 80x40, 16^2 290 -> 58;
+// FP64 600x100, 20^2 500 -> 67 (40 and 60 with the tiled stencils of lks_stencil_tile.cu).
 #include <climits>
 
 #include "lks_flag.cuh"
@@ -24,10 +24,9 @@ constexpr int NVC = 3;  // force x, y and torque
 
 // Lanes per cell (LC) and the largest CTA. FP32: the gather is bound by issue, and uneven rows and each
 // lane's setup cost more with every lane, while fewer leave the chip idle on small boxes: 2 lanes split a
-// cell's candidate rows while that gives each thread one cell, 1 beyond
-// (forward us per step, 2 lanes and 1: 512x256 with 128x128 design points 37.4 and 39.7; 1024x512 with
-// 256x256 57.9 and 55.8). FP64 issues one warp instruction per 64 cycles and
-// scheduler, so 16 lanes take one to four candidates each and a small box spreads over all SMs.
+// cell's candidate rows while that gives each thread one cell, 1 beyond (forward us per step, 2 lanes
+// and 1: 512x256 with 128x128 design points 37.4 and 39.7; 1024x512 with 256x256 57.9 and 55.8). FP64
+// issues one warp instruction per 64 cycles and scheduler, so 16 lanes take one to four candidates each and a small box spreads over all SMs.
 constexpr int kLanes64 = 16;
 template <typename T>
 constexpr int max_threads() { return sizeof(T) == 4 ? 640 : 512; }
