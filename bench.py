@@ -117,30 +117,28 @@ def _peaks():
 
 
 # Algorithmic bytes per launch of each kernel family. N = analysis cells, box_cells = body-box
-# cells, ND = design points, esz = bytes per field value, K = N_itr (the persistent families
-# "couple" and "adj_body" run all K iterations of a step in one launch).
-def _alg_bytes(family: str, P, box_cells: int, esz: int, persistent: bool = True) -> float:
+# cells, ND = design points, esz = bytes per field value, K = N_itr. A body family's launches per step
+# depend on the chosen form (all K iterations in one launch, one launch per iteration, several steps
+# in one launch), so its bytes are those of a step, divided by its launches per step.
+def _alg_bytes(family: str, P, box_cells: int, esz: int, launches_per_step: float = 1.0) -> float:
     N, ND = P.n_cells, P.n_design
     d, K = P.dim, P.n_itr
     if family == "stencil_fwd":
         return 2 * (d + 1) * esz * N  # read p, u; write p*, u*
     if family == "stencil_adj":
         return (3 * d + 2) * esz * N  # read the adjoint (d+1 planes) and u(t-1) (d planes); write d+1 planes
-    if family == "couple":
-        per_iter = d * esz * box_cells + 4 * ND  # read u* in the box (+ kappa^ref)
-        if persistent:  # K iterations, then u(t) and the stored u* written once
-            return K * per_iter + 2 * d * esz * box_cells
-        return per_iter
+    if family == "couple":  # each iteration reads u* in the box (+ kappa^ref), the last writes u(t), stored u*
+        return (K * (d * esz * box_cells + 4 * ND) + 2 * d * esz * box_cells) / launches_per_step
     if family == "recompute":
         return 3 * d * esz * box_cells + 4 * ND  # read u*, write u and the stored u*
     cell = (5 * d + 1) * esz * box_cells      # read stored u*, acc r/w, scratch write (2d+1 planes)
     design = (2 * d + 1) * esz * box_cells + 20 * ND  # read scratch once, dJ/dkappa^ref r/w + kappa^ref
     if family == "adj_cell":
-        return cell
+        return K * cell / launches_per_step
     if family == "adj_design":
-        return design
+        return K * design / launches_per_step
     if family == "adj_body":
-        return K * (cell + design)
+        return K * (cell + design) / launches_per_step
     if family == "alks_stencil":
         # the paper's adjoint equilibrium and gather. 2D, one tiled pass: read p~, u~, s~
         # (1 + d + d(d+1)/2 planes) and u (d), write the star moments. 3D, two passes: read the
@@ -649,7 +647,7 @@ def main():
         peak, peak_kind = _peaks()
         per_launch_s = dom_ms / 1000.0 / dom_n
         persistent = lks.lks_persistent_coupling(solver.handle, -1)
-        alg = _alg_bytes(dom, P, _box_cells(P), 4, persistent)
+        alg = _alg_bytes(dom, P, _box_cells(P), 4, dom_n / P.n_steps)
         achieved = alg / per_launch_s / 1e9
         line["roofline"] = {"bound": "hbm", "kernel": dom, "achieved": achieved, "peak": peak, "unit": "GB/s",
                             "frac": achieved / peak, "traffic": _traffic(P.name, dom), "peak_source": peak_kind,
