@@ -1370,7 +1370,7 @@ template <typename T>
 void launch_adj_cell(const Geo& g, const Ctrl* ctrl, const Dof* it, const T* kref, const T* boxstore, int nbox, T* Lb,
                      long long lstride, T* acc, T* scratch, int k, int di, cudaStream_t st) {
   if constexpr (sizeof(T) == 4)
-    if (g.free_tiled)
+    if (g.free_tiled && free_cell_pays(g))
       return launch_adj_cell_free(g, ctrl, it, kref, boxstore, nbox, Lb, lstride, acc, scratch, k, di, st);
   LKS_BOX_DISPATCH(k_adj_cell, box_grid(g), box_threads(g), g, ctrl, it, kref, boxstore, nbox, Lb, lstride, acc,
                    scratch, k, di);
@@ -1382,7 +1382,7 @@ void launch_adj_design(const Geo& g, Ctrl* ctrl, const Dof* it, const T* kref, c
   unsigned nb = (unsigned)design_ctas(g);
   bool done = false;
   if constexpr (sizeof(T) == 4) {
-    if (g.free_tiled) {
+    if (g.free_tiled && free_design_pays(g)) {
       nb = (unsigned)free_design_ctas(g);
       launch_adj_design_free(g, ctrl, it, kref, scratch, dkref, partials, k, di, st);
       done = true;

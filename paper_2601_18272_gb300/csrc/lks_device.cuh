@@ -164,7 +164,7 @@ struct Geo {
   int margin;     // cells of drift allowed within one step
   long long box_cells;
   int flag_ctas, flag_threads, flag_lanes;  // shape of the flag-exchange coupling kernels (0: another form runs)
-  int free_tiled;  // free rotation, FP32, cosine kernel: the tiled reverse kernels run (lks_free3d.cu)
+  int free_tiled;  // free rotation, FP32, cosine kernel: the tiled reverse kernels may run (lks_free3d.cu)
   int coop_fwd, coop_adj;  // CTAs of the cooperative coupling kernels (0: the per-iteration kernels)
 };
 

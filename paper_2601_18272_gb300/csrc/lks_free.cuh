@@ -8,9 +8,12 @@ namespace lks {
 constexpr int kFreeTile = 8;          // cells per tile edge
 constexpr int kFreeDesignCtas = 304;  // design-point kernel: two CTAs per SM, striding over the tiles
 
-// Shared memory of the kernels; Geo::free_tiled tells whether a handle runs them.
+// Shared memory of the kernels; Geo::free_tiled tells whether a handle may run them, free_*_pays whether
+// they are the faster ones for its body box.
 bool prepare_free3d();
 int free_tiles(const Geo& g);
+bool free_cell_pays(const Geo& g);
+bool free_design_pays(const Geo& g);
 void launch_adj_cell_free(const Geo& g, const Ctrl* ctrl, const Dof* it, const float* kref, const float* boxstore, int nbox,
                           float* Lb, long long lstride, float* acc, float* scratch, int k, int di, cudaStream_t st);
 int free_design_ctas(const Geo& g);

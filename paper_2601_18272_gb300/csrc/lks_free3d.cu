@@ -19,6 +19,7 @@
 // single gradient entries by up to 8e-4 of their rms (BF16, 12 steps), where no more than that is wanted;
 // the forward must not depend on the snapshots' format either.
 #include <algorithm>
+#include <climits>
 
 #include "lks_body_common.cuh"
 #include "lks_free.cuh"
@@ -560,6 +561,16 @@ int free_tiles(const Geo& g) {
   const dim3 n = free_grid(g);
   return (int)(n.x * n.y * n.z);
 }
+
+// Where the tiles pay. Few tiles leave the chip idle for the whole of a tile's sort and sums (about 22 us for
+// the cell phase), and a box-shaped body leaves the corners of its box, a tile each, without design points.
+// GB300, us per iteration, per point or cell -> tiles:
+//   cell phase        ball, box of 40^3 cells 21.8 -> 22.7, 44^3 25.0 -> 22.9, 52^3 37.4 -> 30.5;
+//                     solid, 42^3 18.8 -> 22.7, 48^3 21.5 -> 21.3, 56^3 29.5 -> 22.8, 90^3 97.8 -> 49.4
+//   design points     ball, 36^3 46.6 -> 47.3, 40^3 53.9 -> 46.3, 52^3 70.6 -> 57.1;
+//                     solid, 56^3 46.7 -> 49.6, 90^3 75.3 -> 79.7, 104^3 95.4 -> 80.2
+bool free_cell_pays(const Geo& g) { return g.box_cells >= 80000; }
+bool free_design_pays(const Geo& g) { return g.box_cells >= (g.rad4 != INT_MAX ? 55000 : 1000000); }
 
 int free_design_ctas(const Geo& g) { return std::min(free_tiles(g), kFreeDesignCtas); }
 

@@ -2,7 +2,8 @@
 and against the persistent kernels (lks_persistent_coupling mode 1), which gather per cell: odd box
 sizes, a design smaller and larger than a tile, solid and ball domains, the identity with points exactly
 on cells' corners, quarter turns (points on corners up to rounding), a body across the periodic boundary,
-one iteration, masked rotation. Held to twice the other form's FP32 error plus 2e-5."""
+one iteration, masked rotation. Small boxes take the per-cell kernels in one or both phases; the larger
+bodies ("tiles-...") reach the tiles: balls in both phases, a solid one in the cell phase only. Held to twice the other form's FP32 error plus 2e-5."""
 from __future__ import annotations
 
 import numpy as np
@@ -25,6 +26,14 @@ def _cases():
     yield "wrapped", body6(nx=30, ny=28, nz=26, nd=8, centre=(29.7, 0.4, 25.8), nt=2, bc=PER), (-0.6, 1.1, 0.2)
     yield "one-iteration", body6(nx=28, ny=26, nz=26, nd=7, centre=(13.2, 12.7, 12.2), nt=3, n_itr=1), (0.2, 0.9, -0.4)
     yield "masked", body6(nx=28, ny=26, nz=26, nd=7, centre=(13.2, 12.7, 12.2), nt=2, mask=DOF_TX | DOF_TY), (0.2, 0.9, -0.4)
+    ball = dict(nd=41, radius=19.5, sphere=True, nt=2)
+    yield "tiles-ball", body6(nx=58, ny=56, nz=57, centre=(28.3, 27.6, 28.1), **ball), (0.9, 0.1, 0.2)
+    yield "tiles-identity-corners", body6(nx=56, ny=56, nz=56, centre=(28.0, 27.0, 28.0), **ball), (0.0, 0.0, 0.0)
+    yield "tiles-quarter-turn", body6(nx=56, ny=56, nz=56, centre=(28.0, 27.0, 28.0), **ball), (0.0, 0.0, Q)
+    yield "tiles-wrapped", body6(nx=56, ny=55, nz=57, centre=(55.7, 0.4, 56.2), bc=PER, **ball), (-0.6, 1.1, 0.2)
+    yield "tiles-masked", body6(nx=56, ny=56, nz=56, centre=(27.3, 28.1, 27.8), mask=DOF_TX | DOF_TY, n_itr=1,
+                                **ball), (0.2, 0.9, -0.4)
+    yield "tiles-solid", body6(nx=66, ny=65, nz=64, nd=29, centre=(32.3, 31.6, 32.1), nt=2), (0.3, -0.2, 0.5)
 
 
 CASES = list(_cases())
@@ -57,7 +66,7 @@ def _rel(a, b):
 def test_tiles_match_fp64_and_the_per_cell_gather(name, problem, rotvec):
     P, g = problem
     state = perturbed_state6(P, rotvec=rotvec)
-    if name in ("identity-corners", "quarter-turn"):
+    if name.endswith(("identity-corners", "quarter-turn")):
         state[2][12:21] = np.round(state[2][12:21])
     ref = _run(P, g, state, 64, 0, ckpt_policy=CKPT_STORE_ALL)
     new = _run(P, g, state, 32, 2, ckpt_policy=CKPT_BINOMIAL, ckpt_every=1)
