@@ -304,7 +304,8 @@ struct lks_handle {
   double host_s0[kNdofFree];
   size_t bytes = 0;
   std::vector<void*> allocs;
-  cudaStream_t cap = nullptr, cap2 = nullptr;  // capture streams: the chain, and a branch beside it
+  // capture streams: graphs of one chain; a chain with a branch beside it (high priority); the branch
+  cudaStream_t cap = nullptr, cap_high = nullptr, cap2 = nullptr;
   cudaEvent_t fork_ev = nullptr, coef_ev[2] = {nullptr, nullptr};
   std::map<std::string, cudaGraphExec_t> graphs;
   std::map<std::string, int> graph_kernels;
@@ -419,9 +420,10 @@ void collect_timers(lks_handle* h) {
   }
 }
 
-// Run `body` either directly (timing mode) or as a cached CUDA graph captured on a private stream.
+// Run `body` either directly (timing mode) or as a cached CUDA graph captured on a private stream
+// (branch: the one of high priority, for a chain with a branch beside it).
 template <typename Body>
-int run_graph(lks_handle* h, const std::string& key, cudaStream_t st, Body&& body) {
+int run_graph(lks_handle* h, const std::string& key, cudaStream_t st, Body&& body, bool branch = false) {
   if (h->timing) {
     Launcher L{h, st, false};
     body(L);
@@ -431,10 +433,11 @@ int run_graph(lks_handle* h, const std::string& key, cudaStream_t st, Body&& bod
   auto itg = h->graphs.find(key);
   if (itg == h->graphs.end()) {
     cudaGraph_t graph;
-    CK(cudaStreamBeginCapture(h->cap, cudaStreamCaptureModeThreadLocal));
-    Launcher L{h, h->cap, true};
+    const cudaStream_t cap = branch ? h->cap_high : h->cap;
+    CK(cudaStreamBeginCapture(cap, cudaStreamCaptureModeThreadLocal));
+    Launcher L{h, cap, true};
     body(L);
-    cudaError_t e = cudaStreamEndCapture(h->cap, &graph);
+    cudaError_t e = cudaStreamEndCapture(cap, &graph);
     if (e != cudaSuccess) {
       g_last_cuda_error = (int)e;
       return LKS_ERR_CUDA;
@@ -809,7 +812,7 @@ int adjoint_impl(lks_handle* h, double seed, cudaStream_t st) {
       const int n = std::min(h->chunk, t1);
       L0("init", [&](cudaStream_t s) { launch_set_step(h->ctrl, t1, 0, s); });
       TRY(run_graph(h, std::string(kind) + "sa_" + std::to_string(n), st,
-                    [&](Launcher& L) { enqueue_adj_steps<T>(h, L, S, n); }));
+                    [&](Launcher& L) { enqueue_adj_steps<T>(h, L, S, n); }, h->rev_on && !h->alks_mode));
     }
   } else {
     Slots<T> S = ring_slots<T>(h);
@@ -832,7 +835,7 @@ int adjoint_impl(lks_handle* h, double seed, cudaStream_t st) {
       TRY(run_graph(h, "rec_" + std::to_string(n), st, [&](Launcher& L) { enqueue_recompute<T>(h, L, S, n); }));
       L0("init", [&](cudaStream_t s) { launch_set_step(h->ctrl, t0 + n, t0, s); });
       TRY(run_graph(h, std::string(kind) + "u_" + std::to_string(n), st,
-                    [&](Launcher& L) { enqueue_adj_steps<T>(h, L, S, n); }));
+                    [&](Launcher& L) { enqueue_adj_steps<T>(h, L, S, n); }, h->rev_on && !h->alks_mode));
     }
   }
   if (h->rev_on && !h->alks_mode) L0("adj_design", [&](cudaStream_t s) { launch_rev_dksum(g, h->rev, h->dkref, s); });
@@ -1107,7 +1110,8 @@ int lks_create(const lks_problem* P, lks_handle** out) {
   if (r == LKS_OK) r = set_default_initial_state(h);
   int low = 0, high = 0;  // the chain's kernels go before the branch's (graph nodes keep the priority)
   cudaDeviceGetStreamPriorityRange(&low, &high);
-  if (r == LKS_OK && (cudaStreamCreateWithPriority(&h->cap, cudaStreamNonBlocking, high) != cudaSuccess ||
+  if (r == LKS_OK && (cudaStreamCreateWithFlags(&h->cap, cudaStreamNonBlocking) != cudaSuccess ||
+                      cudaStreamCreateWithPriority(&h->cap_high, cudaStreamNonBlocking, high) != cudaSuccess ||
                       cudaStreamCreateWithPriority(&h->cap2, cudaStreamNonBlocking, low) != cudaSuccess ||
                       cudaEventCreateWithFlags(&h->fork_ev, cudaEventDisableTiming) != cudaSuccess ||
                       cudaEventCreateWithFlags(&h->coef_ev[0], cudaEventDisableTiming) != cudaSuccess ||
@@ -1544,6 +1548,7 @@ void lks_destroy(lks_handle* h) {
   cudaFree(h->words);
   cudaFree(h->rev.block);
   if (h->cap) cudaStreamDestroy(h->cap);
+  if (h->cap_high) cudaStreamDestroy(h->cap_high);
   if (h->cap2) cudaStreamDestroy(h->cap2);
   for (cudaEvent_t e : {h->fork_ev, h->coef_ev[0], h->coef_ev[1]})
     if (e) cudaEventDestroy(e);
