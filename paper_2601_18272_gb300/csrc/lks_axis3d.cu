@@ -619,10 +619,16 @@ __global__ void __launch_bounds__(128) k_design_axis3d(Geo g, Ctrl* ctrl, const 
   id[slow] = q / g.nd[fast];
   id[fast] = q - id[slow] * g.nd[fast];
   id[a3] = ch * Z;
-  const int np = min(Z, g.nd[a3] - id[a3]);  // points of this thread
+  int np = min(Z, g.nd[a3] - id[a3]);  // points of this thread
+  // A ball: only the column's points in the design domain (consecutive ones). The body box is sized to the
+  // domain, so the window of a point off it may lie outside the box, and must not decide for the others.
+  if (g.rad4 != INT_MAX) {
+    const int left = g.rad4 - dsq(id[b], g.nd[b]) - dsq(id[c], g.nd[c]);
+    while (np > 0 && dsq(id[a3] + np - 1, g.nd[a3]) > left) --np;
+    while (np > 0 && dsq(id[a3], g.nd[a3]) > left) ++id[a3], --np;
+    if (np == 0) return;
+  }
   const T r[3] = {(T)id[0] - pivot<T>(g, 0), (T)id[1] - pivot<T>(g, 1), (T)id[2] - pivot<T>(g, 2)};
-  const int left = g.rad4 == INT_MAX ? INT_MAX : g.rad4 - dsq(id[b], g.nd[b]) - dsq(id[c], g.nd[c]);
-  if (left < 0) return;  // the column lies off the design domain
   const long long BC = g.box_cells;
   const int st[3] = {1, g.B[0], g.B[0] * g.B[1]}, S2 = 2 * g.s;
   bool inside = true;
@@ -710,8 +716,7 @@ __global__ void __launch_bounds__(128) k_design_axis3d(Geo g, Ctrl* ctrl, const 
   const int m0 = id[0] * sd[0] + id[1] * sd[1] + id[2] * sd[2];
 #pragma unroll
   for (int j = 0; j < Z; ++j)
-    if (j < np && (left == INT_MAX || dsq(id[a3] + j, g.nd[a3]) <= left))
-      dkp[(long long)blockIdx.y * g.ND + m0 + j * sd[a3]] += acc[j];
+    if (j < np) dkp[(long long)blockIdx.y * g.ND + m0 + j * sd[a3]] += acc[j];
 }
 
 constexpr size_t list_bytes(int warps) { return (size_t)warps * kListMax * 32 * sizeof(unsigned); }
