@@ -566,6 +566,8 @@ void enqueue_fwd_steps(lks_handle* h, Launcher& L, const Slots<T>& S, int nsteps
   }
 }
 
+// Graphs with recomputed steps hold the form of the forward that ran (Geo::fwd_form).
+std::string recompute_key(const lks_handle* h, const char* name) { return name + std::to_string(h->g.fwd_form) + "_"; }
 template <typename T>
 void enqueue_recompute(lks_handle* h, Launcher& L, const Slots<T>& S, int nsteps) {
   const Geo& g = h->g;
@@ -761,7 +763,7 @@ int binomial_reverse(lks_handle* h, cudaStream_t st) {
       case LKS_BIN_ADVANCE: {  // state(a) -> state(a + b)
         const int t0 = op.a, n = op.b;
         L0("init", [&](cudaStream_t x) { launch_set_step(h->ctrl, t0 + 1, t0, x); });
-        TRY(run_graph(h, "bin_adv_" + std::to_string(n), st, [&](Launcher& L) { enqueue_recompute<T>(h, L, W, n); }));
+        TRY(run_graph(h, recompute_key(h, "bin_adv_") + std::to_string(n), st, [&](Launcher& L) { enqueue_recompute<T>(h, L, W, n); }));
         break;
       }
       case LKS_BIN_STORE:  // snapshot slot a <- state(b), c steps past the working pair's base
@@ -770,7 +772,8 @@ int binomial_reverse(lks_handle* h, cudaStream_t st) {
       case LKS_BIN_REVERSE: {  // step a from state(a - 1) in the working pair (base b)
         const int t = op.a, t0 = op.b;
         L0("init", [&](cudaStream_t x) { launch_set_step(h->ctrl, t, t0, x); });
-        TRY(run_graph(h, std::string(h->alks_mode ? "alks_" : (h->rev_on ? "rev_" : "adj_")) + "bin_rev1", st, [&](Launcher& L) {
+        const char* kind = h->alks_mode ? "alks_" : (h->rev_on ? "rev_" : "adj_");
+        TRY(run_graph(h, recompute_key(h, kind) + "bin_rev1", st, [&](Launcher& L) {
           enqueue_recompute<T>(h, L, W, 1);
           enqueue_adj_steps<T>(h, L, W, 1);
         }));
@@ -832,7 +835,7 @@ int adjoint_impl(lks_handle* h, double seed, cudaStream_t st) {
         });
       }
       L0("init", [&](cudaStream_t s) { launch_set_step(h->ctrl, t0 + 1, t0, s); });
-      TRY(run_graph(h, "rec_" + std::to_string(n), st, [&](Launcher& L) { enqueue_recompute<T>(h, L, S, n); }));
+      TRY(run_graph(h, recompute_key(h, "rec_") + std::to_string(n), st, [&](Launcher& L) { enqueue_recompute<T>(h, L, S, n); }));
       L0("init", [&](cudaStream_t s) { launch_set_step(h->ctrl, t0 + n, t0, s); });
       TRY(run_graph(h, std::string(kind) + "u_" + std::to_string(n), st,
                     [&](Launcher& L) { enqueue_adj_steps<T>(h, L, S, n); }, h->rev_on && !h->alks_mode));
@@ -1162,6 +1165,7 @@ int lks_forward(lks_handle* h, const double* gamma_dev, double* J_host, void* st
   cudaStream_t st = (cudaStream_t)stream;
   choose_coupling(h);
   const Geo& g = h->g;
+  h->g.fwd_form = g.flag_ctas == 0 ? 0 : (g.dim == 2 ? g.flag_lanes : 1);
   h->fwd_done = h->adj_done = h->exact_done = h->alks_done = false;
   if ((const void*)gamma_dev != (const void*)h->gamma)
     CK(cudaMemcpyAsync(h->gamma, gamma_dev, (size_t)g.ND * sizeof(double), cudaMemcpyDeviceToDevice, st));

@@ -78,7 +78,7 @@ __device__ __forceinline__ int column_list(const Geo& g, const T (&d)[3], T cs, 
                                            unsigned (*list)[32], int lane) {
   constexpr int b = Axes<AX>::B, c = Axes<AX>::C;
   const T S = (T)g.s;
-  const T xib = cs * d[b] + sn * d[c] + pivot<T>(g, b), xic = cs * d[c] - sn * d[b] + pivot<T>(g, c);
+  const T xib = dot2(cs, d[b], sn, d[c]) + pivot<T>(g, b), xic = dot2(cs, d[c], -sn, d[b]) + pivot<T>(g, c);
   const float csf = (float)cs, snf = (float)sn, pad = 2e-3f, Sp = (float)g.s + pad;
   const float xibf = (float)xib, xicf = (float)xic, h = Sp * (fabsf(csf) + fabsf(snf)) + pad;
   const int ib0 = max(0, (int)ceilf(xibf - h)), ib1 = active ? min(g.nd[b] - 1, (int)floorf(xibf + h)) : -1;
@@ -104,7 +104,7 @@ __device__ __forceinline__ int column_list(const Geo& g, const T (&d)[3], T cs, 
     const T ec = (T)ic - xic;
     for (int ib = j0; ib <= j1; ++ib) {
       const T eb = (T)ib - xib;
-      if (fabs(cs * eb - sn * ec) < S && fabs(sn * eb + cs * ec) < S && n < kListMax)
+      if (fabs(dot2(cs, eb, -sn, ec)) < S && fabs(dot2(sn, eb, cs, ec)) < S && n < kListMax)
         list[n++][lane] = (unsigned)ib | ((unsigned)ic << 16);
     }
   }
@@ -121,8 +121,8 @@ struct Column {
     ib = (int)(e & 0xffffu);
     ic = (int)(e >> 16);
     const T eb = (T)ib - xib, ec = (T)ic - xic;
-    ob = cs * eb - sn * ec;
-    oc = sn * eb + cs * ec;
+    ob = dot2(cs, eb, -sn, ec);
+    oc = dot2(sn, eb, cs, ec);
     lb = ob + d[b];
     lc = oc + d[c];
   }
@@ -189,7 +189,7 @@ template <typename T, int AX, bool BALL, int Z>
 __device__ __forceinline__ void plane_sums(const Geo& g, const T* __restrict__ kref, const T (&d)[3], T cs, T sn, int n,
                                            const unsigned (*list)[32], int lane, PlaneSums<T, Z>& o) {
   constexpr int b = Axes<AX>::B, c = Axes<AX>::C, a = Axes<AX>::A;
-  const T xib = cs * d[b] + sn * d[c] + pivot<T>(g, b), xic = cs * d[c] - sn * d[b] + pivot<T>(g, c);
+  const T xib = dot2(cs, d[b], sn, d[c]) + pivot<T>(g, b), xic = dot2(cs, d[c], -sn, d[b]) + pivot<T>(g, c);
   const Axial<T, AX> ax(g, d[a]);
   int sb, sc, sa;
   design_strides<AX>(g, sb, sc, sa);
@@ -210,8 +210,8 @@ __device__ __forceinline__ void plane_sums(const Geo& g, const T* __restrict__ k
       en = list[i + 1][lane];
       load_window<T, Z>(column_at(en), ax.ia0, g.nd[a], sa, kn);
     }
-    const T w2 = wfun(g.wk, q.ob) * wfun(g.wk, q.oc);
-    const T wb = w2 * q.lb, wc = w2 * q.lc;
+    const T w2 = mul_(wfun(g.wk, q.ob), wfun(g.wk, q.oc));
+    const T wb = mul_(w2, q.lb), wc = mul_(w2, q.lc);
     int left = 0;
     if (BALL) left = g.rad4 - dsq(q.ib, g.nd[b]) - dsq(q.ic, g.nd[c]);
     if (!BALL) {
@@ -221,10 +221,10 @@ __device__ __forceinline__ void plane_sums(const Geo& g, const T* __restrict__ k
     }
 #pragma unroll
     for (int j = 0; j < Z; ++j) {
-      const T s = ax.w[0] * kv[j] + ax.w[1] * kv[j + 1] + ax.w[2] * kv[j + 2] + ax.w[3] * kv[j + 3];
-      o.kap[j] += w2 * s;
-      o.Lb[j] += wb * s;
-      o.Lc[j] += wc * s;
+      const T s = fma_(ax.w[3], kv[j + 3], fma_(ax.w[2], kv[j + 2], dot2(ax.w[1], kv[j + 1], ax.w[0], kv[j])));
+      o.kap[j] = fma_(w2, s, o.kap[j]);
+      o.Lb[j] = fma_(wb, s, o.Lb[j]);
+      o.Lc[j] = fma_(wc, s, o.Lc[j]);
       if (BALL) {  // the points of the design domain only (kappa is zero off it)
         T s1 = T(0);
 #pragma unroll
@@ -232,9 +232,9 @@ __device__ __forceinline__ void plane_sums(const Geo& g, const T* __restrict__ k
           const int ia = ax.ia0 + j + m;
           if (ia >= 0 && ia < g.nd[a] && dsq(ia, g.nd[a]) <= left) s1 += ax.w[m];
         }
-        o.phi[j] += w2 * s1;
-        o.Pb[j] += wb * s1;
-        o.Pc[j] += wc * s1;
+        o.phi[j] = fma_(w2, s1, o.phi[j]);
+        o.Pb[j] = fma_(wb, s1, o.Pb[j]);
+        o.Pc[j] = fma_(wc, s1, o.Pc[j]);
       }
     }
   }
@@ -247,9 +247,9 @@ __device__ __forceinline__ void plane_sums(const Geo& g, const T* __restrict__ k
         const int ia = ax.ia0 + j + m;
         if (ia >= 0 && ia < g.nd[a]) s1 += ax.w[m];
       }
-      o.phi[j] = f2 * s1;
-      o.Pb[j] = pb2 * s1;
-      o.Pc[j] = pc2 * s1;
+      o.phi[j] = mul_(f2, s1);
+      o.Pb[j] = mul_(pb2, s1);
+      o.Pc[j] = mul_(pc2, s1);
     }
 }
 
@@ -305,7 +305,7 @@ struct LaneCells {
 template <typename T, int AX, typename U>
 __device__ __forceinline__ T solid_velocity(int a, const U& ug, T om, T phi, T Pb, T Pc) {
   constexpr int b = Axes<AX>::B, c = Axes<AX>::C;
-  return ug[a] * phi + (a == b ? -om * Pc : (a == c ? om * Pb : T(0)));
+  return a == b ? dot2(ug[a], phi, -om, Pc) : (a == c ? dot2(ug[a], phi, om, Pb) : mul_(ug[a], phi));
 }
 
 // A running sum of FP32 values as a double-float pair, or of doubles.
@@ -388,7 +388,7 @@ __global__ void __launch_bounds__(512, 1)
 #pragma unroll
         for (int a = 0; a < 3; ++a) {
           const T sv = solid_velocity<T, AX>(a, P.ug, P.om, A.phi[j], A.Pb[j], A.Pc[j]);
-          uu[a] = (us[j][a] + A.kap[j] * sv) * inv;
+          uu[a] = brinkman(us[j][a], A.kap[j], sv, inv);
         }
         if (work >> j & 1u) {
 #pragma unroll
@@ -456,7 +456,7 @@ __global__ void __launch_bounds__(kApplyWarps * 32) k_apply_axis3d(Geo g, Slots<
     for (int a = 0; a < 3; ++a) {
       const T sv = solid_velocity<T, AX>(a, P.ug, P.om, A.phi[j], A.Pb[j], A.Pc[j]);
       bs[a * g.box_cells + bl0 + (long long)j * sbx] = us[j][a];
-      if (body) dst[(a + 1) * g.N + lc.at(j)] = (us[j][a] + A.kap[j] * sv) * inv;
+      if (body) dst[(a + 1) * g.N + lc.at(j)] = brinkman(us[j][a], A.kap[j], sv, inv);
     }
   }
 }
@@ -489,7 +489,7 @@ __global__ void __launch_bounds__(kRevThreads) k_coef_axis3d(Geo g, const Ctrl* 
     const LanePos lp = lane_pos<AX>(g, u0, tiles, Z, lane);
     const T d[3] = {P.rel(0, lo[0] + lp.j[0]), P.rel(1, lo[1] + lp.j[1]), P.rel(2, lo[2] + lp.j[2])};
     const int n = column_list<T, AX>(g, d, P.cs, P.sn, lp.ok, list, lane);
-    const T xib = P.cs * d[b] + P.sn * d[c] + pivot<T>(g, b), xic = P.cs * d[c] - P.sn * d[b] + pivot<T>(g, c);
+    const T xib = dot2(P.cs, d[b], P.sn, d[c]) + pivot<T>(g, b), xic = dot2(P.cs, d[c], -P.sn, d[b]) + pivot<T>(g, c);
     const Axial<T, AX> ax(g, d[a3]);
     int sb, sc, sa;
     design_strides<AX>(g, sb, sc, sa);

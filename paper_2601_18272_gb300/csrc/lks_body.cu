@@ -1360,9 +1360,9 @@ void launch_couple_last(const Geo& g, Ctrl* ctrl, Dof* it, const Moments* mom, c
 template <typename T>
 void launch_apply(const Geo& g, const Slots<T>& S, const Ctrl* ctrl, const Dof* it, const T* kref, T* boxstore,
                   int nbox, int di, cudaStream_t st) {
-  // the sums in the forward's order (bit for bit its state): the columns only where it takes them too
-  // (small boxes and the other coupling modes run k_couple)
-  if (g.flag_ctas > 0 && axis3d_fits(g)) return launch_apply_axis3d<T>(g, S, ctrl, it, kref, boxstore, nbox, di, st);
+  // the sums in the order of the forward that ran (bit for bit its state), whatever form the next one takes
+  if (g.fwd_form > 0 && g.dim == 2) return launch_apply_flag2d<T>(g, S, ctrl, it, kref, boxstore, nbox, di, st);
+  if (g.fwd_form > 0) return launch_apply_axis3d<T>(g, S, ctrl, it, kref, boxstore, nbox, di, st);
   LKS_BOX_DISPATCH(k_apply, box_grid(g), box_threads(g), g, S, ctrl, it, kref, boxstore, nbox, di);
 }
 

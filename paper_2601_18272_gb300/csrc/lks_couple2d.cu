@@ -35,10 +35,10 @@ constexpr int max_threads() { return sizeof(T) == 4 ? 640 : 512; }
 // the design frame: phi, kappa, sum W e, sum W kappa e; then moved to the pivot (sum W r).
 template <typename T>
 __device__ __forceinline__ void to_pivot(T xb, T xc, T eb, T ec, T kb, T kc, Acc<T>& o) {
-  o.wr[0] = eb + xb * o.phi;
-  o.wr[1] = ec + xc * o.phi;
-  o.kr[0] = kb + xb * o.kap;
-  o.kr[1] = kc + xc * o.kap;
+  o.wr[0] = fma_(xb, o.phi, eb);
+  o.wr[1] = fma_(xc, o.phi, ec);
+  o.kr[0] = fma_(xb, o.kap, kb);
+  o.kr[1] = fma_(xc, o.kap, kc);
   o.wr[2] = o.kr[2] = T(0);
 }
 
@@ -50,7 +50,7 @@ template <int LC>
 __device__ __forceinline__ void gather2d(const Geo& g, const float* __restrict__ kref, const float (&d)[2], float cs,
                                          float sn, int cl, bool active, Acc<float>& o) {
   const float S = (float)g.s, pad = 1e-3f, tiny = 1e-6f;
-  const float xb = cs * d[0] + sn * d[1], xc = cs * d[1] - sn * d[0];
+  const float xb = dot2(cs, d[0], sn, d[1]), xc = dot2(cs, d[1], -sn, d[0]);
   const float xib = xb + g.xicf[0], xic = xc + g.xicf[1];
   const float h = S * (fabsf(cs) + fabsf(sn));
   const int nx = g.nd[0];
@@ -87,7 +87,7 @@ __device__ __forceinline__ void gather2d(const Geo& g, const float* __restrict__
       float kv[6];
 #pragma unroll
       for (int j = 0; j < 6; ++j) kv[j] = __ldg(kr + min(j0 + j, j1));
-      const float ob0 = -nw * ec, oc0 = cw * ec;
+      const float ob0 = mul_(-nw, ec), oc0 = mul_(cw, ec);
       float ps = 0.0f, pk = 0.0f;
 #pragma unroll
       for (int j = 0; j < 6; ++j) {
@@ -96,9 +96,9 @@ __device__ __forceinline__ void gather2d(const Geo& g, const float* __restrict__
         const float ob = fmaf(cw, eb, ob0), oc = fmaf(nw, eb, oc0);
         bool ok = ib <= j1 && fabsf(ob) < Sw && fabsf(oc) < Sw;
         if (ball) ok = ok && dsq(ib, nx) + dsq(ic, g.nd[1]) <= g.rad4;
-        float w = cosine ? (1.0f + __cosf(ob)) * (1.0f + __cosf(oc)) : (1.0f - fabsf(ob)) * (1.0f - fabsf(oc));
+        float w = cosine ? mul_(1.0f + __cosf(ob), 1.0f + __cosf(oc)) : mul_(1.0f - fabsf(ob), 1.0f - fabsf(oc));
         w = ok ? w : 0.0f;
-        const float wk = w * kv[j];
+        const float wk = mul_(w, kv[j]);
         ps += w;
         pk += wk;
         sb = fmaf(w, eb, sb);
@@ -110,12 +110,12 @@ __device__ __forceinline__ void gather2d(const Geo& g, const float* __restrict__
       kc = fmaf(pk, ec, kc);
     }
     const float f = cosine ? 0.0625f : 1.0f;
-    phi *= f;
-    kap *= f;
-    sb *= f;
-    sc *= f;
-    kb *= f;
-    kc *= f;
+    phi = mul_(phi, f);
+    kap = mul_(kap, f);
+    sb = mul_(sb, f);
+    sc = mul_(sc, f);
+    kb = mul_(kb, f);
+    kc = mul_(kc, f);
   }
 #pragma unroll
   for (int off = 1; off < LC; off <<= 1) {
@@ -140,7 +140,7 @@ __device__ __forceinline__ void gather2d(const Geo& g, const double* __restrict_
                                          double cs, double sn, int cl, bool active, Acc<double>& o) {
   static_assert(LC == kLanes64, "a 4 x 4 pattern of lanes");
   const double S = (double)g.s;
-  const double xb = cs * d[0] + sn * d[1], xc = cs * d[1] - sn * d[0];
+  const double xb = dot2(cs, d[0], sn, d[1]), xc = dot2(cs, d[1], -sn, d[0]);
   const double xib = xb + g.xic[0], xic = xc + g.xic[1];
   const float csf = (float)cs, snf = (float)sn, pad = 2e-3f, Sp = (float)g.s + pad;
   const float xibf = (float)xib, xicf = (float)xic;
@@ -157,15 +157,15 @@ __device__ __forceinline__ void gather2d(const Geo& g, const double* __restrict_
       if (fabsf(csf * ebf - snf * ecf) >= Sp || fabsf(snf * ebf + csf * ecf) >= Sp) continue;
       if (dsq(ib, g.nd[0]) + dsq(ic, g.nd[1]) > g.rad4) continue;
       const double eb = (double)ib - xib, ec = (double)ic - xic;
-      const double ob = cs * eb - sn * ec, oc = sn * eb + cs * ec;
+      const double ob = dot2(cs, eb, -sn, ec), oc = dot2(sn, eb, cs, ec);
       if (fabs(ob) >= S || fabs(oc) >= S) continue;
-      const double w = wfun(g.wk, ob) * wfun(g.wk, oc), wk = w * kref[ib + ic * g.nd[0]];
+      const double w = mul_(wfun(g.wk, ob), wfun(g.wk, oc)), wk = mul_(w, kref[ib + ic * g.nd[0]]);
       v[0] += w;
       v[1] += wk;
-      v[2] += w * eb;
-      v[3] += w * ec;
-      v[4] += wk * eb;
-      v[5] += wk * ec;
+      v[2] = fma_(w, eb, v[2]);
+      v[3] = fma_(w, ec, v[3]);
+      v[4] = fma_(wk, eb, v[4]);
+      v[5] = fma_(wk, ec, v[5]);
     }
   // halving over lane bits 3, 2, 1 (value index bits 2, 1, 0), then the pair of bit 0
   const bool b3 = cl & 8, b2 = cl & 4, b1 = cl & 2;
@@ -181,6 +181,15 @@ __device__ __forceinline__ void gather2d(const Geo& g, const double* __restrict_
   const double sb = __shfl_sync(0xffffffffu, c, 4, 16), sc = __shfl_sync(0xffffffffu, c, 6, 16);
   const double kb = __shfl_sync(0xffffffffu, c, 8, 16), kc = __shfl_sync(0xffffffffu, c, 10, 16);
   to_pivot(xb, xc, sb, sc, kb, kc, o);
+}
+
+// u^S of a cell from its sums; returns 1 / (1 + kappa).
+template <typename T>
+__device__ __forceinline__ T solid_velocity(const Pose<T, 2>& P, const Acc<T>& A, T (&us)[2]) {
+  const T dwr[2] = {-dot2(P.sn, A.wr[0], P.cs, A.wr[1]), dot2(P.cs, A.wr[0], -P.sn, A.wr[1])};
+#pragma unroll
+  for (int a = 0; a < 2; ++a) us[a] = dot2(P.ug[a], A.phi, P.om, dwr[a]);
+  return T(1) / (T(1) + A.kap);
 }
 
 template <typename T, int LC>
@@ -263,16 +272,13 @@ __global__ void __launch_bounds__(max_threads<T>(), 1)
       }
       if (n < 0 || forbidden<2>(g, cc.px, cc.py, 0)) atomicOr(&ctrl->status, ST_BODY_OUTSIDE);
       if (n < 0) continue;
-      T dwr[3], L[3];
-      drot<2>(P.cs, P.sn, A.wr, dwr);
+      T L[3], u[2], us[2];
       rot<2>(P.cs, P.sn, A.kr, L);
-      const T inv = T(1) / (T(1) + A.kap);
-      T u[2];
+      const T inv = solid_velocity(P, A, us);
 #pragma unroll
       for (int a = 0; a < 2; ++a) {
-        const T us = P.ug[a] * A.phi + P.om * dwr[a];
         const T ustar = c0 == first ? ust0[a] : dst[(a + 1) * N + n];
-        u[a] = (ustar + A.kap * us) * inv;
+        u[a] = brinkman(ustar, A.kap, us[a], inv);
         v[a] += A.kap * u[a];
         if (last) {
           if (bs) bs[a * g.box_cells + bl] = ustar;
@@ -303,6 +309,47 @@ __global__ void __launch_bounds__(max_threads<T>(), 1)
     if (last) return;
     __syncthreads();
     if (gave_up) return;
+  }
+}
+
+// Recompute of one step's Brinkman update from the stored iterate s^(K-1), by the forward's gather with
+// its lanes, so that the recomputed state is the forward's to the bit (k_apply of lks_body.cu sums a cell's
+// points in another order and goes with k_couple).
+constexpr int kApplyThreads = 128;
+template <typename T, int LC>
+__global__ void __launch_bounds__(kApplyThreads) k_apply_flag(Geo g, Slots<T> S, const Ctrl* ctrl, const Dof* it,
+                                                              const T* __restrict__ kref, T* __restrict__ boxstore,
+                                                              int nbox, int di) {
+  const int t = ctrl->t0 + di, base = ctrl->base, K = g.K;
+  const Dof* row = it + (long long)(t - 1) * (K + 1);
+  Pose<T, 2> P;
+  P.set(row[K - 1]);
+  T* __restrict__ dst = slot_ptr(S, t, base);
+  T* bs = boxstore + (long long)((t - base - 1) % nbox) * g.box_cells * 2;
+  int lo[3];
+  box_origin<2>(g, row[0], lo[0], lo[1], lo[2]);
+  const long long N = g.N;
+  const unsigned q = blockIdx.x * (unsigned)kApplyThreads + threadIdx.x;
+  const int bl = (int)(q / LC), cl = (int)(q % LC);
+  const bool in = bl < (int)g.box_cells;
+  const int j1 = bl / g.B[0], px = lo[0] + bl - j1 * g.B[0], py = lo[1] + j1;
+  long long n = 0;
+  const bool ing = in && cell_index<2>(g, px, py, 0, n);
+  T ust[2] = {T(0), T(0)};
+  if (ing) {
+    ust[0] = dst[N + n];
+    ust[1] = dst[2 * N + n];
+  }
+  const T d[2] = {P.rel(0, px), P.rel(1, py)};
+  Acc<T> A;
+  gather2d<LC>(g, kref, d, P.cs, P.sn, cl, in, A);
+  if (!ing || cl != 0) return;
+  T us[2];
+  const T inv = solid_velocity(P, A, us);
+#pragma unroll
+  for (int a = 0; a < 2; ++a) {
+    bs[a * g.box_cells + bl] = ust[a];
+    if (A.phi != T(0)) dst[(a + 1) * N + n] = brinkman(ust[a], A.kap, us[a], inv);
   }
 }
 
@@ -366,6 +413,25 @@ void launch_couple_flag(const Geo& g, const Slots<T>& S, Ctrl* ctrl, Dof* it, co
     run(k_couple_flag<float, 2>);
 }
 
+template <typename T>
+void launch_apply_flag2d(const Geo& g, const Slots<T>& S, const Ctrl* ctrl, const Dof* it, const T* kref, T* boxstore,
+                         int nbox, int di, cudaStream_t st) {
+  auto run = [&](auto kernel, int lanes) {
+    launch(kernel, dim3((unsigned)((g.box_cells * lanes + kApplyThreads - 1) / kApplyThreads)), kApplyThreads, 0, st, g, S,
+           ctrl, it, kref, boxstore, nbox, di);
+  };
+  if constexpr (sizeof(T) == 8)
+    run(k_apply_flag<double, kLanes64>, kLanes64);
+  else if (g.fwd_form == 1)
+    run(k_apply_flag<float, 1>, 1);
+  else
+    run(k_apply_flag<float, 2>, 2);
+}
+
+template void launch_apply_flag2d<float>(const Geo&, const Slots<float>&, const Ctrl*, const Dof*, const float*, float*,
+                                         int, int, cudaStream_t);
+template void launch_apply_flag2d<double>(const Geo&, const Slots<double>&, const Ctrl*, const Dof*, const double*,
+                                          double*, int, int, cudaStream_t);
 template void launch_couple_flag<float>(const Geo&, const Slots<float>&, Ctrl*, Dof*, const float*, const Moments*,
                                         void*, float*, int, int, cudaStream_t);
 template void launch_couple_flag<double>(const Geo&, const Slots<double>&, Ctrl*, Dof*, const double*, const Moments*,

@@ -164,6 +164,9 @@ struct Geo {
   int margin;     // cells of drift allowed within one step
   long long box_cells;
   int flag_ctas, flag_threads, flag_lanes;  // shape of the flag-exchange coupling kernels (0: another form runs)
+  // form of the gather in the forward that last ran, which the recompute of its steps follows bit for bit: the
+  // lanes per cell of k_couple_flag (2D) or 1 for k_couple_axis3d; 0: gather_cell (k_couple, k_couple_coop)
+  int fwd_form;
   int free_tiled;  // free rotation, FP32, cosine kernel: the tiled reverse kernels may run (lks_free3d.cu)
   int coop_fwd, coop_adj;  // CTAs of the cooperative coupling kernels (0: the per-iteration kernels)
 };

@@ -20,6 +20,19 @@ namespace lks {
 
 namespace {
 
+// Roundings spelled out where a forward kernel and its recompute must agree to the bit: how the compiler
+// joins the products and sums of an expression into multiply-adds is its own choice in each kernel.
+__device__ __forceinline__ float fma_(float a, float b, float c) { return fmaf(a, b, c); }
+__device__ __forceinline__ double fma_(double a, double b, double c) { return fma(a, b, c); }
+__device__ __forceinline__ float mul_(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ double mul_(double a, double b) { return __dmul_rn(a, b); }
+// a b + c d
+template <typename T>
+__device__ __forceinline__ T dot2(T a, T b, T c, T d) { return fma_(a, b, mul_(c, d)); }
+// The Brinkman update of a cell: (u* + kappa u^S) / (1 + kappa), inv the reciprocal.
+template <typename T>
+__device__ __forceinline__ T brinkman(T ustar, T kap, T us, T inv) { return mul_(fma_(kap, us, ustar), inv); }
+
 // One value as two 64-bit words (number << 32 | payload) and back.
 struct Words {
   unsigned long long a, b;

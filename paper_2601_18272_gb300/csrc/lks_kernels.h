@@ -139,6 +139,10 @@ size_t couple_flag_bytes(int ctas);
 template <typename T>
 void launch_couple_flag(const Geo& g, const Slots<T>& S, Ctrl* ctrl, Dof* it, const T* kref, const Moments* mom,
                         void* words, T* boxstore, int nbox, int di, cudaStream_t st);
+// Recompute of a step whose forward ran the 2D form (g.fwd_form lanes per cell).
+template <typename T>
+void launch_apply_flag2d(const Geo& g, const Slots<T>& S, const Ctrl* ctrl, const Dof* it, const T* kref, T* boxstore,
+                         int nbox, int di, cudaStream_t st);
 
 // 3D forms about one rotation axis (lks_axis3d.cu). setup and launch of the coupling are reached
 // through setup_couple_flag and launch_couple_flag, the coefficient and design kernels through
