@@ -253,7 +253,8 @@ LKS_API int lks_get_initial_adjoint(lks_handle* h, double* lam_p_host, double* l
  * accepts (|x_n - x^ref_m| below the kernel's half-width on every axis, m in the design domain):
  * stats_host [box cells][5] = (count, least linear design index or -1, largest index, sum of the
  * indices, sum of their squares), capacity in values (at least 5 * box cells, else LKS_ERR_ARG).
- * The acceptance is decided in the field precision of the handle. Synchronous (legacy default
+ * The acceptance is decided by the gather of the coupling form that a march from s would take
+ * (lks_persistent_coupling), in the field precision of the handle. Synchronous (legacy default
  * stream; allocates and frees a small device buffer). Errors: LKS_ERR_NONFINITE (s not finite),
  * LKS_ERR_UNSUPPORTED (s rotated but the workspace holds an axis-aligned box), LKS_ERR_CUDA. */
 LKS_API int lks_support_sets(lks_handle* h, const double* s_host, int* box_host, long long* stats_host,

@@ -1444,6 +1444,9 @@ int lks_support_sets(lks_handle* h, const double* s_host, int* box_host, long lo
   const bool rotated = (g.dof_mask & LKS_DOF_ROT) || start_rotated;
   if (rotated && !h->box_rot_ok) return LKS_ERR_UNSUPPORTED;
   setup_box(&g, h->P.design_radius, rotated);
+  // and the form its forward would take
+  g.flag_ctas = g.flag_threads = 0;
+  if (h->coop_mode == 2 && !h->no_words) setup_couple_flag(&g, h->prec == LKS_FP64);
   for (int a = 0; a < 3; ++a) {
     box_host[a] = (a < g.dim) ? d.xi[a] - g.hb[a] - g.s - g.margin : 0;
     box_host[3 + a] = g.B[a];

@@ -19,6 +19,7 @@
 //   k_coef_axis3d    the sums of the reverse by linear maps (k_rev_coef of lks_reverse.cu)
 //   k_design_axis3d  its dJ/dkappa^ref: a lane takes one column of design points and ZD of them
 #include <climits>
+#include <type_traits>
 
 #include "lks_flag.cuh"
 #include "lks_reverse.cuh"
@@ -133,6 +134,7 @@ struct Column {
 template <typename T, int AX>
 struct Axial {
   T w[4], dw[4];
+  bool in[4];  // the tap lies within the support
   int ia0;
   __device__ __forceinline__ Axial(const Geo& g, T da) {
     constexpr int a = Axes<AX>::A;
@@ -142,7 +144,8 @@ struct Axial {
     for (int q = 0; q < 4; ++q) {
       const T o = fr + (T)(g.s - 1 - q);  // x_n - x^ref along the axis
       w[q] = dw[q] = T(0);
-      if (q < 2 * g.s && fabs(o) < S) {
+      in[q] = q < 2 * g.s && fabs(o) < S;
+      if (in[q]) {
         if constexpr (sizeof(T) == 8) {
           if (g.wk == W_COS4) {
             double s, c;
@@ -185,9 +188,12 @@ template <typename T, int Z>
 struct PlaneSums {
   T phi[Z], kap[Z], Pb[Z], Pc[Z], Lb[Z], Lc[Z];
 };
-template <typename T, int AX, bool BALL, int Z>
+// visit (a test export): called with the plane and the linear index of each design point that is summed.
+struct NoPlaneVisit {};
+template <typename T, int AX, bool BALL, int Z, typename Visit = NoPlaneVisit>
 __device__ __forceinline__ void plane_sums(const Geo& g, const T* __restrict__ kref, const T (&d)[3], T cs, T sn, int n,
-                                           const unsigned (*list)[32], int lane, PlaneSums<T, Z>& o) {
+                                           const unsigned (*list)[32], int lane, PlaneSums<T, Z>& o,
+                                           Visit visit = Visit()) {
   constexpr int b = Axes<AX>::B, c = Axes<AX>::C, a = Axes<AX>::A;
   const T xib = dot2(cs, d[b], sn, d[c]) + pivot<T>(g, b), xic = dot2(cs, d[c], -sn, d[b]) + pivot<T>(g, c);
   const Axial<T, AX> ax(g, d[a]);
@@ -214,6 +220,13 @@ __device__ __forceinline__ void plane_sums(const Geo& g, const T* __restrict__ k
     const T wb = mul_(w2, q.lb), wc = mul_(w2, q.lc);
     int left = 0;
     if (BALL) left = g.rad4 - dsq(q.ib, g.nd[b]) - dsq(q.ic, g.nd[c]);
+    if constexpr (!std::is_same_v<Visit, NoPlaneVisit>)
+      for (int j = 0; j < Z; ++j)
+        for (int m = 0; m < 4; ++m) {
+          const int ia = ax.ia0 + j + m;
+          if (ax.in[m] && ia >= 0 && ia < g.nd[a] && (!BALL || dsq(ia, g.nd[a]) <= left))
+            visit(j, q.ib * sb + q.ic * sc + ia * sa);
+        }
     if (!BALL) {
       f2 += w2;
       pb2 += wb;
@@ -459,6 +472,31 @@ __global__ void __launch_bounds__(kApplyWarps * 32) k_apply_axis3d(Geo g, Slots<
       if (body) dst[(a + 1) * g.N + lc.at(j)] = brinkman(us[j][a], A.kap[j], sv, inv);
     }
   }
+}
+
+// The box of the iterate s, gathered as k_couple_axis3d does, with the accepted index sets as out[box cell][5].
+template <typename T, int AX, bool BALL>
+__global__ void __launch_bounds__(kApplyWarps * 32) k_support_axis3d(Geo g, Dof s, const T* __restrict__ kref,
+                                                                     long long* __restrict__ out) {
+  constexpr int Z = Planes<T>::ZC, a3 = Axes<AX>::A;
+  __shared__ unsigned lists[kApplyWarps][kListMax][32];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int u0 = blockIdx.x * kApplyWarps + warp, tiles = plane_tiles<AX>(g);
+  if (u0 >= plane_units<AX>(g, Z)) return;
+  int lo[3];
+  box_origin<3>(g, s, lo[0], lo[1], lo[2]);
+  const DofView<T> P(s);
+  const LanePos lp = lane_pos<AX>(g, u0, tiles, Z, lane);
+  const T d[3] = {P.rel(0, lo[0] + lp.j[0]), P.rel(1, lo[1] + lp.j[1]), P.rel(2, lo[2] + lp.j[2])};
+  const int n = column_list<T, AX>(g, d, P.cs, P.sn, lp.ok, lists[warp], lane);
+  SetStats st[Z];
+  PlaneSums<T, Z> A;
+  auto visit = [&](int j, int m) { st[j].add(m); };
+  plane_sums<T, AX, BALL, Z>(g, kref, d, P.cs, P.sn, n, lists[warp], lane, A, visit);
+  const int sbx = a3 == 0 ? 1 : (a3 == 1 ? g.B[0] : g.B[0] * g.B[1]);
+  const long long bl0 = lp.j[0] + (long long)g.B[0] * (lp.j[1] + (long long)g.B[1] * lp.j[2]);
+  for (int j = 0; j < Z; ++j)
+    if (lp.ok && lp.j[a3] + j < g.B[a3]) st[j].store(out, bl0 + (long long)j * sbx);
 }
 
 // The planes and sums of k_rev_coef (whole design domain; a ball takes that kernel). Sums over the
@@ -767,6 +805,12 @@ void apply_ax(const Geo& g, const Slots<T>& S, const Ctrl* ctrl, const Dof* it, 
   launch(k_apply_axis3d<T, AX, BALL>, dim3((unsigned)((units + kApplyWarps - 1) / kApplyWarps)), kApplyWarps * 32, 0, st,
          g, S, ctrl, it, kref, boxstore, nbox, di);
 }
+template <typename T, int AX, bool BALL>
+void support_ax(const Geo& g, const Dof& s, const T* kref, long long* out, cudaStream_t st) {
+  const long long units = plane_units<AX>(g, Planes<T>::ZC);
+  launch(k_support_axis3d<T, AX, BALL>, dim3((unsigned)((units + kApplyWarps - 1) / kApplyWarps)), kApplyWarps * 32, 0, st,
+         g, s, kref, out);
+}
 template <typename T, int AX>
 int coef_ctas_ax(const Geo& g) {
   const long long units = plane_units<AX>(g, Planes<T>::ZR);
@@ -824,6 +868,11 @@ void launch_apply_axis3d(const Geo& g, const Slots<T>& S, const Ctrl* ctrl, cons
   LKS_AXIS_BALL(apply_ax, g, S, ctrl, it, kref, boxstore, nbox, di, st);
 }
 
+template <typename T>
+void launch_support_axis3d(const Geo& g, const Dof& s, const T* kref, long long* out, cudaStream_t st) {
+  LKS_AXIS_BALL(support_ax, g, s, kref, out, st);
+}
+
 bool coef_axis3d_fits(const Geo& g) { return axis3d_fits(g) && g.rad4 == INT_MAX; }
 int coef_axis3d_ctas(const Geo& g, bool fp64) {
   if (fp64) return g.ax == 0 ? coef_ctas_ax<double, 0>(g) : g.ax == 1 ? coef_ctas_ax<double, 1>(g) : coef_ctas_ax<double, 2>(g);
@@ -845,6 +894,7 @@ void launch_design_axis3d(const Geo& g, const RevBuffers& R, Ctrl* ctrl, const D
                                         int, int, cudaStream_t);                                                      \
   template void launch_apply_axis3d<T>(const Geo&, const Slots<T>&, const Ctrl*, const Dof*, const T*, T*, int, int,   \
                                        cudaStream_t);                                                                 \
+  template void launch_support_axis3d<T>(const Geo&, const Dof&, const T*, long long*, cudaStream_t);                   \
   template void launch_coef_axis3d<T>(const Geo&, const RevBuffers&, const Ctrl*, const Dof*, const T*, const T*, int, \
                                       int, int, cudaStream_t);                                                        \
   template void launch_design_axis3d<T>(const Geo&, const RevBuffers&, Ctrl*, const Dof*, int, int, cudaStream_t);

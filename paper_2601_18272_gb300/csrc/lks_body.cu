@@ -1187,22 +1187,6 @@ __global__ void __launch_bounds__(BoxCta<D>::threads, 1)
 
 // ---- index sets of the spread (test export) -------------------------------------------------
 
-// Per box cell: the number of design points the gather accepts, the least and largest of their
-// linear indices, and the sums of the indices and of their squares.
-struct SetStats {
-  long long c, lo, hi, s1, s2;
-};
-struct StatVisit {
-  SetStats* st;
-  __device__ __forceinline__ void operator()(int m) const {
-    st->c += 1;
-    st->lo = min(st->lo, (long long)m);
-    st->hi = max(st->hi, (long long)m);
-    st->s1 += m;
-    st->s2 += (long long)m * m;
-  }
-};
-
 // The box of the iterate s (the box a step starting from s would use), gathered as the coupling
 // gathers it, recording the accepted index sets into out[box cell][5].
 template <typename T, int D, int AX>
@@ -1214,7 +1198,7 @@ __global__ void __launch_bounds__(BoxCta<D>::threads) k_support_sets(Geo g, Dof 
   const int px = lo[0] + cc.j0, py = lo[1] + cc.j1, pz = lo[2] + cc.j2;
   const DofView<T> V(s);
   const T d[3] = {V.rel(0, px), V.rel(1, py), D == 3 ? V.rel(2, pz) : T(0)};
-  SetStats st{0, LLONG_MAX, -1, 0, 0};
+  SetStats st;
   Acc<T> A;
   if constexpr (AX == AX_FREE) {
     const FreeView<T> FV(s);
@@ -1222,21 +1206,9 @@ __global__ void __launch_bounds__(BoxCta<D>::threads) k_support_sets(Geo g, Dof 
   } else {
     gather_lanes<T, D, AX, LN>(g, kref, d, V.cs, V.sn, cc.lane, cc.active, A, StatVisit{&st});
   }
-#pragma unroll
-  for (int off = 1; off < LN; off <<= 1) {
-    st.c += __shfl_xor_sync(0xffffffffu, st.c, off);
-    st.lo = min(st.lo, __shfl_xor_sync(0xffffffffu, st.lo, off));
-    st.hi = max(st.hi, __shfl_xor_sync(0xffffffffu, st.hi, off));
-    st.s1 += __shfl_xor_sync(0xffffffffu, st.s1, off);
-    st.s2 += __shfl_xor_sync(0xffffffffu, st.s2, off);
-  }
+  st.lanes<LN>();
   if (!cc.active || cc.lane != 0) return;
-  const long long bl = cc.j0 + (long long)g.B[0] * (cc.j1 + (long long)g.B[1] * cc.j2);
-  out[5 * bl + 0] = st.c;
-  out[5 * bl + 1] = st.c ? st.lo : -1;
-  out[5 * bl + 2] = st.hi;
-  out[5 * bl + 3] = st.s1;
-  out[5 * bl + 4] = st.s2;
+  st.store(out, cc.j0 + (long long)g.B[0] * (cc.j1 + (long long)g.B[1] * cc.j2));
 }
 
 }  // namespace
@@ -1323,6 +1295,8 @@ void setup_coop(Geo* g, bool fp64) {
 
 template <typename T>
 void launch_support_sets(const Geo& g, const Dof& s, const T* kref, long long* out, cudaStream_t st) {
+  if (g.flag_ctas > 0 && g.dim == 2) return launch_support_flag2d<T>(g, s, kref, out, st);
+  if (g.flag_ctas > 0) return launch_support_axis3d<T>(g, s, kref, out, st);
   LKS_BOX_DISPATCH(k_support_sets, box_grid(g), box_threads(g), g, s, kref, out);
 }
 

@@ -3,6 +3,8 @@
 // dispatch on the dimension and rotation axis.
 #pragma once
 
+#include <climits>
+
 #include "lks_kernels.h"
 
 namespace lks {
@@ -121,6 +123,43 @@ inline int design_ctas(const Geo& g) {
   const int n = (g.ND + kDesignPointsPerCta - 1) / kDesignPointsPerCta;
   return n < kMaxDesignCtas ? n : kMaxDesignCtas;
 }
+
+// Index sets of the spread (test export). Per box cell: the number of design points the gather accepts, the least
+// and largest of their linear indices, and the sums of the indices and of their squares.
+struct SetStats {
+  long long c = 0, lo = LLONG_MAX, hi = -1, s1 = 0, s2 = 0;
+  __device__ __forceinline__ void add(int m) {
+    c += 1;
+    lo = min(lo, (long long)m);
+    hi = max(hi, (long long)m);
+    s1 += m;
+    s2 += (long long)m * m;
+  }
+  // over the LC lanes of a cell
+  template <int LC>
+  __device__ __forceinline__ void lanes() {
+#pragma unroll
+    for (int off = 1; off < LC; off <<= 1) {
+      c += __shfl_xor_sync(0xffffffffu, c, off);
+      lo = min(lo, __shfl_xor_sync(0xffffffffu, lo, off));
+      hi = max(hi, __shfl_xor_sync(0xffffffffu, hi, off));
+      s1 += __shfl_xor_sync(0xffffffffu, s1, off);
+      s2 += __shfl_xor_sync(0xffffffffu, s2, off);
+    }
+  }
+  __device__ __forceinline__ void store(long long* out, long long bl) const {
+    out += 5 * bl;
+    out[0] = c;
+    out[1] = c ? lo : -1;
+    out[2] = hi;
+    out[3] = s1;
+    out[4] = s2;
+  }
+};
+struct StatVisit {
+  SetStats* st;
+  __device__ __forceinline__ void operator()(int m) const { st->add(m); }
+};
 
 __host__ __device__ inline int box_threads(const Geo& g) { return kBoxCtaCellsX * (g.dim == 2 ? kBoxCtaCellsY2D : kBoxCtaCellsY) * LN; }
 __host__ __device__ inline dim3 box_grid(const Geo& g) {

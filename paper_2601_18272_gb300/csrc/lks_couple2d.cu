@@ -46,9 +46,9 @@ __device__ __forceinline__ void to_pivot(T xb, T xc, T eb, T ec, T kb, T kc, Acc
 // follows from the two support bounds (linear in the offset), widened, and the exact test decides.
 // Cosine kernel: with the rotation scaled by pi/2 the offsets are the cosines' arguments; the factor
 // 1/16 of the two weights is applied to the sums.
-template <int LC>
+template <int LC, typename Visit = NoVisit>
 __device__ __forceinline__ void gather2d(const Geo& g, const float* __restrict__ kref, const float (&d)[2], float cs,
-                                         float sn, int cl, bool active, Acc<float>& o) {
+                                         float sn, int cl, bool active, Acc<float>& o, Visit visit = Visit()) {
   const float S = (float)g.s, pad = 1e-3f, tiny = 1e-6f;
   const float xb = dot2(cs, d[0], sn, d[1]), xc = dot2(cs, d[1], -sn, d[0]);
   const float xib = xb + g.xicf[0], xic = xc + g.xicf[1];
@@ -98,6 +98,7 @@ __device__ __forceinline__ void gather2d(const Geo& g, const float* __restrict__
         if (ball) ok = ok && dsq(ib, nx) + dsq(ic, g.nd[1]) <= g.rad4;
         float w = cosine ? mul_(1.0f + __cosf(ob), 1.0f + __cosf(oc)) : mul_(1.0f - fabsf(ob), 1.0f - fabsf(oc));
         w = ok ? w : 0.0f;
+        if (ok) visit(ib + ic * nx);
         const float wk = mul_(w, kv[j]);
         ps += w;
         pk += wk;
@@ -135,9 +136,9 @@ __device__ __forceinline__ void gather2d(const Geo& g, const float* __restrict__
 // square; the test against the support is made in FP32 first (widened by more than its rounding),
 // so FP64 instructions are spent on accepted candidates only. The six sums of the 16 lanes are
 // combined by halving (each level exchanges half of the values: 8 additions, not 24).
-template <int LC>
+template <int LC, typename Visit = NoVisit>
 __device__ __forceinline__ void gather2d(const Geo& g, const double* __restrict__ kref, const double (&d)[2],
-                                         double cs, double sn, int cl, bool active, Acc<double>& o) {
+                                         double cs, double sn, int cl, bool active, Acc<double>& o, Visit visit = Visit()) {
   static_assert(LC == kLanes64, "a 4 x 4 pattern of lanes");
   const double S = (double)g.s;
   const double xb = dot2(cs, d[0], sn, d[1]), xc = dot2(cs, d[1], -sn, d[0]);
@@ -159,6 +160,7 @@ __device__ __forceinline__ void gather2d(const Geo& g, const double* __restrict_
       const double eb = (double)ib - xib, ec = (double)ic - xic;
       const double ob = dot2(cs, eb, -sn, ec), oc = dot2(sn, eb, cs, ec);
       if (fabs(ob) >= S || fabs(oc) >= S) continue;
+      visit(ib + ic * g.nd[0]);
       const double w = mul_(wfun(g.wk, ob), wfun(g.wk, oc)), wk = mul_(w, kref[ib + ic * g.nd[0]]);
       v[0] += w;
       v[1] += wk;
@@ -353,6 +355,24 @@ __global__ void __launch_bounds__(kApplyThreads) k_apply_flag(Geo g, Slots<T> S,
   }
 }
 
+// The box of the iterate s, gathered as k_couple_flag does, with the accepted index sets as out[box cell][5].
+template <typename T, int LC>
+__global__ void __launch_bounds__(kApplyThreads) k_support_flag(Geo g, Dof s, const T* __restrict__ kref,
+                                                                long long* __restrict__ out) {
+  Pose<T, 2> P;
+  P.set(s);
+  int lo[3];
+  box_origin<2>(g, s, lo[0], lo[1], lo[2]);
+  const unsigned q = blockIdx.x * (unsigned)kApplyThreads + threadIdx.x;
+  const int bl = (int)(q / LC), cl = (int)(q % LC), j1 = bl / g.B[0];
+  const T d[2] = {P.rel(0, lo[0] + bl - j1 * g.B[0]), P.rel(1, lo[1] + j1)};
+  SetStats st;
+  Acc<T> A;
+  gather2d<LC>(g, kref, d, P.cs, P.sn, cl, bl < (int)g.box_cells, A, StatVisit{&st});
+  st.lanes<LC>();
+  if (bl < (int)g.box_cells && cl == 0) st.store(out, bl);
+}
+
 // CTAs and threads of the kernel with LC lanes; *passes: cells per thread.
 template <typename T, int LC>
 int flag_shape(const Geo& g, int* threads, long long* passes) {
@@ -413,12 +433,17 @@ void launch_couple_flag(const Geo& g, const Slots<T>& S, Ctrl* ctrl, Dof* it, co
     run(k_couple_flag<float, 2>);
 }
 
+namespace {
+unsigned apply_ctas(const Geo& g, int lanes) {
+  return (unsigned)((g.box_cells * lanes + kApplyThreads - 1) / kApplyThreads);
+}
+}  // namespace
+
 template <typename T>
 void launch_apply_flag2d(const Geo& g, const Slots<T>& S, const Ctrl* ctrl, const Dof* it, const T* kref, T* boxstore,
                          int nbox, int di, cudaStream_t st) {
   auto run = [&](auto kernel, int lanes) {
-    launch(kernel, dim3((unsigned)((g.box_cells * lanes + kApplyThreads - 1) / kApplyThreads)), kApplyThreads, 0, st, g, S,
-           ctrl, it, kref, boxstore, nbox, di);
+    launch(kernel, dim3(apply_ctas(g, lanes)), kApplyThreads, 0, st, g, S, ctrl, it, kref, boxstore, nbox, di);
   };
   if constexpr (sizeof(T) == 8)
     run(k_apply_flag<double, kLanes64>, kLanes64);
@@ -428,6 +453,19 @@ void launch_apply_flag2d(const Geo& g, const Slots<T>& S, const Ctrl* ctrl, cons
     run(k_apply_flag<float, 2>, 2);
 }
 
+template <typename T>
+void launch_support_flag2d(const Geo& g, const Dof& s, const T* kref, long long* out, cudaStream_t st) {
+  auto run = [&](auto kernel, int lanes) { launch(kernel, dim3(apply_ctas(g, lanes)), kApplyThreads, 0, st, g, s, kref, out); };
+  if constexpr (sizeof(T) == 8)
+    run(k_support_flag<double, kLanes64>, kLanes64);
+  else if (g.flag_lanes == 1)
+    run(k_support_flag<float, 1>, 1);
+  else
+    run(k_support_flag<float, 2>, 2);
+}
+
+template void launch_support_flag2d<float>(const Geo&, const Dof&, const float*, long long*, cudaStream_t);
+template void launch_support_flag2d<double>(const Geo&, const Dof&, const double*, long long*, cudaStream_t);
 template void launch_apply_flag2d<float>(const Geo&, const Slots<float>&, const Ctrl*, const Dof*, const float*, float*,
                                          int, int, cudaStream_t);
 template void launch_apply_flag2d<double>(const Geo&, const Slots<double>&, const Ctrl*, const Dof*, const double*,

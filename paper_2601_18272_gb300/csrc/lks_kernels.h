@@ -144,6 +144,12 @@ template <typename T>
 void launch_apply_flag2d(const Geo& g, const Slots<T>& S, const Ctrl* ctrl, const Dof* it, const T* kref, T* boxstore,
                          int nbox, int di, cudaStream_t st);
 
+// launch_support_sets for the gathers of these forms.
+template <typename T>
+void launch_support_flag2d(const Geo& g, const Dof& s, const T* kref, long long* out, cudaStream_t st);
+template <typename T>
+void launch_support_axis3d(const Geo& g, const Dof& s, const T* kref, long long* out, cudaStream_t st);
+
 // 3D forms about one rotation axis (lks_axis3d.cu). setup and launch of the coupling are reached
 // through setup_couple_flag and launch_couple_flag, the coefficient and design kernels through
 // launch_rev_coef and launch_rev_design.
@@ -219,8 +225,8 @@ template <typename T>
 void launch_design_axis3d(const Geo& g, const RevBuffers& R, Ctrl* ctrl, const Dof* it, int nsteps, int di,
                           cudaStream_t st);
 
-// Test export: the design points the coupling's gather accepts for each cell of the box of the
-// iterate s, as out[box cell][5] = (count, least index or -1, largest index, sum, sum of squares).
+// Test export: the design points the coupling's gather (the form of g.flag_ctas) accepts for each cell of
+// the box of the iterate s, as out[box cell][5] = (count, least index or -1, largest index, sum, sum of squares).
 template <typename T>
 void launch_support_sets(const Geo& g, const Dof& s, const T* kref, long long* out, cudaStream_t st);
 
