@@ -321,14 +321,6 @@ __device__ __forceinline__ T solid_velocity(int a, const U& ug, T om, T phi, T P
   return a == b ? dot2(ug[a], phi, -om, Pc) : (a == c ? dot2(ug[a], phi, om, Pb) : mul_(ug[a], phi));
 }
 
-// A running sum of FP32 values as a double-float pair, or of doubles.
-__device__ __forceinline__ void run_add(Df& s, float b) {
-  const float t = s.hi + b, bb = t - s.hi;
-  s.lo += (s.hi - (t - bb)) + (b - bb);
-  s.hi = t;
-}
-__device__ __forceinline__ void run_add(Dd& s, double b) { s.v += b; }
-
 template <typename T, int AX, bool BALL>
 __global__ void __launch_bounds__(512, 1)
     k_couple_axis3d(Geo g, Slots<T> S, Ctrl* ctrl, Dof* it, const T* __restrict__ kref,
@@ -502,8 +494,11 @@ __global__ void __launch_bounds__(kApplyWarps * 32) k_support_axis3d(Geo g, Dof 
 // The planes and sums of k_rev_coef (whole design domain; a ball takes that kernel). Sums over the
 // design columns per plane, of kappa: with W, dW/db, dW/dc times 1, l_b, l_c, with dW/da likewise, and
 // the rotation derivative times l_b, l_c; without kappa the planes share the in-plane sums.
+// A thread's planes are added as pairs (packed FP32). FP32 runs two CTAs per SM (128 registers): with 22 more
+// for the pairs, one CTA of 184 took 90 us a step of the 48^3 body (planes and matrices together) and left the
+// chain's kernels no place beside it; two take 70, against 80 before the pairs (170 registers, FP32 sums).
 template <typename T, int AX>
-__global__ void __launch_bounds__(kRevThreads) k_coef_axis3d(Geo g, const Ctrl* ctrl, const Dof* it,
+__global__ void __launch_bounds__(kRevThreads, sizeof(T) == 4 ? 2 : 1) k_coef_axis3d(Geo g, const Ctrl* ctrl, const Dof* it,
                                                              const T* __restrict__ kref,
                                                              const T* __restrict__ boxstore, int nbox,
                                                              T* __restrict__ slabs, long long slab,
@@ -517,9 +512,9 @@ __global__ void __launch_bounds__(kRevThreads) k_coef_axis3d(Geo g, const Ctrl* 
   const Dof* row = it + (long long)(t - 1) * (K + 1);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int u0 = blockIdx.x * NW + warp, tiles = plane_tiles<AX>(g);
-  T v[RS::N];
+  typename SumOf<T>::type v[RS::N];
 #pragma unroll
-  for (int q = 0; q < RS::N; ++q) v[q] = T(0);
+  for (int q = 0; q < RS::N; ++q) v[q].zero();
   if (u0 < plane_units<AX>(g, Z)) {
     int lo[3];
     box_origin<3>(g, row[0], lo[0], lo[1], lo[2]);
@@ -627,7 +622,14 @@ __global__ void __launch_bounds__(kRevThreads) k_coef_axis3d(Geo g, const Ctrl* 
       T one[RS::N];
       rev_cell<T, 3, AX>(g, P, A, ing, bs, bl, slabs + (long long)i * slab + bl, k, one);
 #pragma unroll
-      for (int q = 0; q < RS::N; ++q) v[q] += one[q];
+      for (int q = 0; q < RS::N; q += 2) {
+        if (j == 0) {
+          v[q].set(one[q]);
+          v[q + 1].set(one[q + 1]);
+        } else {
+          run_add2(v[q], v[q + 1], one[q], one[q + 1]);
+        }
+      }
     }
   }
   row_sums<RS::N>(v, reinterpret_cast<T*>(rev_smem),
@@ -819,7 +821,7 @@ int coef_ctas_ax(const Geo& g) {
 template <typename T, int AX>
 void coef_ax(const Geo& g, const RevBuffers& R, const Ctrl* ctrl, const Dof* it, const T* kref, const T* boxstore, int nbox,
              int nsteps, int di, cudaStream_t st) {
-  const size_t rows = (size_t)RevSums<3>::N * (kRevThreads + 1) * sizeof(T), lists = list_bytes(kRevThreads / 32);
+  const size_t rows = row_bytes<T>(RevSums<3>::N), lists = list_bytes(kRevThreads / 32);
   launch(k_coef_axis3d<T, AX>, dim3((unsigned)coef_ctas_ax<T, AX>(g), g.K, nsteps), kRevThreads, rows > lists ? rows : lists,
          st, g, ctrl, it, kref, boxstore, nbox, (T*)R.slabs, R.slab, (typename Partial<T>::type*)R.mpart, di);
 }

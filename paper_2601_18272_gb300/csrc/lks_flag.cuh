@@ -90,6 +90,26 @@ template <>
 struct SumOf<double> {
   using type = Dd;
 };
+// A running sum of FP32 values as a double-float pair, or of doubles.
+__device__ __forceinline__ void run_add(Df& s, float b) {
+  const float t = s.hi + b, bb = t - s.hi;
+  s.lo += (s.hi - (t - bb)) + (b - bb);
+  s.hi = t;
+}
+__device__ __forceinline__ void run_add(Dd& s, double b) { s.v += b; }
+// Two sums at once (FP32 in packed instructions).
+__device__ __forceinline__ void run_add2(Df& s, Df& t, float b, float c) {
+  const float2 h = make_float2(s.hi, t.hi), x = make_float2(b, c), one = make_float2(-1.0f, -1.0f);
+  const float2 sum = __fadd2_rn(h, x), bb = __ffma2_rn(one, h, sum);
+  const float2 e = __fadd2_rn(__ffma2_rn(one, __ffma2_rn(one, bb, sum), h), __ffma2_rn(one, bb, x));
+  const float2 lo = __fadd2_rn(make_float2(s.lo, t.lo), e);
+  s = Df{sum.x, lo.x};
+  t = Df{sum.y, lo.y};
+}
+__device__ __forceinline__ void run_add2(Dd& s, Dd& t, double b, double c) {
+  s.v += b;
+  t.v += c;
+}
 template <int STRIDE, typename V>
 __device__ __forceinline__ void warp_total(V& v) {
 #pragma unroll

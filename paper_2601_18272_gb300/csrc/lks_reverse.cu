@@ -283,9 +283,9 @@ __global__ void __launch_bounds__(kRevThreads) k_rev_const(Geo g, const Ctrl* ct
   int lo[3];
   box_origin<D>(g, it[(long long)(t - 1) * (K + 1)], lo[0], lo[1], lo[2]);
   const T* P0 = slabs + (long long)i * slab + (long long)K * RP::per_itr * BC;
-  T v[NC];
+  typename SumOf<T>::type v[NC];
 #pragma unroll
-  for (int q = 0; q < NC; ++q) v[q] = T(0);
+  for (int q = 0; q < NC; ++q) v[q].zero();
   for (long long bl = blockIdx.x * (long long)kRevThreads + threadIdx.x; bl < BC;
        bl += (long long)gridDim.x * kRevThreads) {
     long long n;
@@ -296,13 +296,16 @@ __global__ void __launch_bounds__(kRevThreads) k_rev_const(Geo g, const Ctrl* ct
 #pragma unroll
     for (int a = 0; a < D; ++a) {
       lam[a] = Lcur[(a + 1) * N + n];
-      v[D + 1 + a] += lam[a] * bphi;
+      run_add(v[D + 1 + a], lam[a] * bphi);
     }
 #pragma unroll
-    for (int e = 0; e <= D; ++e)
+    for (int e = 0; e <= D; ++e) {
+      T s = T(0);
 #pragma unroll
-      for (int a = 0; a < D; ++a) v[e] += lam[a] * P[(RP::Q + e * D + a) * BC];
-    v[2 * D + 1] += lam[c] * P[RP::bP * BC] - lam[b] * P[(RP::bP + 1) * BC];
+      for (int a = 0; a < D; ++a) s += lam[a] * P[(RP::Q + e * D + a) * BC];
+      run_add(v[e], s);
+    }
+    run_add(v[2 * D + 1], lam[c] * P[RP::bP * BC] - lam[b] * P[(RP::bP + 1) * BC]);
   }
   row_sums<NC>(v, reinterpret_cast<T*>(rev_smem), cpart + blockIdx.x * NC);
 }
@@ -529,9 +532,6 @@ unsigned rev_ctas(const Geo& g) {
   return (unsigned)(n < kRevMaxCtas ? n : kRevMaxCtas);
 }
 
-template <typename T, int D>
-size_t rev_row_bytes(int nv) { return (size_t)nv * RowBuf<1>::pitch * sizeof(T); }
-
 template <typename T, int D, int AX>
 void coef_ax(const Geo& g, const RevBuffers& R, Ctrl* ctrl, const Dof* it, const T* kref, const Moments* mom,
              const T* boxstore, int nbox, int nsteps, int di, cudaStream_t st) {
@@ -541,7 +541,7 @@ void coef_ax(const Geo& g, const RevBuffers& R, Ctrl* ctrl, const Dof* it, const
     nc = (unsigned)coef_axis3d_ctas(g, sizeof(T) == 8);
     launch_coef_axis3d<T>(g, R, ctrl, it, kref, boxstore, nbox, nsteps, di, st);
   } else {
-    launch(k_rev_coef<T, D, AX>, dim3(nc, g.K, nsteps), kRevThreads, rev_row_bytes<T, D>(RevSums<D>::N), st, g,
+    launch(k_rev_coef<T, D, AX>, dim3(nc, g.K, nsteps), kRevThreads, row_bytes<T>(RevSums<D>::N), st, g,
            (const Ctrl*)ctrl, it, kref, boxstore, nbox, (T*)R.slabs, R.slab, (PT*)R.mpart, di);
   }
   launch(k_rev_mat<T, D, AX>, dim3(g.K, nsteps), kRevThreads, 0, st, g, (const Ctrl*)ctrl, it, mom, (const PT*)R.mpart,
@@ -552,7 +552,7 @@ void step_ax(const Geo& g, const RevBuffers& R, Ctrl* ctrl, const Dof* it, T* Lb
              cudaStream_t st) {
   using PT = typename Partial<T>::type;
   const unsigned nc = rev_ctas(g);
-  launch(k_rev_const<T, D, AX>, nc, kRevThreads, rev_row_bytes<T, D>(rev_nconst<D>()), st, g, (const Ctrl*)ctrl, it,
+  launch(k_rev_const<T, D, AX>, nc, kRevThreads, row_bytes<T>(rev_nconst<D>()), st, g, (const Ctrl*)ctrl, it,
          (const T*)R.slabs, R.slab, (const T*)Lb, lstride, (PT*)R.cpart, di, i);
   launch(k_rev_apply<T, D, AX>, nc + 1, kRevThreads, (size_t)g.K * (sizeof(RevMat) + 4 * (sizeof(double) + sizeof(T))), st, g, ctrl, it,
          (T*)R.slabs, R.slab, Lb, lstride, (const PT*)R.cpart, (int)nc, (const RevMat*)R.mats, (T*)R.lamh, di, i);

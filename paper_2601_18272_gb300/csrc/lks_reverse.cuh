@@ -4,7 +4,7 @@
 
 #include <climits>
 
-#include "lks_body_common.cuh"
+#include "lks_flag.cuh"
 
 namespace lks {
 
@@ -87,6 +87,69 @@ __device__ __forceinline__ void row_sums(const double (&v)[NV], double* buf, dou
     if (row < NV && seg == 0) out[row] = s;
   }
 }
+// Sum of each of N (a power of two) values over the warp's lanes by halving (each level exchanges half of the
+// values); lane l ends with that of value l mod N.
+template <int N>
+__device__ __forceinline__ float halve_sums(float (&x)[N], int lane) {
+#pragma unroll
+  for (int h = N / 2; h > 0; h >>= 1)
+#pragma unroll
+    for (int i = 0; i < h; ++i) {
+      const float send = (lane & h) ? x[i] : x[h + i], keep = (lane & h) ? x[h + i] : x[i];
+      x[i] = keep + __shfl_xor_sync(0xffffffffu, send, h);
+    }
+#pragma unroll
+  for (int off = N; off < 32; off <<= 1) x[0] += __shfl_xor_sync(0xffffffffu, x[0], off);
+  return x[0];
+}
+// The same for threads that have summed several cells, as pairs: the high parts through the rows, the low ones
+// by shuffles within each warp, whose sums the row's eight threads add. (Rows for both, twice the buffer, gave
+// the kernels another split of L1 and shared memory, and with it no place beside the other branch's CTAs:
+// gradients 2 % (128x64x64) to 6 % (157x67x70 duct) longer.)
+__host__ __device__ constexpr int pow2_from(int n) { return n <= 8 ? 8 : (n <= 16 ? 16 : 32); }
+template <int NV>
+__device__ __forceinline__ void row_sums(const Df (&v)[NV], float* buf, float2* out) {
+  constexpr int pitch = RowBuf<NV>::pitch, N = pow2_from(NV);
+  static_assert(NV * 8 <= kRevThreads && kRevThreads == 256, "eight threads per value, one per warp");
+  const int tid = threadIdx.x, lane = tid & 31, row = tid >> 3, seg = tid & 7;
+  float* low = buf + NV * pitch;  // [warp][N]
+  __syncthreads();
+  float x[N];
+#pragma unroll
+  for (int i = 0; i < N; ++i) x[i] = i < NV ? v[i < NV ? i : 0].lo : 0.0f;
+#pragma unroll
+  for (int i = 0; i < NV; ++i) buf[i * pitch + tid] = v[i].hi;
+  const float l = halve_sums<N>(x, lane);
+  if (lane < N) low[(tid >> 5) * N + lane] = l;
+  __syncthreads();
+  if ((tid & ~31) < NV * 8) {  // whole warps (shuffles below)
+    float hi = 0.0f, lo = 0.0f;
+    if (row < NV) {
+      const float* p = buf + row * pitch + seg;
+#pragma unroll 8
+      for (int j = 0; j < kRevThreads / 8; ++j) {
+        const float b = p[8 * j], s = hi + b, bb = s - hi;
+        lo += (hi - (s - bb)) + (b - bb);
+        hi = s;
+      }
+      lo += low[seg * N + row];
+    }
+#pragma unroll
+    for (int off = 4; off > 0; off >>= 1)
+      df_add(hi, lo, __shfl_down_sync(0xffffffffu, hi, off, 8), __shfl_down_sync(0xffffffffu, lo, off, 8));
+    if (row < NV && seg == 0) out[row] = make_float2(hi, lo);
+  }
+}
+template <int NV>
+__device__ __forceinline__ void row_sums(const Dd (&v)[NV], double* buf, double* out) {
+  double x[NV];
+#pragma unroll
+  for (int i = 0; i < NV; ++i) x[i] = v[i].v;
+  row_sums<NV>(x, buf, out);
+}
+// Shared memory of row_sums for nv values (of pairs, too).
+template <typename T>
+size_t row_bytes(int nv) { return ((size_t)nv * RowBuf<1>::pitch + (sizeof(T) == 4 ? 8 * pow2_from(nv) : 0)) * sizeof(T); }
 // Row `row` of partials [n][nv] summed by 8 threads in a fixed order (result in seg 0's thread).
 __device__ __forceinline__ double part_sum(const float2* p, int n, int nv, int row, int seg) {
   float hi = 0.0f, lo = 0.0f;
