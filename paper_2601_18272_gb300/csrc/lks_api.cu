@@ -589,7 +589,7 @@ void enqueue_rev_steps(lks_handle* h, Launcher& L, const Slots<T>& S, int nsteps
   const Geo& g = h->g;
   const int per = h->rev.steps, nc = (nsteps + per - 1) / per;
   auto steps_of = [&](int c) { return std::min(per, nsteps - c * per); };
-  const bool fork = L.capturing && nc > 1;
+  const bool fork = L.capturing && nc > 1 && h->rev.other > 0;
   Launcher side = L;
   side.kernels = 0;
   if (fork) side.st = h->cap2;
@@ -887,8 +887,8 @@ int give_back_optional(lks_handle* h, bool* gave) {
 }
 
 // Chooses the form of the exact reverse: the linear maps for bodies about one axis in the automatic
-// coupling mode, when the workspace limit and the device have room for their buffers; else the
-// per-iteration or persistent kernels.
+// coupling mode, when they stay within kRevMaxBytes and the workspace limit and the device have room for
+// their buffers; else the per-iteration or persistent kernels.
 int choose_reverse(lks_handle* h, cudaStream_t st) {
   h->rev_on = false;
   if (h->coop_mode != 2 || !reverse_affine_fits(h->g)) return LKS_OK;
@@ -896,6 +896,7 @@ int choose_reverse(lks_handle* h, cudaStream_t st) {
                   : h->P.ckpt_policy == LKS_CKPT_UNIFORM ? std::min(h->P.ckpt_every, h->P.n_steps) : h->chunk;
   RevBuffers R;
   const size_t need = reverse_layout(h->g, h->prec == LKS_FP64, seg, &R);
+  if (need > kRevMaxBytes) return LKS_OK;
   if (need > h->rev_bytes) {  // the first call, or a larger body box since (its graphs are gone)
     cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
     CK(cudaStreamIsCapturing(st, &cs));

@@ -190,7 +190,7 @@ struct RevBuffers {
   int splits = 0;      // partial dJ/dkappa^ref of the design kernel
   // a second set of the chunk's buffers (slabs, mpart, mats, lamh): the next chunk's planes are made and
   // the last one's dJ/dkappa^ref is summed beside the chain of this one
-  size_t other = 0;    // bytes from a buffer of the first set to its twin
+  size_t other = 0;    // bytes from a buffer of the first set to its twin (0: one set, chunk after chunk)
   RevBuffers set(int i) const {
     RevBuffers r = *this;
     if (i & 1)
@@ -198,6 +198,12 @@ struct RevBuffers {
     return r;
   }
 };
+// Limit of a handle's maps. A step's planes take 69 values per box cell in 3D and 52 in 2D at five iterations, which
+// grows with the body and not with the march: 2.5 GB a set at a 160^3 design, 10 at 256^3 (FP32). They pay
+// at every size measured (us per step of the gradient, per-iteration kernels -> one set -> two: 64^3 1644 -> 715 ->
+// 692, 128^3 10013 -> 3732 -> 3635, 192^3 33461 -> 11584 -> 11367; 1600^2 6415 -> 3380 -> 3048), so the limit
+// is there to leave the device to its other users: 16 GiB, a seventeenth of it.
+constexpr size_t kRevMaxBytes = (size_t)16 << 30;
 bool reverse_affine_fits(const Geo& g);
 size_t reverse_layout(const Geo& g, bool fp64, int max_steps, RevBuffers* R);
 void launch_rev_init(const Geo& g, const RevBuffers& R, Ctrl* ctrl, int nt, cudaStream_t st);

@@ -625,8 +625,10 @@ size_t reverse_layout(const Geo& g, bool fp64, int max_steps, RevBuffers* R) {
   const size_t mpart = take(R->steps * K * nc * nm * 8);
   const size_t mats = take(R->steps * K * (long long)sizeof(RevMat));
   const size_t lamh = take(R->steps * K * 4 * esz);
-  R->other = off;
-  off *= 2;
+  // a second set only where a chunk follows another in a segment, and while the two stay within the limit
+  const bool two = max_steps > R->steps && 2 * off <= kRevMaxBytes;
+  R->other = two ? off : 0;
+  if (two) off *= 2;
   const size_t cpart = take((long long)kRevMaxCtas * 8 * 8);
   const size_t dkp = take((long long)R->splits * g.ND * 8);
   if (R->block) {
