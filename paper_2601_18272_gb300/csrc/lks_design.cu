@@ -104,10 +104,11 @@ FilterTab make_table(const Geo& g) {
   return t;
 }
 
-// Sum of w_ij src_j over the filter disc of i (points of the design domain).
+// Sum of w_ij src_j over the filter disc of i (points of the design domain). All lanes of the warp call it, for
+// its vote; those without a point of their own (in false) get 0.
 template <bool NEED_W>
 __device__ __forceinline__ double filter_sum(const Geo& g, const FilterTab& tab, const double* __restrict__ src,
-                                             const int* i, double* W) {
+                                             const int* i, bool in, double* W) {
   const double R = g.frad;
   const int rr = (int)floor(R);
   const int ez = (g.dim == 3) ? rr : 0;
@@ -117,7 +118,8 @@ __device__ __forceinline__ double filter_sum(const Geo& g, const FilterTab& tab,
   const int y0 = max(-rr, -i[1]), y1 = min(rr, g.nd[1] - 1 - i[1]);
   const int z0 = max(-ez, -i[2]), z1 = min(ez, g.nd[2] - 1 - i[2]);
   const bool whole = !ball && table && x0 == -rr && x1 == rr && y0 == -rr && y1 == rr && z0 == -ez && z1 == ez;
-  const bool even = __all_sync(__activemask(), whole);
+  const bool even = __all_sync(0xffffffffu, whole || !in);
+  if (!in) return 0.0;
   for (int dz = even ? -ez : z0; dz <= (even ? ez : z1); ++dz)
     for (int dy = even ? -rr : y0; dy <= (even ? rr : y1); ++dy) {
       const int r2 = dy * dy + dz * dz;
@@ -162,16 +164,18 @@ __global__ void __launch_bounds__(kDB) k_filter_project(Geo g, const __grid_cons
   make_projection(g, pr);
   __syncthreads();
   const int m = blockIdx.x * kDB + threadIdx.x;
-  if (m >= g.ND) return;
   int i[3];
-  design_ijk(g, m, i);
-  if (!in_domain(g, i)) {
+  design_ijk(g, min(m, g.ND - 1), i);
+  const bool in = m < g.ND && in_domain(g, i);
+  double gt = 0.0, w = 1.0;
+  if (g.frad > 0.0) gt = filter_sum<true>(g, tab, g1, i, in, &w) / w;
+  if (m >= g.ND) return;
+  if (!in) {
     gtil[m] = gbar[m] = 0.0;
     W[m] = 1.0;
     return;
   }
-  double gt = g1[m], w = 1.0;
-  if (g.frad > 0.0) gt = filter_sum<true>(g, tab, g1, i, &w) / w;
+  if (!(g.frad > 0.0)) gt = g1[m];
   gtil[m] = gt;
   W[m] = w;
   if (g.pbeta > 0.0)
@@ -220,10 +224,10 @@ __global__ void __launch_bounds__(kDB) k_project_T(Geo g, GradIn in, const doubl
 __global__ void __launch_bounds__(kDB) k_filter_T(Geo g, const __grid_constant__ FilterTab tab,
                                                   const double* __restrict__ v, double* __restrict__ out) {
   const int m = blockIdx.x * kDB + threadIdx.x;
-  if (m >= g.ND) return;
   int i[3];
-  design_ijk(g, m, i);
-  out[m] = in_domain(g, i) ? filter_sum<false>(g, tab, v, i, nullptr) : 0.0;
+  design_ijk(g, min(m, g.ND - 1), i);
+  const double s = filter_sum<false>(g, tab, v, i, m < g.ND && in_domain(g, i), nullptr);
+  if (m < g.ND) out[m] = s;
 }
 
 __global__ void __launch_bounds__(kDB) k_orbit_sum(Geo g, const double* __restrict__ v, double* __restrict__ out) {
