@@ -258,13 +258,16 @@ void adj_shape(const Geo& g, const Slots<T>& S, T* Lb, long long lstride, const 
 }  // namespace
 
 // Tiles pay while the strips of the other form are short: a strip of L rows works on L + 4. FP64
-// (instruction count decides): below 12 rows; 600x100 predictor / transpose 24 / 41 -> 17 / 18 us,
-// 80x40 25 / 42 -> 7 / 7. FP32 (the tile's loads cost more): only where strips have two or three rows,
+// (instruction count decides): the predictor below 4 rows, the transpose, whose strips do more per row, below
+// 12. Strips -> tiles, predictor / transpose in us: 80x40 25 / 42 -> 7 / 7; 600x100 24 / 42 -> 17 / 19; 1024x512
+// 149 / 258 -> 102 / 101; 2600x1300 712 / 1168 -> 623 / 603; 3000x1500 (3 rows) 840 / 1315 -> 827 / 795; 3300x1700
+// (4) 969 / 1497 -> 1030 / 994; 4096x2048 (7) 1305 / 1915 -> 1524 / 1468; 5000x2500 (10) 1799 / 2547 -> 2281 / 2193.
+// FP32 (the tile's loads cost more): only where strips have two or three rows,
 // and the predictor, whose chain is shorter, only on the smallest grids: 512x256 7 / 11 -> 6 / 7,
 // 1024x512 12.4 / 18 -> 13 / 13.5, 2048x1024 21 / 32 -> 40 / 44 us. (Events around each launch, less
 // their 3.5 us.)
 bool stencil_tile_pays(const Geo& g, int rows, bool fp64, bool transpose) {
-  if (fp64) return rows < 12;
+  if (fp64) return rows < (transpose ? 12 : 4);
   return rows < 4 && g.N <= (transpose ? 1LL << 20 : 1LL << 18);
 }
 
