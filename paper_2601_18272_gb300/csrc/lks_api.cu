@@ -916,6 +916,7 @@ int choose_reverse(lks_handle* h, cudaStream_t st) {
     }
     h->rev_bytes = need;
     h->bytes += need;
+    if (h->prec == LKS_FP32 && coef_axis3d_fits(h->g)) prepare_coef_axis3d(h->g);
   }
   reverse_layout(h->g, h->prec == LKS_FP64, seg, &h->rev);
   h->rev_on = true;

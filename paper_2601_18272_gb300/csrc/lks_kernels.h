@@ -224,6 +224,7 @@ void launch_rev_design(const Geo& g, const RevBuffers& R, Ctrl* ctrl, const Dof*
 // Their 3D forms; coef_axis3d_fits: the whole design grid is the design domain.
 bool coef_axis3d_fits(const Geo& g);
 int coef_axis3d_ctas(const Geo& g, bool fp64);
+void prepare_coef_axis3d(const Geo& g);  // once per handle, FP32
 template <typename T>
 void launch_coef_axis3d(const Geo& g, const RevBuffers& R, const Ctrl* ctrl, const Dof* it, const T* kref, const T* boxstore,
                         int nbox, int nsteps, int di, cudaStream_t st);

@@ -564,7 +564,7 @@ void coef_ax(const Geo& g, const RevBuffers& R, Ctrl* ctrl, const Dof* it, const
     nc = (unsigned)coef_axis3d_ctas(g, sizeof(T) == 8);
     launch_coef_axis3d<T>(g, R, ctrl, it, kref, boxstore, nbox, nsteps, di, st);
   } else {
-    launch(k_rev_coef<T, D, AX>, dim3(nc, g.K, nsteps), kRevThreads, row_bytes<T>(RevSums<D>::N), st, g,
+    launch(k_rev_coef<T, D, AX>, dim3(nc, g.K, nsteps), kRevThreads, row_bytes<T>(RevSums<D>::N, false), st, g,
            (const Ctrl*)ctrl, it, kref, boxstore, nbox, (T*)R.slabs, R.slab, (PT*)R.mpart, di);
   }
   launch(k_rev_mat<T, D, AX>, dim3(g.K, nsteps), kRevThreads, 0, st, g, (const Ctrl*)ctrl, it, mom, (const PT*)R.mpart,
@@ -577,7 +577,7 @@ void step_ax(const Geo& g, const RevBuffers& R, Ctrl* ctrl, const Dof* it, T* Lb
   const unsigned nc = rev_ctas(g);
   const bool many = g.box_cells > (long long)nc * kRevThreads;
   launch(many ? k_rev_const<T, D, AX, true> : k_rev_const<T, D, AX, false>, nc, kRevThreads,
-         row_bytes<T>(rev_nconst<D>()), st, g, (const Ctrl*)ctrl, it, (const T*)R.slabs, R.slab, (const T*)Lb, lstride,
+         row_bytes<T>(rev_nconst<D>(), many), st, g, (const Ctrl*)ctrl, it, (const T*)R.slabs, R.slab, (const T*)Lb, lstride,
          (PT*)R.cpart, di, i);
   launch(k_rev_apply<T, D, AX>, nc + 1, kRevThreads, (size_t)g.K * (sizeof(RevMat) + 4 * (sizeof(double) + sizeof(T))), st, g, ctrl, it,
          (T*)R.slabs, R.slab, Lb, lstride, (const PT*)R.cpart, (int)nc, (const RevMat*)R.mats, (T*)R.lamh, di, i);

@@ -147,9 +147,11 @@ __device__ __forceinline__ void row_sums(const Dd (&v)[NV], double* buf, double*
   for (int i = 0; i < NV; ++i) x[i] = v[i].v;
   row_sums<NV>(x, buf, out);
 }
-// Shared memory of row_sums for nv values (of pairs, too).
+// Shared memory of row_sums for nv values or pairs.
 template <typename T>
-size_t row_bytes(int nv) { return ((size_t)nv * RowBuf<1>::pitch + (sizeof(T) == 4 ? 8 * pow2_from(nv) : 0)) * sizeof(T); }
+size_t row_bytes(int nv, bool pairs) {
+  return ((size_t)nv * RowBuf<1>::pitch + (sizeof(T) == 4 && pairs ? 8 * pow2_from(nv) : 0)) * sizeof(T);
+}
 // Row `row` of partials [n][nv] summed by 8 threads in a fixed order (result in seg 0's thread).
 __device__ __forceinline__ double part_sum(const float2* p, int n, int nv, int row, int seg) {
   float hi = 0.0f, lo = 0.0f;
