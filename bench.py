@@ -119,18 +119,30 @@ def _peaks():
 # Algorithmic bytes per launch of each kernel family. N = analysis cells, box_cells = body-box
 # cells, ND = design points, esz = bytes per field value, K = N_itr. A body family's launches per step
 # depend on the chosen form (all K iterations in one launch, one launch per iteration, several steps
-# in one launch), so its bytes are those of a step, divided by its launches per step.
-def _alg_bytes(family: str, P, box_cells: int, esz: int, launches_per_step: float = 1.0) -> float:
+# in one launch), so its bytes are those of a step, divided by its launches per step. maps: the reverse
+# ran by linear maps, whose planes per box cell (4 + 2d an iteration, and the last one's) are written by
+# adj_cell and read by adj_body and adj_design.
+def _alg_bytes(family: str, P, box_cells: int, esz: int, launches_per_step: float = 1.0, maps: bool = False) -> float:
     N, ND = P.n_cells, P.n_design
     d, K = P.dim, P.n_itr
     if family == "stencil_fwd":
         return 2 * (d + 1) * esz * N  # read p, u; write p*, u*
     if family == "stencil_adj":
         return (3 * d + 2) * esz * N  # read the adjoint (d+1 planes) and u(t-1) (d planes); write d+1 planes
-    if family == "couple":  # each iteration reads u* in the box (+ kappa^ref), the last writes u(t), stored u*
-        return (K * (d * esz * box_cells + 4 * ND) + 2 * d * esz * box_cells) / launches_per_step
+    if family == "couple":  # a launch reads u* in the box and kappa^ref, the last one writes u(t), stored u*
+        launches = min(K, round(launches_per_step))
+        return (launches * (d * esz * box_cells + 4 * ND) + 2 * d * esz * box_cells) / launches_per_step
     if family == "recompute":
         return 3 * d * esz * box_cells + 4 * ND  # read u*, write u and the stored u*
+    if maps and family in ("adj_cell", "adj_design", "adj_body"):
+        last = d + 1 + (d + 1) * d + 3  # 1/(1+kappa), du/dkappa; du/d(x^G, theta), u^G and omega parts
+        if family == "adj_cell":  # read the stored u* and kappa^ref, write the planes
+            b = esz * box_cells * (d + K * (4 + 2 * d) + last) + 4 * ND
+        elif family == "adj_body":  # constant part: its planes and the adjoint; apply: the rest, adjoint r/w
+            b = esz * box_cells * ((last - d - 1) + d + (d + 1) + 2 * d + K * (5 + d))
+        else:  # u and dJ/dkappa of every iteration, dJ/dkappa^ref r/w
+            b = esz * box_cells * K * (d + 1) + 16 * ND
+        return b / launches_per_step
     cell = (5 * d + 1) * esz * box_cells      # read stored u*, acc r/w, scratch write (2d+1 planes)
     design = (2 * d + 1) * esz * box_cells + 20 * ND  # read scratch once, dJ/dkappa^ref r/w + kappa^ref
     if family == "adj_cell":
@@ -647,7 +659,8 @@ def main():
         peak, peak_kind = _peaks()
         per_launch_s = dom_ms / 1000.0 / dom_n
         persistent = lks.lks_persistent_coupling(solver.handle, -1)
-        alg = _alg_bytes(dom, P, _box_cells(P), 4, dom_n / P.n_steps)
+        maps = "adj_body" in fams and "adj_cell" in fams  # (the persistent reverse is one family)
+        alg = _alg_bytes(dom, P, _box_cells(P), 4, dom_n / P.n_steps, maps)
         achieved = alg / per_launch_s / 1e9
         line["roofline"] = {"bound": "hbm", "kernel": dom, "achieved": achieved, "peak": peak, "unit": "GB/s",
                             "frac": achieved / peak, "traffic": _traffic(P.name, dom), "peak_source": peak_kind,
