@@ -261,8 +261,9 @@ LKS_API int lks_support_sets(lks_handle* h, const double* s_host, int* box_host,
                              size_t capacity);
 
 /* Test hook of the bounded waits of the coupling kernels: skip != 0 makes the first CTA of every
- * persistent coupling kernel skip its barrier arrivals (its published words in 2D's default form), so the other CTAs' waits run out (after one second) and the
- * forward or adjoint returns LKS_ERR_TIMEOUT; skip = 0 restores normal operation. Synchronises the
+ * persistent coupling kernel skip its barrier arrivals, and that of the default form about one axis
+ * withhold its iterates, so the other CTAs' waits run out (after one second) and the forward (or the
+ * adjoint of mode 1) returns LKS_ERR_TIMEOUT; skip = 0 restores normal operation. Synchronises the
  * device. Errors: LKS_ERR_ARG, LKS_ERR_CUDA. */
 LKS_API int lks_debug_sync_skip(lks_handle* h, int skip);
 
@@ -279,11 +280,12 @@ LKS_API int lks_debug_copy_skip(lks_handle* h, int skip);
  * holds its grid, mode 0 as one launch per iteration (with the finish kernels), mode 2 (the default)
  * by the problem: about one rotation axis the forward runs as one cooperative launch per step whose
  * CTAs exchange their sums through flagged words (bounded waits of one second, LKS_ERR_TIMEOUT) and
- * the reverse by linear maps of the iterations (no waits); with free rotation both run as one launch
- * per iteration. The words and the maps' buffers are allocated by the
- * first lks_forward and lks_adjoint if hbm_budget_bytes and the device have room; without it 2D bodies
- * whose box has more tiles than the persistent grid has CTAs take the persistent launch and the others
- * one launch per iteration. Mode -1 only asks. Returns 1 if the grid-barrier kernels are chosen (in
+ * the reverse by linear maps of the iterations (no waits); with free rotation, and in the forward of
+ * 3D bodies with small boxes, each iteration is one launch. The words and the maps' buffers (at most
+ * 16 GiB a handle, beyond which the reverse runs per iteration) are allocated by the first lks_forward
+ * and lks_adjoint if hbm_budget_bytes and the device have room; without it 2D bodies whose box has
+ * more tiles than the persistent grid has CTAs take the persistent launch and the others one launch
+ * per iteration. Mode -1 only asks. Returns 1 if the grid-barrier kernels are chosen (in
  * mode 2: the body is 2D and its box has more tiles than their grid has CTAs, so that a CTA of the
  * persistent launch works on several tiles), 0 if not, or -status on error (LKS_ERR_ARG,
  * LKS_ERR_CUDA). Changing the mode synchronises the device; results agree to rounding (the per-CTA

@@ -293,7 +293,7 @@ struct lks_handle {
   Dof* it = nullptr;
   Ctrl* ctrl = nullptr;
   Moments* mom = nullptr;
-  void* words = nullptr;  // 2D: the coupling sums' flagged words (allocated by the first lks_forward)
+  void* words = nullptr;  // the coupling sums' flagged words, one rotation axis (allocated by the first lks_forward)
   bool no_words = false;  // the budget or the device had no room for them: the other forms run
   double* partials = nullptr;
   long long pstride = 0;  // elements per half of the double-buffered coupling partials
@@ -545,7 +545,7 @@ void enqueue_fwd_steps(lks_handle* h, Launcher& L, const Slots<T>& S, int nsteps
   T* bs = store_box ? (T*)h->boxstore : nullptr;
   for (int i = 0; i < nsteps; ++i) {
     L("stencil_fwd", [&](cudaStream_t s) { launch_stencil_fwd<T>(g, S, h->ctrl, i, s); });
-    if (g.flag_ctas > 0) {  // 2D: all N_itr iterations and the last EOM, sums exchanged through flagged words
+    if (g.flag_ctas > 0) {  // all N_itr iterations and the last EOM, sums exchanged through flagged words
       L("couple", [&](cudaStream_t s) {
         launch_couple_flag<T>(g, S, h->ctrl, h->it, (const T*)h->kref, h->mom, h->words, bs, h->nbox, i, s);
       });
@@ -847,7 +847,7 @@ int adjoint_impl(lks_handle* h, double seed, cudaStream_t st) {
   return LKS_OK;
 }
 
-// Room for the flagged words of the 2D coupling; without it the handle keeps to the other forms.
+// Room for the flagged words of the coupling; without it the handle keeps to the other forms.
 void choose_coupling(lks_handle* h) {
   if (h->g.flag_ctas == 0 || h->words) return;
   const size_t need = (couple_flag_bytes(kFlagMaxCtas) + 255) & ~(size_t)255;

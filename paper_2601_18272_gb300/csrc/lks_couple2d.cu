@@ -158,7 +158,7 @@ __device__ __forceinline__ void gather2d(const Geo& g, const double* __restrict_
       if (fabsf(csf * ebf - snf * ecf) >= Sp || fabsf(snf * ebf + csf * ecf) >= Sp) continue;
       if (dsq(ib, g.nd[0]) + dsq(ic, g.nd[1]) > g.rad4) continue;
       const double eb = (double)ib - xib, ec = (double)ic - xic;
-      const double ob = dot2(cs, eb, -sn, ec), oc = dot2(sn, eb, cs, ec);
+      const double ob = dot2(-sn, ec, cs, eb), oc = dot2(cs, ec, sn, eb);  // (the products of eb leave the loop)
       if (fabs(ob) >= S || fabs(oc) >= S) continue;
       visit(ib + ic * g.nd[0]);
       const double w = mul_(wfun(g.wk, ob), wfun(g.wk, oc)), wk = mul_(w, kref[ib + ic * g.nd[0]]);

@@ -6,7 +6,7 @@
 // beside 32 bits of payload, so the arrival of the data is the synchronisation: one trip through L2
 // each way, and every waiting CTA polls one or two lines. (A form in which every CTA polled the words
 // of all others and ran the EOM itself needed one trip only, but took 4.3 us an iteration without
-// gather and EOM on 148 SMs: 57 lines polled by all of them.) A word's number tells it from the one
+// gather and EOM with 152 CTAs: 57 lines polled by all of them.) A word's number tells it from the one
 // two iterations earlier in the same place (two places by the iteration's parity): sums of iteration
 // e + 2 are published after the iterate of e + 1 was read, which CTA 0 publishes after it has read
 // the sums of e; and likewise the other way. All sums are taken in a fixed order (warps, CTA, then 32

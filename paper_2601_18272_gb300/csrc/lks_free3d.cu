@@ -16,8 +16,7 @@
 //
 // The forward keeps the per-cell gather (k_couple): the tiled one took 135 us against 257, but its other
 // rounding moves values of reduced-precision snapshots across a rounding step of 1/512, and with that
-// single gradient entries by up to 8e-4 of their rms (BF16, 12 steps), where no more than that is wanted;
-// the forward must not depend on the snapshots' format either.
+// single gradient entries by up to 8e-4 of their rms (BF16, 12 steps), where no more than that is wanted.
 #include <algorithm>
 #include <climits>
 
