@@ -268,9 +268,10 @@ __device__ __forceinline__ bool box_cell(const Geo& g, const int (&lo)[3], long 
   return cell_index<D>(g, lo[0] + j0, lo[1] + j1, lo[2] + j2, n);
 }
 
-// MANY: boxes of more cells than the launch has threads. A thread's cells are then summed as pairs, and their
+// MANY: boxes of more cells than the launch has threads. A thread's cells are then summed as pairs in FP32, whose
 // loads go out several cells at a time (one after the other took 25 % longer for the step's two kernels on
-// 5 million cells).
+// 5 million cells); FP64 adds every term to the sums directly (forming a cell's terms first: 31 -> 38 us a
+// step for the two kernels on 93,000 cells).
 template <typename T, int D, int AX, bool MANY>
 __global__ void __launch_bounds__(kRevThreads) k_rev_const(Geo g, const Ctrl* ctrl, const Dof* it,
                                                            const T* __restrict__ slabs, long long slab, const T* Lb,
@@ -286,7 +287,7 @@ __global__ void __launch_bounds__(kRevThreads) k_rev_const(Geo g, const Ctrl* ct
   int lo[3];
   box_origin<D>(g, it[(long long)(t - 1) * (K + 1)], lo[0], lo[1], lo[2]);
   const T* P0 = slabs + (long long)i * slab + (long long)K * RP::per_itr * BC;
-  // the cell's terms (zero off the box and the grid)
+  // adds the cell's terms (zero off the box and the grid)
   auto cell = [&](long long bl, T (&v)[NC]) {
     long long n = 0;
     const bool in = bl < BC && box_cell<D>(g, lo, bl, n);
@@ -298,22 +299,27 @@ __global__ void __launch_bounds__(kRevThreads) k_rev_const(Geo g, const Ctrl* ct
     for (int a = 0; a < D; ++a) {
       const T l = Lcur[(a + 1) * N + n];
       lam[a] = in ? l : T(0);
-      v[D + 1 + a] = lam[a] * bphi;
+      v[D + 1 + a] += lam[a] * bphi;
     }
 #pragma unroll
-    for (int e = 0; e <= D; ++e) {
-      v[e] = T(0);
+    for (int e = 0; e <= D; ++e)
 #pragma unroll
       for (int a = 0; a < D; ++a) v[e] += lam[a] * P[(RP::Q + e * D + a) * BC];
-    }
-    v[2 * D + 1] = lam[c] * P[RP::bP * BC] - lam[b] * P[(RP::bP + 1) * BC];
+    v[2 * D + 1] += lam[c] * P[RP::bP * BC] - lam[b] * P[(RP::bP + 1) * BC];
   };
   const long long stride = (long long)gridDim.x * kRevThreads;
   long long bl = blockIdx.x * (long long)kRevThreads + threadIdx.x;
   auto* out = cpart + blockIdx.x * NC;
-  if constexpr (!MANY) {
+  if constexpr (!MANY || sizeof(T) == 8) {
     T v[NC];
-    cell(bl, v);
+#pragma unroll
+    for (int q = 0; q < NC; ++q) v[q] = T(0);
+    if constexpr (!MANY) {
+      cell(bl, v);
+    } else {
+#pragma unroll 4
+      for (; bl < BC; bl += stride) cell(bl, v);
+    }
     row_sums<NC>(v, reinterpret_cast<T*>(rev_smem), out);
   } else {
     constexpr int U = D == 2 ? 4 : 2;
@@ -323,7 +329,11 @@ __global__ void __launch_bounds__(kRevThreads) k_rev_const(Geo g, const Ctrl* ct
     for (; bl < BC; bl += U * stride) {
       T x[U][NC];
 #pragma unroll
-      for (int u = 0; u < U; ++u) cell(bl + u * stride, x[u]);
+      for (int u = 0; u < U; ++u) {
+#pragma unroll
+        for (int q = 0; q < NC; ++q) x[u][q] = T(0);
+        cell(bl + u * stride, x[u]);
+      }
 #pragma unroll
       for (int u = 0; u < U; ++u)
 #pragma unroll
